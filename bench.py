@@ -351,10 +351,10 @@ def run_ours(args, rank, world, local_rank, raw):
     sgs_bytes_per_step = cstats["cost_bytes_read"]
     sgs_launch_ms = sgs_ms / max(sgs_launches, 1)
     sgs_gbs = (sgs_bytes_per_step / launches_per_step) / (sgs_launch_ms / 1000.0) / 1e9
-    roofline_sgs = {"bound": "hbm", "kernel": "k_sgs_lazy_cl", "achieved": round(sgs_gbs, 1),
+    roofline_sgs = {"bound": "hbm", "kernel": "k_sgs_push", "achieved": round(sgs_gbs, 1),
                     "peak": hbm, "unit": "GB/s", "frac": round(sgs_gbs / hbm, 4),
                     "frac_of_nominal": round(sgs_gbs / HBM_NOMINAL_GBS, 4),
-                    "traffic": read_traffic("k_sgs_lazy", sgs_bytes_per_step // launches_per_step),
+                    "traffic": read_traffic("k_sgs_push", sgs_bytes_per_step // launches_per_step),
                     "peak_source": peak_kind,
                     "algorithmic_bytes_per_launch": sgs_bytes_per_step // launches_per_step,
                     "avg_launch_ms": round(sgs_launch_ms, 3),

@@ -104,11 +104,11 @@ typedef enum {
  *                                   which the kernel records CP_ETIMEOUT and
  *                                   returns (> 0; default 2000)
  *   sgs_mode                        how SGS finds each step's winner: 0 =
- *                                   lazy (a gain computed at an earlier step
- *                                   bounds the current one, so only
- *                                   candidates whose bound could still win
- *                                   are re-evaluated; default), 1 = every
- *                                   gain every step (the same picks); 2 =
+ *                                   every candidate's gain is kept up to
+ *                                   date, a pick taking off exactly the
+ *                                   terms it lowers (default); 1 = every
+ *                                   gain summed afresh every step (the same
+ *                                   picks); 2 =
  *                                   the rule as Sec. 3.5 prints it: at step
  *                                   l the entropic semi-relaxed OT of Eq.
  *                                   srpot_sinkhorn from the l selected
@@ -235,8 +235,9 @@ int coverprune_cost(const void* feats, int dtype, const float* pos, const int32_
  *   F(S) = sum_j v_j m_j.  Each of the K steps adds the unselected token t
  *   with the largest local decrease
  *       gain(t) = sum_{j in M_g(t)} v_j max(m_j - C(t, j), 0)
- *   (the lowest index among equal gains).  Gains are evaluated in float32
- *   with a fixed summation order, so repeated calls return identical results.
+ *   (the lowest index among equal gains).  A gain's terms are float32 and
+ *   add up in 64-bit fixed point, which has no order, and its leading 24 bits
+ *   decide; repeated calls return identical results.
  *
  *   kept       [B, K] int64, the selected indices in ascending order
  *   order      [B, K] int64 or NULL, the indices in selection order
@@ -373,17 +374,17 @@ int coverprune_profile_read(double* ms, int64_t* launches, int n);
 /*
  * Counters of the last coverprune_select that used workspace `ws`
  * (synchronises `stream` first):
- *   gain_evaluations  candidate gains computed, over all scenes and steps;
- *                     each reads one row of the cost (N floats) or of the
- *                     local slab (g floats)
- *   rounds            decision rounds over all scenes and steps (lazy mode:
- *                     a step needs one or more; full sweep: one per step)
+ *   gain_evaluations  sgs_mode 1: candidate gains computed, over all scenes
+ *                     and steps, each from one row of the cost (N floats) or
+ *                     of the local slab (g floats); sgs_mode 0: terms of
+ *                     gains updated after the first pick, one per live
+ *                     (candidate, target) pair of a lowered target
+ *   rounds            decision rounds over all scenes (one per step)
  *   cost_bytes_read   bytes of cost rows (or slab rows and their neighbour
- *                     indices) the selection reads: every gain evaluation,
- *                     and once per scene and step the winner's row for the
- *                     coverage update; the dense lazy kernel skips row
- *                     blocks whose terms are known to be zero, so this can
- *                     be well below gain_evaluations * 4N
+ *                     indices) and of live lists the steps read: sgs_mode 1
+ *                     a row per gain, and once per scene and step the
+ *                     winner's row for the coverage update; sgs_mode 0 the
+ *                     winners' rows and 8 bytes per updated term
  * Returns CP_OK, CP_EINVAL or CP_ECUDA.
  */
 typedef struct {

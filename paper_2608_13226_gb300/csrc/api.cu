@@ -200,10 +200,9 @@ static DevParams dev_params(const cp_params* p, int64_t N) {
 struct Plan {
   size_t hdr, counters, stats, norms, inv, tok, nbr, r, v;
   size_t grid_info, grid_start, grid_pts;         // neighbour grid (kk <= kKnnGridMax)
-  size_t cost, slab, partials, order32, g0;       // select
+  size_t cost, slab, partials, order32, g0, push;  // select
   size_t lit;                                     // literal SGS (sgs_mode 2) scratch
   size_t lfeats, ltok, lperm, lpos, lflags, lunits, lnunits;  // local Morton tiles
-  size_t rev_off, rev;                            // local SGS reverse neighbourhoods
   size_t perm, prefix, gs, proto, score;          // lite
   size_t total;
   int64_t ldc;
@@ -256,11 +255,8 @@ static void plan_ws(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtyp
   if (op == CP_OP_SELECT) {
     pl->cost = take(sizeof(float) * BN * (size_t)pl->ldc);
     if (d.sgs_mode == 2) pl->lit = take(sgs_literal_ws_bytes(B, N, K));
-    if (d.g < N && d.sgs_mode != 2) {
-      pl->slab = take(sizeof(float) * BN * (size_t)d.g);
-      pl->rev_off = take(sizeof(int32_t) * (BN + (size_t)B));
-      pl->rev = take(sizeof(int32_t) * BN * (size_t)d.g);
-    }
+    if (d.g < N && d.sgs_mode != 2) pl->slab = take(sizeof(float) * BN * (size_t)d.g);
+    if (d.sgs_mode == 0) pl->push = take(sgs_push_ws_bytes(B, N, d.g, pl->ldc));
     if (local_tiles_path(op, dtype, N, d)) {
       const size_t T = (size_t)local_tiles(N);
       pl->lfeats = take(2 * BN * (size_t)D);
@@ -548,7 +544,7 @@ int coverprune_select(const void* feats, int dtype, const float* pos, const int3
     CP_TRY(launch_capacity(feats, dtype, inv, pos, frame, nm, nbr, d, B, N, D, at<float>(ws, pl.r),
                            v, nullptr, s, dtype == CP_BF16 ? C : nullptr, pl.ldc, pos_of));
   }
-  // the dense lazy selection starts from bounds the cost pass sums
+  // the dense selection's first pick starts from bounds the cost pass sums
   float* g0 = (dtype == CP_BF16 && d.g >= N && d.sgs_mode == 0) ? at<float>(ws, pl.g0) : nullptr;
   // local SGS reads only the N x g slab: for bf16 it comes straight from
   // the stored cosines, and the dense cost is never formed (the literal rule
@@ -578,8 +574,7 @@ int coverprune_select(const void* feats, int dtype, const float* pos, const int3
     else
       CP_TRY(launch_sgs(C, pl.ldc, slab, nbr, v, d, B, N, K, order32, gains, objective,
                         at<uint64_t>(ws, pl.partials), at<uint32_t>(ws, pl.counters), status, s,
-                        g0, slab ? at<int32_t>(ws, pl.rev_off) : nullptr,
-                        slab ? at<int32_t>(ws, pl.rev) : nullptr));
+                        g0, at<void>(ws, pl.push)));
   }
   Stage st(CP_STAGE_OUTPUT, s);
   CP_TRY(launch_sort_kept(order32, B, K, kept, order, s));

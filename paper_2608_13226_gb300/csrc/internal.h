@@ -20,7 +20,7 @@ struct DevParams {
   int g;       // SGS neighbourhood incl. the token itself; == N means all
   int kk;      // neighbours stored per token = max(n_cap, g-1) (g < N) or n_cap
   int cap_mode;
-  int sgs_mode;  // 0 = lazy evaluation of gains, 1 = every gain every step, 2 = literal rule
+  int sgs_mode;  // 0 = gains kept up to date, 1 = every gain every step, 2 = literal rule
   int norm_mode;  // feature normaliser: 0 = min-max over all pairs, 1 = d_f / 2
   float sot_eps;  // literal rule: entropic weight of the semi-relaxed OT
   int sot_iters;  // literal rule: Sinkhorn iterations per greedy step
@@ -163,14 +163,22 @@ int launch_slab(const float* cost, int64_t ldc, const int32_t* nbr, const DevPar
 // Column tiles of the elementwise cost pass: the number of partial row sums
 // it writes per row into g0, [B][fst_apply_slots(ldc)][N].
 int fst_apply_slots(int64_t ldc);
-// K5: K greedy steps; order32[b*K + l] = token added at step l.  Local
-// lazy SGS (g < N) also needs rev_off [B][N+1] and rev [B][N*g] (scratch for
-// the reverse neighbourhoods).
+// K5: K greedy steps; order32[b*K + l] = token added at step l.  sgs_mode 0
+// needs push_ws (sgs_push_ws_bytes bytes, 256-byte aligned), sgs_mode 1
+// partials and counters.
 int launch_sgs(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
                const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                int32_t* order32, float* gains, double* objective, uint64_t* partials,
-               uint32_t* counters, int* status, cudaStream_t s, const float* g0 = nullptr,
-               int32_t* rev_off = nullptr, int32_t* rev = nullptr);
+               uint32_t* counters, int* status, cudaStream_t s, const float* g0, void* push_ws);
+// sgs_mode 0: exact gains kept up to date over lists of live candidates.  g0
+// (dense, may be null): the cost pass's partial sums of the first gains.
+size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc);
+int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
+                    const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
+                    int32_t* order32, float* gains, double* objective, int* status,
+                    cudaStream_t s, const float* g0, void* ws);
+// The fixed-point scale of the gains for a coverage cost m0 (sgs_gain.cuh).
+int gain_fx(float m0);
 // K5 as Sec. 3.5 prints it (sgs_mode 2): entropic semi-relaxed OT residual
 // and the residual-weighted local cost; needs the dense cost [B][N][ldc]
 // and sgs_literal_ws_bytes(B, N, K) bytes of scratch (256-byte aligned).

@@ -31,7 +31,7 @@ def main():
     ap.add_argument("--norm-mode", type=int, default=0, choices=(0, 1),
                     help="feature normaliser: 0 min-max over all pairs, 1 bounded (d_f / 2)")
     ap.add_argument("--sgs-mode", type=int, default=0, choices=(0, 1, 2),
-                    help="0 lazy, 1 every gain every step, 2 the rule as printed (entropic OT)")
+                    help="0 gains kept up to date, 1 every gain every step, 2 the rule as printed (entropic OT)")
     ap.add_argument("--warmup", type=int, default=1)
     ap.add_argument("--repeat", type=int, default=3)
     ap.add_argument("--stages", action="store_true",
