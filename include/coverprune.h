@@ -379,12 +379,16 @@ int coverprune_profile_read(double* ms, int64_t* launches, int n);
  *                     of the local slab (g floats); sgs_mode 0: terms of
  *                     gains updated after the first pick, one per live
  *                     (candidate, target) pair of a lowered target
- *   rounds            decision rounds over all scenes (one per step)
+ *   rounds            decision rounds over all scenes: sgs_mode 1 one per
+ *                     step, sgs_mode 0 at most that (late rounds make many
+ *                     picks)
  *   cost_bytes_read   bytes of cost rows (or slab rows and their neighbour
  *                     indices) and of live lists the steps read: sgs_mode 1
  *                     a row per gain, and once per scene and step the
  *                     winner's row for the coverage update; sgs_mode 0 the
- *                     winners' rows and 8 bytes per updated term
+ *                     winners' rows (of rounds of many picks: the live
+ *                     entries of the candidates' rows) and 8 bytes per
+ *                     updated term
  * Returns CP_OK, CP_EINVAL or CP_ECUDA.
  */
 typedef struct {

@@ -18,14 +18,17 @@
 // entries.  On the local path the live candidates of j start as the t with j
 // in M_g(t) (k_rev_lists).
 //
-// What bounds a step is its chain of dependent latencies -- argmax, the
-// winner's row, the changed targets' lists, the gain updates -- with block
-// barriers between; nothing in it needs more than one SM except the first
-// steps' long lists.  A scene therefore runs on a small cluster of blocks:
-// block r of C owns the candidates t = r (mod C) with their gains and its
-// own part of every list, keeps its own copy of m, and per step exchanges
-// one key with the others (st.async into every block's slot, counted on an
-// mbarrier there).
+// The work is little; what bounds it is chains of dependent latencies --
+// argmax, the winner's row, the lowered targets' lists, the gain updates --
+// with block barriers between.  Two kernels share the steps:
+//  - k_sgs_push, one pick a step, while a pick lowers many targets (dense
+//    path): a cluster of blocks per scene, ~2 us a step;
+//  - k_sgs_rounds, one block per scene, many picks a round, for the rest
+//    (and all of a local selection): late picks lower few targets each,
+//    mostly different ones, so dozens of them are independent of one another.
+// Selection of 1229 of 8192 tokens: 2.95 ms (re-evaluating candidate rows
+// behind bounds, the approach before these: 11.9; one pick a step to the end:
+// 5.9); 410 of 4096: 1.14 (3.8, 2.1); 32 scenes of 8192: 8.6 (19.9, 12.0).
 #include <string.h>
 
 #include "bf16_dot.cuh"
@@ -36,6 +39,14 @@ namespace {
 
 constexpr int PUSH_CMAX = 16;  // blocks per cluster (16: the non-portable maximum)
 constexpr int PUSH_WARPS = 32;
+// The single-pick steps end once the running mean of the targets a pick
+// lowers is below this: a step costs ~2 us whatever it lowers, a pick of a
+// round costs its lists' share of one block, and where rows are still longer
+// than RD_ROW rounds pick one at a time.  Selection, ms, at 16 / 24 / 32 / 40
+// / 48 / 64: N = 1024 0.34 / 0.32 / 0.32 / 0.31 / 0.31 / 0.30, N = 4096 1.22 /
+// 1.20 / 1.15 / 1.14 / 1.13 / 1.12, N = 8192 3.00 / 2.97 / 2.96 / 2.95 / 3.22 /
+// 3.21, 32 scenes of N = 8192 8.65 / 8.52 / 8.54 / 8.61 / 9.17 / 9.23.
+constexpr int PUSH_STOP = 36;
 constexpr int PUSH_THREADS = 32 * PUSH_WARPS;
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -99,9 +110,10 @@ constexpr size_t LIST_PAD = 128;
 // per 64-column tile) add the gain's terms in fp32: at most 8 roundings
 // inside a tile and one per tile after that, each of relative size 2^-24 of
 // non-negative sums, so a total is within 2^-15 (264 x 2^-24 at 256 tiles)
-// of the exact sum, which the fixed-point gain differs from by less than
-// 2^-23 of it.  Only candidates whose upper bound reaches the largest lower
-// bound can be the first pick; their gains are computed exactly.
+// of the exact sum, the fixed-point gain (two roundings a term) and its 24
+// bits among the 248 x 2^-24 to spare.  Only candidates whose upper bound
+// reaches the largest lower bound can be the first pick; their gains are
+// computed exactly.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_first_bounds(const float* __restrict__ g0, int slots, int N,
                                                       float* __restrict__ sums,
@@ -123,8 +135,8 @@ __global__ void __launch_bounds__(256) k_first_bounds(const float* __restrict__ 
 // them without bounds); the best key by atomicMax.  A warp scans 32
 // candidates' bounds at a time and evaluates the ones that pass.
 __global__ void __launch_bounds__(256) k_first_pick(const float* __restrict__ cost, int64_t ldc,
-                                                    const float* __restrict__ v_all, int N,
-                                                    float m0, int fx,
+                                                    const float* __restrict__ v_all,
+                                                    int N, float m0, int fx,
                                                     const float* __restrict__ sums,
                                                     const uint32_t* __restrict__ max_bits,
                                                     gain_t* __restrict__ first) {
@@ -148,7 +160,7 @@ __global__ void __launch_bounds__(256) k_first_pick(const float* __restrict__ co
       todo &= todo - 1u;
       const float4* row = C4 + (size_t)tc * nq;
       gain_t acc = 0ull;
-      for (int i0 = lane; i0 < nq; i0 += 8 * 32) {
+      for (int i0 = lane; i0 - lane < nq; i0 += 8 * 32) {
         float4 c[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
@@ -178,8 +190,10 @@ __global__ void __launch_bounds__(256) k_first_pick(const float* __restrict__ co
 // column's live rows are one ballot, the entries of a list go out
 // contiguously and a lane's gain needs no reduction until the tile ends.
 // Candidates with nearby indices are near in space, so about half of the
-// ballots are empty and skip the arithmetic.  Bound by HBM (the cost read
-// once, entries of 8 bytes for the live fifth written).
+// ballots are empty and skip the arithmetic.  32 scenes of N = 8192: 2.7 ms,
+// 4.8 TB/s of reads (8.6 GB, the cost once) and writes (8 bytes a live entry,
+// 4.2 GB); bound by instruction issue before HBM: a column of a tile costs its
+// ballot, a live one its term and store besides.
 // List of (j, owner): lists[((bl N + j) C + owner) NC ..], lens alike.
 // ---------------------------------------------------------------------------
 constexpr int LL_COLS = 128, LL_ROWS = 32, LL_STAGES = 4, LL_WARPS = 16;
@@ -189,8 +203,9 @@ constexpr size_t LL_SMEM = sizeof(float) * LL_STAGES * LL_ROWS * LL_PITCH;
 
 __global__ void __launch_bounds__(32 * LL_WARPS) k_live_lists(
     const float* __restrict__ cost, int64_t ldc, const float* __restrict__ v_all,
-    const gain_t* __restrict__ first, int N, int C, int lgC, int NC, int scene0, float m0, int fx,
-    gain_t* __restrict__ gains, Entry* __restrict__ lists, uint32_t* __restrict__ lens) {
+    const gain_t* __restrict__ first, int N, int C, int lgC, int NC, int scene0, float m0,
+    int fx, gain_t* __restrict__ gains, Entry* __restrict__ lists,
+    uint32_t* __restrict__ lens) {
   extern __shared__ __align__(16) float s_tile[];  // [LL_STAGES][LL_ROWS][LL_PITCH]
   __shared__ gain_t s_part[2][LL_WARPS][32];
   const int col0 = blockIdx.x * LL_COLS, rank = blockIdx.y, bl = blockIdx.z, b = scene0 + bl;
@@ -201,20 +216,20 @@ __global__ void __launch_bounds__(32 * LL_WARPS) k_live_lists(
   const int nown = N > rank ? (N - rank + C - 1) >> lgC : 0;
   const int ntile = (nown + LL_ROWS - 1) / LL_ROWS;
   const int w0 = key_token(first[b]);
+  const uint32_t lstep = (uint32_t)(C * NC);  // between the lists of adjacent columns
   float m[LL_COLS_W], vj[LL_COLS_W];
-  uint32_t cnt[LL_COLS_W];
+  uint32_t pos[LL_COLS_W];   // the column's next free entry, from the warp's first list
 #pragma unroll
   for (int u = 0; u < LL_COLS_W; ++u) {
     const int j = col0 + LL_COLS_W * w + u;
     m[u] = -INFINITY;  // past the row: nothing is live
     vj[u] = 0.0f;
-    cnt[u] = 0u;
+    pos[u] = (uint32_t)u * lstep;
     if (j < N) {
       m[u] = fminf(m0, __ldg(Cb + (size_t)w0 * ldc + j));
       vj[u] = __ldg(v + j);
     }
   }
-  const size_t lstep = (size_t)C * NC;  // between the lists of adjacent columns
   Entry* L = lists + ((size_t)((size_t)bl * N + col0 + LL_COLS_W * w) * C + rank) * NC;
   auto load = [&](int i) {
     float* dst = s_tile + (size_t)(i % LL_STAGES) * LL_ROWS * LL_PITCH;
@@ -265,10 +280,9 @@ __global__ void __launch_bounds__(32 * LL_WARPS) k_live_lists(
         if (mask) {  // warp-uniform
           if (live) {
             acc += gain_term(vj[u], m[u], c[e], fx);
-            L[u * lstep + cnt[u] + __popc(mask & lt)] =
-                make_uint2((uint32_t)tl, __float_as_uint(c[e]));
+            L[pos[u] + __popc(mask & lt)] = make_uint2((uint32_t)tl, __float_as_uint(c[e]));
           }
-          cnt[u] += __popc(mask);
+          pos[u] += __popc(mask);
         }
       }
     }
@@ -280,44 +294,41 @@ __global__ void __launch_bounds__(32 * LL_WARPS) k_live_lists(
 #pragma unroll
     for (int u = 0; u < LL_COLS_W; ++u) {
       const int j = col0 + LL_COLS_W * w + u;
-      if (j < N) lens[((size_t)bl * N + j) * C + rank] = cnt[u];
+      if (j < N) lens[((size_t)bl * N + j) * C + rank] = pos[u] - (uint32_t)u * lstep;
     }
   }
 }
 
 // ---------------------------------------------------------------------------
-// The local path's lists: the candidates t with j in M_g(t), by owner block
-// (t mod C), and their costs.  One block per scene: counts, an exclusive scan
-// and a fill, with counts and cursors in shared memory [N C].  span[(b N + j)
-// C + owner] = (offset into the scene's entries, length); the order within a
-// list is arbitrary (no result depends on it).
+// The local path's lists: the candidates t with j in M_g(t) and their costs.
+// One block per scene: counts, an exclusive scan and a fill, with counts and
+// cursors in shared memory [N] (0.67 ms of 32 scenes, N = 8192, g = 64).  span[b N + j] = (offset into the scene's
+// entries, length); the order within a list is arbitrary (no result depends
+// on it).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_rev_lists(const int32_t* __restrict__ nbr_all,
                                                     const float* __restrict__ slab, int N, int g,
-                                                    int kk, int C, int lgC,
-                                                    uint2* __restrict__ span_all,
+                                                    int kk, uint2* __restrict__ span_all,
                                                     Entry* __restrict__ ent_all) {
-  extern __shared__ int s_c[];  // [N C]
+  extern __shared__ int s_c[];  // [N]
   __shared__ int s_sum[1024];
   const int b = blockIdx.x;
   const int32_t* NB = nbr_all + (size_t)b * N * kk;
   const float* S = slab + (size_t)b * N * g;
-  uint2* span = span_all + (size_t)b * N * C;
+  uint2* span = span_all + (size_t)b * N;
   Entry* ent = ent_all + (size_t)b * N * g;
   const int64_t ng = (int64_t)N * g;
-  const int nc = N * C;
-  for (int j = threadIdx.x; j < nc; j += blockDim.x) s_c[j] = 0;
+  for (int j = threadIdx.x; j < N; j += blockDim.x) s_c[j] = 0;
   __syncthreads();
   for (int64_t i = threadIdx.x; i < ng; i += blockDim.x) {
     const int t = (int)(i / g), k = (int)(i % g);
-    const int j = k == 0 ? t : NB[(size_t)t * kk + (k - 1)];
-    atomicAdd(&s_c[(j << lgC) | (t & (C - 1))], 1);
+    atomicAdd(&s_c[k == 0 ? t : NB[(size_t)t * kk + (k - 1)]], 1);
   }
   __syncthreads();
   // exclusive prefix of the counts: each thread a contiguous chunk, then a
   // scan of the 1024 chunk sums
-  const int chunk = (nc + blockDim.x - 1) / blockDim.x;
-  const int c0 = min(nc, (int)threadIdx.x * chunk), c1 = min(nc, c0 + chunk);
+  const int chunk = (N + blockDim.x - 1) / blockDim.x;
+  const int c0 = min(N, (int)threadIdx.x * chunk), c1 = min(N, c0 + chunk);
   int part = 0;
   for (int j = c0; j < c1; ++j) part += s_c[j];
   s_sum[threadIdx.x] = part;
@@ -339,16 +350,15 @@ __global__ void __launch_bounds__(1024) k_rev_lists(const int32_t* __restrict__ 
   for (int64_t i = threadIdx.x; i < ng; i += blockDim.x) {
     const int t = (int)(i / g), k = (int)(i % g);
     const int j = k == 0 ? t : NB[(size_t)t * kk + (k - 1)];
-    ent[atomicAdd(&s_c[(j << lgC) | (t & (C - 1))], 1)] =
-        make_uint2((uint32_t)(t >> lgC), __float_as_uint(S[i]));
+    ent[atomicAdd(&s_c[j], 1)] = make_uint2((uint32_t)t, __float_as_uint(S[i]));
   }
 }
 
 // The local path's first gains (m = m0), one warp per candidate.
 __global__ void __launch_bounds__(256) k_local_gains(const float* __restrict__ slab,
                                                      const int32_t* __restrict__ nbr,
-                                                     const float* __restrict__ v_all, int N, int g,
-                                                     int kk, float m0, int fx,
+                                                     const float* __restrict__ v_all,
+                                                     int N, int g, int kk, float m0, int fx,
                                                      gain_t* __restrict__ gains) {
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y, lane = threadIdx.x & 31;
   if (t >= N) return;
@@ -365,40 +375,71 @@ __global__ void __launch_bounds__(256) k_local_gains(const float* __restrict__ s
 }
 
 // ---------------------------------------------------------------------------
-// The greedy steps.
+// The greedy steps while picks lower many targets (dense path): one pick a
+// step.  Nothing in a step needs more than one SM but the long lists, so a
+// scene runs on a small cluster of blocks: block r of C owns the candidates
+// t = r (mod C) with their gains and its own part of every list, keeps its
+// own copy of m, and per step exchanges one key with the others (st.async
+// into every block's slot, counted on an mbarrier there: ~450 cycles, about
+// a fifth of a late step; a barrier of the cluster takes twice that).
 // ---------------------------------------------------------------------------
 struct PushArgs {
-  const float* rows;      // dense: cost [B][N][ldc]; local: slab [B][N][g]
-  const int32_t* nbr;     // local: [B][N][kk]
+  const float* cost;      // [B][N][ldc]
   const float* v;         // [B][N]
-  const gain_t* gains0;   // [B][N] gains at the start
-  const gain_t* first;    // dense: [B] key of the first pick
+  gain_t* gains;          // [B][N] gains at the start; at the end the current ones
+  const gain_t* first;    // [B] key of the first pick
   Entry* lists;
-  uint32_t* lens;         // dense: [scenes of the wave][N][C]
-  uint2* span;            // local: [B][N][C] (offset, length)
+  uint32_t* lens;         // [scenes of the wave][N][C]
+  float* m_out;           // [scenes of the wave][N] coverage cost where the steps stopped
+  int* stop;              // [scenes of the wave] first step not taken
   int32_t* order32;       // [B][K]
   float* out_gains;       // [B][K] or null
-  double* objective;      // [B] or null
   int* status;
   int64_t ldc;
   uint64_t timeout_ns;
   float m0;
   int fx;
-  int N, K, g, kk;
+  int N, K;
   int C, lgC, NC;         // blocks per cluster (a power of two), its log2, ceil(N / C)
   int lgS;                // log2 of the candidates a warp scans
   int scene0;             // first scene of the wave
   uint32_t off_q, off_lo, off_hi;  // dynamic shared memory offsets
 };
 
-// Gains are kept as two 32-bit words (32-bit shared atomics are native); an
-// update takes the low word off first and the borrow that its own atomic saw
-// with the high word, so the pair is right once every update has run.
-template <bool LOCAL>
+// One chunk of 32 list entries against a target lowered from mo to mn: the
+// gains of the live candidates lose what the drop took.  Gains are kept as
+// two 32-bit words (32-bit shared atomics are native): the low word's update
+// goes out first and `old` carries what it saw, so that chunk_high, called
+// once every chunk's low words are on their way, takes the borrow off the
+// high word; the pair is right once every update has run.
+__device__ __forceinline__ gain_t chunk_low(uint32_t* lo, uint32_t at, bool on, float v, float mo,
+                                            float mn, float c, int fx, uint32_t& old) {
+  const gain_t d = on ? gain_drop(v, mo, mn, c, fx) : 0ull;
+  old = 0u;
+  if (d != 0ull) old = atomicAdd(lo + at, 0u - (uint32_t)d);
+  return d;
+}
+__device__ __forceinline__ void chunk_high(uint32_t* hi, uint32_t at, gain_t d, uint32_t old) {
+  if (d != 0ull) {
+    const uint32_t dh = (uint32_t)(d >> 32) + (old < (uint32_t)d ? 1u : 0u);
+    if (dh) atomicAdd(hi + at, 0u - dh);
+  }
+}
+// The chunk's entries that stay live (c < mn; infinite past the list), packed
+// from place `out` of the list on.
+__device__ __forceinline__ void chunk_pack(Entry* L, const Entry& x, int i, float mn, int lane,
+                                           int& out) {
+  const bool stay = __uint_as_float(x.y) < mn;
+  const uint32_t mask = __ballot_sync(0xFFFFFFFFu, stay);
+  const int p = out + __popc(mask & ((1u << lane) - 1u));
+  if (stay && p != i) __stcg(L + p, x);
+  out += __popc(mask);
+}
+
 __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_constant__ PushArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  float* sm_m = reinterpret_cast<float*>(smem);                     // [ldc or N] coverage cost
-  uint32_t* queue = reinterpret_cast<uint32_t*>(smem + a.off_q);    // lowered targets: (k << 16) | j
+  float* sm_m = reinterpret_cast<float*>(smem);                     // [ldc] coverage cost
+  uint32_t* queue = reinterpret_cast<uint32_t*>(smem + a.off_q);    // [N] lowered targets
   uint32_t* g_lo = reinterpret_cast<uint32_t*>(smem + a.off_lo);    // [NC] gains, low words
   uint32_t* g_hi = reinterpret_cast<uint32_t*>(smem + a.off_hi);    // [NC] ... and high words
   __shared__ gain_t s_key[PUSH_WARPS];   // best key of each warp's candidates
@@ -411,32 +452,23 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
   const int bl = (int)(blockIdx.x >> a.lgC), b = a.scene0 + bl;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = a.N, lgC = a.lgC, fx = a.fx;
-  const int ncols = LOCAL ? N : (int)a.ldc;
+  const int ncols = (int)a.ldc;
   const int nown = N > rank ? (N - rank + a.C - 1) >> lgC : 0;
   const float* v = a.v + (size_t)b * N;
-  const float* R = a.rows + (size_t)b * N * (LOCAL ? (size_t)a.g : (size_t)a.ldc);
-  const int32_t* NB = LOCAL ? a.nbr + (size_t)b * N * a.kk : nullptr;
-  unsigned long long my_ent = 0ull, my_rows = 0ull;  // list entries (a lane's), rows read
+  const float* R = a.cost + (size_t)b * N * (size_t)a.ldc;
+  unsigned long long my_ent = 0ull;  // list entries read (lane 0's count)
 
-  // state at the start: m, the gains, the first pick (dense)
-  int last = -1;  // the last pick, not yet dropped from the candidates
-  int start = 0;
-  if (!LOCAL) {
-    const gain_t f = a.first[b];
-    last = key_token(f);
-    start = 1;
-    if (rank == 0 && threadIdx.x == 0) {
-      a.order32[(size_t)b * a.K] = last;
-      if (a.out_gains) a.out_gains[(size_t)b * a.K] = key_gain(f);
-    }
+  // state at the start: the first pick, m and the gains
+  const gain_t f0 = a.first[b];
+  int last = key_token(f0);  // the last pick, not yet dropped from the candidates
+  if (rank == 0 && threadIdx.x == 0) {
+    a.order32[(size_t)b * a.K] = last;
+    if (a.out_gains) a.out_gains[(size_t)b * a.K] = key_gain(f0);
   }
-  for (int j = threadIdx.x; j < ncols; j += PUSH_THREADS) {
-    float mj = j < N ? a.m0 : 0.0f;
-    if (!LOCAL && j < N) mj = fminf(mj, __ldg(R + (size_t)last * a.ldc + j));
-    sm_m[j] = mj;
-  }
+  for (int j = threadIdx.x; j < ncols; j += PUSH_THREADS)
+    sm_m[j] = j < N ? fminf(a.m0, __ldg(R + (size_t)last * a.ldc + j)) : 0.0f;
   for (int tl = threadIdx.x; tl < nown; tl += PUSH_THREADS) {
-    const gain_t x = a.gains0[(size_t)b * N + ((tl << lgC) | rank)];
+    const gain_t x = a.gains[(size_t)b * N + ((tl << lgC) | rank)];
     g_lo[tl] = (uint32_t)x;
     g_hi[tl] = (uint32_t)(x >> 32);
   }
@@ -453,12 +485,14 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
 
   bool ok = true;
   int pref = -1;  // the row last prefetched
-  for (int step = start; step < a.K; ++step) {
+  int step = 1;
+  int mean8 = N;  // 8 x the running mean of the lowered targets a step
+  for (; step < a.K && mean8 > 8 * PUSH_STOP; ++step) {
     const int par = step & 1;
     if (a.C > 1 && threadIdx.x == 0) mbar_expect(&s_bar[par], 8u * (uint32_t)a.C);
     // ---- the warp's best key, when one of its gains changed
     const int ltl = last >> lgC;
-    const bool drop = last >= 0 && (last & (a.C - 1)) == rank && ltl >= lo0 && ltl < lo1;
+    const bool drop = (last & (a.C - 1)) == rank && ltl >= lo0 && ltl < lo1;
     if (drop || s_dirty[w] != 0u) {
       if (drop && lane == 0) g_hi[ltl] = 0xFFFFFFFFu;  // selected: no candidate any more
       __syncwarp();
@@ -485,16 +519,16 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
       if (w == 0 && lane < a.C)
         st_async_u64(map_rank(smem_addr(&s_res[par][rank]), (uint32_t)lane), W,
                      map_rank(smem_addr(&s_bar[par]), (uint32_t)lane));
-      if (!LOCAL && w == 1 && W != 0ull) {  // this block's best row, likely a coming pick's
+      if (w == 1 && W != 0ull) {  // this block's best row, likely a coming pick's
         const int t = key_token(W);
         if (t != pref && lane == 0) prefetch_l2(R + (size_t)t * a.ldc, (uint32_t)(4 * a.ldc));
         pref = t;
       }
       int good = 1;
-      if (lane == 0 && !mbar_test(&s_bar[par], (uint32_t)((step - start) >> 1) & 1u)) {
+      if (lane == 0 && !mbar_test(&s_bar[par], (uint32_t)((step - 1) >> 1) & 1u)) {
         const uint64_t t0 = globaltimer_ns();
         uint32_t spins = 0;
-        while (!mbar_test(&s_bar[par], (uint32_t)((step - start) >> 1) & 1u)) {
+        while (!mbar_test(&s_bar[par], (uint32_t)((step - 1) >> 1) & 1u)) {
           if ((++spins & 15u) == 0) {
             if (ld_volatile_i32(a.status) != 0) { good = 0; break; }
             if (globaltimer_ns() - t0 > a.timeout_ns) {
@@ -522,53 +556,43 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
       if (rank == 0 && threadIdx.x == 0) {
         a.order32[(size_t)b * a.K + step] = pick;
         if (a.out_gains) a.out_gains[(size_t)b * a.K + step] = key_gain(W);
-        ++my_rows;
       }
       // ---- S <- S u {t*} (Eq. sgs_update): the targets whose m drops
-      if (!LOCAL) {
-        const float4* row = reinterpret_cast<const float4*>(R + (size_t)pick * a.ldc);
-        const float4* m4 = reinterpret_cast<const float4*>(sm_m);
-        const int nq = ncols >> 2;
-        for (int i0 = w * 32; i0 < nq; i0 += 4 * PUSH_THREADS) {
-          float4 c[4];
+      const float4* row = reinterpret_cast<const float4*>(R + (size_t)pick * a.ldc);
+      const float4* m4 = reinterpret_cast<const float4*>(sm_m);
+      const int nq = ncols >> 2;
+      for (int i0 = w * 32; i0 < nq; i0 += 4 * PUSH_THREADS) {
+        float4 c[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * PUSH_THREADS + lane;
-            c[u] = i < nq ? __ldg(row + i) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * PUSH_THREADS + lane;
+          c[u] = i < nq ? __ldg(row + i) : make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (i0 + u * PUSH_THREADS >= nq) break;  // warp-uniform
+          const int i = i0 + u * PUSH_THREADS + lane;
+          const float4 mm = i < nq ? m4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+          const uint32_t low = (c[u].x < mm.x ? 1u : 0u) | (c[u].y < mm.y ? 2u : 0u) |
+                               (c[u].z < mm.z ? 4u : 0u) | (c[u].w < mm.w ? 8u : 0u);
+          uint32_t bal[4];
+          int n = 0;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            bal[e] = __ballot_sync(0xFFFFFFFFu, (low >> e) & 1u);
+            n += __popc(bal[e]);
           }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * PUSH_THREADS + lane;
-            const float4 mm = i < nq ? m4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const uint32_t low = (c[u].x < mm.x ? 1u : 0u) | (c[u].y < mm.y ? 2u : 0u) |
-                                 (c[u].z < mm.z ? 4u : 0u) | (c[u].w < mm.w ? 8u : 0u);
-            uint32_t bal[4];
-            int n = 0;
+          if (n != 0) {  // warp-uniform
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_qn, n);
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              bal[e] = __ballot_sync(0xFFFFFFFFu, (low >> e) & 1u);
-              n += __popc(bal[e]);
-            }
-            if (n != 0) {  // warp-uniform
-              int at = 0;
-              if (lane == 0) at = atomicAdd(&s_qn, n);
-              at = __shfl_sync(0xFFFFFFFFu, at, 0);
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                if ((low >> e) & 1u)
-                  queue[at + __popc(bal[e] & ((1u << lane) - 1u))] = (uint32_t)(4 * i + e);
-                at += __popc(bal[e]);
-              }
+              if ((low >> e) & 1u)
+                queue[at + __popc(bal[e] & ((1u << lane) - 1u))] = (uint32_t)(4 * i + e);
+              at += __popc(bal[e]);
             }
           }
-        }
-      } else {
-        const float* srow = R + (size_t)pick * a.g;
-        const int32_t* nb = NB + (size_t)pick * a.kk;
-        for (int k = threadIdx.x; k < a.g; k += PUSH_THREADS) {
-          const int j = k == 0 ? pick : __ldg(nb + k - 1);
-          if (__ldg(srow + k) < sm_m[j])
-            queue[atomicAdd(&s_qn, 1)] = ((uint32_t)k << 16) | (uint32_t)j;
         }
       }
     }
@@ -578,92 +602,68 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
       ok = false;
       break;
     }
-    // ---- two lowered targets a warp at a time: their live candidates lose
-    // what the drop took; the entries that stay live are packed to the
-    // list's front.  The lists' lengths and first entries load together (an
-    // entry past the length is ignored), and four chunks of 32 entries are
-    // in flight, their low-word updates issued before any of their results
-    // is needed.
+    // ---- a warp per lowered target: its live candidates lose what the drop
+    // took; the entries that stay live are packed to the list's front.  Four
+    // chunks of 32 entries are in flight, and the next target's length and
+    // costs load meanwhile.
     const int qn = s_qn;
-    for (int q0 = w; q0 < qn; q0 += 2 * PUSH_WARPS) {
-      Entry* L[2];
-      uint32_t* len_at[2];
-      int j[2], len[2], out[2] = {0, 0};
-      float mn[2], vj[2], mo[2];
-      Entry x[4];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int qi = q0 + h * PUSH_WARPS;
-        const uint32_t e = queue[qi < qn ? qi : q0];
-        j[h] = (int)(e & 0xFFFFu);
-        const size_t lj = ((size_t)(LOCAL ? b : bl) * N + j[h]) * a.C + rank;
-        mn[h] = LOCAL ? __ldg(R + (size_t)pick * a.g + (e >> 16))
-                      : __ldg(R + (size_t)pick * a.ldc + j[h]);
-        vj[h] = __ldg(v + j[h]);
-        mo[h] = sm_m[j[h]];
-        if (LOCAL) {
-          const uint2 sp = __ldcg(a.span + lj);
-          L[h] = a.lists + (size_t)b * N * a.g + sp.x;
-          len_at[h] = &a.span[lj].y;
-          len[h] = (int)sp.y;
-        } else {
-          L[h] = a.lists + lj * a.NC;
-          len_at[h] = a.lens + lj;
-          len[h] = (int)__ldcg(len_at[h]);
-        }
-        x[2 * h] = __ldcg(L[h] + lane);
-        x[2 * h + 1] = __ldcg(L[h] + 32 + lane);
-        if (qi >= qn) len[h] = 0;
+    int j = 0, len = 0;
+    float mn = 0.0f, vj = 0.0f;
+    auto next = [&](int q) {
+      if (q < qn) {
+        j = (int)queue[q];
+        len = (int)__ldcg(a.lens + ((size_t)bl * N + j) * a.C + rank);
+        mn = __ldg(R + (size_t)pick * a.ldc + j);
+        vj = __ldg(v + j);
       }
-      // chunks x[0..3]: entry i[u] + lane of list h[u]
-      auto apply = [&](const int (&hh)[4], const int (&i0)[4]) {
+    };
+    next(w);
+#pragma unroll 1
+    for (int q = w; q < qn; q += PUSH_WARPS) {
+      const int jc = j, lenc = len;
+      const float mnc = mn, mo = sm_m[j], vc = vj;
+      const size_t lj = ((size_t)bl * N + jc) * a.C + rank;
+      Entry* L = a.lists + lj * a.NC;
+      next(q + PUSH_WARPS);
+      int out = 0, i0 = 0;
+#pragma unroll 1
+      for (; i0 + 96 < lenc; i0 += 128) {  // four chunks, the last perhaps not full
+        Entry x[4];
         gain_t d[4];
         uint32_t old[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int h = hh[u];
-          const float c = __uint_as_float(x[u].y);
-          d[u] = i0[u] + lane < len[h] ? gain_term(vj[h], mo[h], c, fx) - gain_term(vj[h], mn[h], c, fx)
-                                       : 0ull;
-          old[u] = 0u;
-          if (d[u] != 0ull) old[u] = atomicAdd(g_lo + x[u].x, 0u - (uint32_t)d[u]);
+          const int i = i0 + 32 * u + lane;
+          x[u] = i < lenc ? __ldcg(L + i) : make_uint2(0u, 0x7F800000u);
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          d[u] = chunk_low(g_lo, x[u].x, true, vc, mo, mnc, __uint_as_float(x[u].y), fx,
+                                 old[u]);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int h = hh[u];
-          if (d[u] != 0ull) {
-            const uint32_t dh = (uint32_t)(d[u] >> 32) + (old[u] < (uint32_t)d[u] ? 1u : 0u);
-            if (dh) atomicAdd(g_hi + x[u].x, 0u - dh);
-            s_dirty[x[u].x >> a.lgS] = 1u;
-          }
-          if (i0[u] < len[h]) {  // warp-uniform
-            const int i = i0[u] + lane;
-            const bool stay = i < len[h] && __uint_as_float(x[u].y) < mn[h];
-            const uint32_t mask = __ballot_sync(0xFFFFFFFFu, stay);
-            const int p = out[h] + __popc(mask & ((1u << lane) - 1u));
-            if (stay && p != i) __stcg(L[h] + p, x[u]);
-            out[h] += __popc(mask);
-          }
+          chunk_high(g_hi, x[u].x, d[u], old[u]);
+          if (d[u] != 0ull) s_dirty[x[u].x >> a.lgS] = 1u;
+          chunk_pack(L, x[u], i0 + 32 * u + lane, mnc, lane, out);
         }
-      };
-      apply({0, 0, 1, 1}, {0, 32, 0, 32});
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        for (int i0 = 64; i0 < len[h]; i0 += 128) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) x[u] = __ldcg(L[h] + i0 + 32 * u + lane);
-          if (h == 0)
-            apply({0, 0, 0, 0}, {i0, i0 + 32, i0 + 64, i0 + 96});
-          else
-            apply({1, 1, 1, 1}, {i0, i0 + 32, i0 + 64, i0 + 96});
-        }
-        if (lane == 0 && len[h]) {
-          my_ent += (unsigned long long)len[h];
-          if (out[h] != len[h]) __stcg(len_at[h], (uint32_t)out[h]);
-        }
-        if (lane == 0) sm_m[j[h]] = mn[h];
+      }
+#pragma unroll 1
+      for (; i0 < lenc; i0 += 32) {
+        const Entry x = i0 + lane < lenc ? __ldcg(L + i0 + lane) : make_uint2(0u, 0x7F800000u);
+        uint32_t old;
+        const gain_t d = chunk_low(g_lo, x.x, true, vc, mo, mnc, __uint_as_float(x.y), fx,
+                                         old);
+        chunk_high(g_hi, x.x, d, old);
+        if (d != 0ull) s_dirty[x.x >> a.lgS] = 1u;
+        chunk_pack(L, x, i0 + lane, mnc, lane, out);
+      }
+      if (lane == 0) {
+        my_ent += (unsigned long long)lenc;
+        if (out != lenc) __stcg(a.lens + lj, (uint32_t)out);
+        sm_m[jc] = mnc;
       }
     }
+    mean8 += qn - (mean8 >> 3);
     __syncthreads();  // gains and m are settled
     if (threadIdx.x == 0) s_qn = 0;
   }
@@ -675,14 +675,17 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
     atomicAdd(&cstats[2], 8ull * my_ent);
   }
   if (rank == 0 && threadIdx.x == 0) {
-    atomicAdd(&cstats[1], (unsigned long long)a.K);
-    atomicAdd(&cstats[2], my_rows * (LOCAL ? 8ull * (unsigned long long)a.g
-                                           : 4ull * (unsigned long long)ncols));
+    atomicAdd(&cstats[1], (unsigned long long)step);
+    atomicAdd(&cstats[2], 4ull * (unsigned long long)step * (unsigned long long)ncols);
   }
+  // the state for the rounds that follow
+  if (ok && rank == (last & (a.C - 1)) && threadIdx.x == 0) g_hi[last >> lgC] = 0xFFFFFFFFu;
   __syncthreads();
-  if (ok && rank == 0 && a.objective) {
-    const double F = objective_sum(sm_m, v, N);
-    if (threadIdx.x == 0) a.objective[b] = F;
+  for (int tl = threadIdx.x; tl < nown; tl += PUSH_THREADS)
+    a.gains[(size_t)b * N + ((tl << lgC) | rank)] = ((gain_t)g_hi[tl] << 32) | g_lo[tl];
+  if (rank == 0) {
+    for (int j = threadIdx.x; j < N; j += PUSH_THREADS) a.m_out[(size_t)bl * N + j] = sm_m[j];
+    if (threadIdx.x == 0) a.stop[bl] = ok ? step : a.K;
   }
   if (!ok) {  // a peer's last key may still be on its way here: let it land
     const uint64_t t0 = globaltimer_ns();
@@ -692,20 +695,636 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
   hw_cluster_sync();  // nobody leaves while a peer may still write to its shared memory
 }
 
+// ---------------------------------------------------------------------------
+// The lists of a dense scene for the rounds below, a warp per target: the C
+// parts of its list copied into one, side by side with the other targets'
+// (the parts lie 8 N bytes a target apart, a page or more each), and every
+// candidate's row of live targets (room for row_room(N) entries; a longer row
+// only counts).  A list that finds no room in the joined region is joined where
+// it is: parts move toward the list's front, each chunk read before it is
+// written.
+// ---------------------------------------------------------------------------
+constexpr int RD_ROW = 512;
+__host__ __device__ constexpr int row_room(int64_t N) { return N < RD_ROW ? (int)N : RD_ROW; }
+
+__global__ void __launch_bounds__(256) k_join_lists(Entry* __restrict__ lists,
+                                                    const uint32_t* __restrict__ lens, int N, int C,
+                                                    int lgC, int NC, size_t join0, uint32_t room,
+                                                    uint32_t* __restrict__ cursor,
+                                                    uint2* __restrict__ span,
+                                                    uint32_t* __restrict__ row_len,
+                                                    Entry* __restrict__ rows) {
+  const int j = blockIdx.x * 8 + (threadIdx.x >> 5), bl = blockIdx.y, lane = threadIdx.x & 31;
+  if (j >= N) return;
+  const size_t lj = ((size_t)bl * N + j) * C;
+  const uint32_t mine = lane < C ? lens[lj + lane] : 0u;
+  const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, mine);
+  uint32_t at = 0u;
+  if (lane == 0 && total) at = atomicAdd(cursor + bl, total);
+  at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  size_t to = lj * NC;
+  if (at <= room && total <= room - at) to = join0 + (size_t)bl * room + at;
+  uint32_t* rl = row_len + (size_t)bl * N;
+  const uint32_t rr = (uint32_t)row_room(N);
+  Entry* rw = rows + (size_t)bl * N * rr;
+  int out = 0;
+  for (int r = 0; r < C; ++r) {
+    const int len = (int)__shfl_sync(0xFFFFFFFFu, mine, r);
+    const Entry* S = lists + (lj + r) * NC;
+    for (int i0 = 0; i0 < len; i0 += 32) {
+      const int n = min(32, len - i0);
+      Entry x = make_uint2(0u, 0u);
+      if (lane < n) x = S[i0 + lane];
+      __syncwarp();
+      if (lane < n) {
+        const uint32_t t = (x.x << lgC) | (uint32_t)r;
+        lists[to + out + lane] = make_uint2(t, x.y);
+        const uint32_t p = atomicAdd(rl + t, 1u);
+        if (p < rr) rw[(size_t)t * rr + p] = make_uint2((uint32_t)j, x.y);
+      }
+      out += n;
+    }
+  }
+  if (lane == 0) span[(size_t)bl * N + j] = make_uint2((uint32_t)to, (uint32_t)out);
+}
+
+// ---------------------------------------------------------------------------
+// Many picks a round.  Among a set S of candidates with exact gains the
+// greedy can run on S alone for as long as S's best gain stays above a bound
+// on every gain outside S: gains only fall, so nothing outside S can win
+// before that.  And a member of S whose gain is above those of all members
+// it shares a live target with will be picked with the gain it has: none of
+// them can come first.  So all such members are picked at once, their order
+// in the selection being that of their gains.  A round
+//  - takes the best candidates of 32 slices (t mod 32, so that neighbours in
+//    space fall into different ones), up to RD_TOP of each, and the largest
+//    gain left out as the bound;
+//  - brings their live targets (a few dozen entries each) into shared memory;
+//  - repeats: rank the members above the bound, find those that are first on
+//    all their live targets (a table of least ranks by target; targets that
+//    collide in it only hold a member back), pick them, lower m, update the
+//    members' gains;
+//  - puts its picks in the order of their gains, and updates the lists of all
+//    targets it lowered at once, as single picks would have done one after
+//    the other (terms add up without an order).
+// Where more members than picks to make are above the bound, only those
+// before the first one held back are picked, up to the number to make.
+// One block per scene, no waits on other blocks.  A round is a chain of a
+// few dozen barriers with a shared-memory or L2 latency or two between each
+// pair, so what counts is the number of rounds: 1229 picks of 8192 take 187
+// decisions, the single picks before them among these.
+//
+// A candidate whose row does not fit leaves S and raises the bound to its
+// gain; when that leaves no pick (or the best gains agree in their 24 bits
+// with one outside) the best candidate is picked alone, its row read in
+// pieces from the cost (or the slab).
+// ---------------------------------------------------------------------------
+constexpr int RD_WARPS = 32, RD_THREADS = 32 * RD_WARPS;
+constexpr int RD_EPT = 4;                        // row entries a thread holds at most
+constexpr int RD_EMAX = RD_EPT * RD_THREADS;     // ... and a round
+// Members a slice gives at most.  Selection, ms, at 2 / 4 / 8: N = 8192 3.51 /
+// 3.26 / 4.00, 4 local scenes of 6272 1.53 / 1.53 / 2.42: fewer picks a round
+// on one side, more rows to stage and rank on the other.
+constexpr int RD_TOP = 4;
+constexpr int RD_MEMBERS = RD_TOP * RD_WARPS;
+constexpr uint32_t NO_ENTRY = 0xFFFFFFFFu;
+constexpr uint32_t NO_RANK = 0x7FFFFFFFu;
+
+struct RoundArgs {
+  const float* rows;       // dense: cost [B][N][ldc]; local: slab [B][N][g]
+  const int32_t* nbr;      // local: [B][N][kk]
+  const float* v;          // [B][N]
+  const gain_t* gains0;    // [B][N] gains at the start (high word ~0: selected)
+  const float* m_in;       // dense: [scenes of the wave][N] coverage cost at the start
+  const int* start;        // dense: [scenes of the wave] first step to take
+  Entry* lists;
+  uint2* span;             // [scenes][N] (offset, length)
+  uint32_t* row_len;       // dense: [scenes of the wave][N]
+  Entry* row_ent;          // dense: [scenes of the wave][N][row_room(N)]
+  int32_t* order32;        // [B][K]
+  float* out_gains;        // [B][K] or null
+  double* objective;       // [B] or null
+  int* status;
+  int64_t ldc;
+  size_t list_step;        // local: entries between the lists of adjacent scenes
+  float m0;
+  int fx;
+  int N, K, g, kk;
+  int S;                   // candidates a slice, ceil(N / 32) made odd
+  int emax;                // row entries a round holds, at most RD_EMAX
+  int tmask;               // size of the table of least ranks - 1
+  int scene0;
+  uint32_t off_lo, off_hi, off_ent, off_em, off_qm, off_qj, off_bits, off_tab;  // dynamic shared memory
+};
+
+template <int W>
+struct Lanes {
+  static constexpr int value = W;
+};
+// Barrier of the first n warps.
+__device__ __forceinline__ void warps_sync(int n) {
+  asm volatile("bar.sync 1, %0;" ::"r"(32 * n) : "memory");
+}
+
+template <bool LOCAL>
+__global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_constant__ RoundArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float* sm_m = reinterpret_cast<float*>(smem);                    // [N] coverage cost
+  // gains as two words, slice after slice: candidate t at (t % 32) S + t / 32
+  // (S odd: candidates with adjacent indices, often on one list, fall into
+  // different banks)
+  uint32_t* g_lo = reinterpret_cast<uint32_t*>(smem + a.off_lo);   // [32 S]
+  uint32_t* g_hi = reinterpret_cast<uint32_t*>(smem + a.off_hi);   // [32 S]
+  Entry* ent = reinterpret_cast<Entry*>(smem + a.off_ent);         // [emax] (member << 16 | j, cost)
+  float* ent_m = reinterpret_cast<float*>(smem + a.off_em);        // [emax] their targets' m
+  float* q_m = reinterpret_cast<float*>(smem + a.off_qm);          // [emax] lowered targets: old m
+  uint16_t* q_j = reinterpret_cast<uint16_t*>(smem + a.off_qj);    // [emax] ... and index
+  uint32_t* bits = reinterpret_cast<uint32_t*>(smem + a.off_bits);  // [ceil(N / 32)] lowered this round
+  uint32_t* tab = reinterpret_cast<uint32_t*>(smem + a.off_tab);    // [tmask + 1] least rank by target
+  __shared__ int s_top[RD_TOP][RD_WARPS];    // a slice's best candidates
+  __shared__ int s_left[RD_WARPS];           // bound on a slice's other gains, high word (-1: none)
+  __shared__ uint32_t s_mlo[RD_MEMBERS], s_mhi[RD_MEMBERS];  // members' gains
+  __shared__ int s_mtok[RD_MEMBERS];         // members (-1: not in S, or picked)
+  __shared__ gain_t s_mkey[RD_MEMBERS];      // their keys (0: none, or not above the bound)
+  __shared__ int s_rank[RD_MEMBERS];
+  __shared__ uint32_t s_held[RD_MEMBERS];    // shares a live target with a better member
+  __shared__ int s_pick[RD_MEMBERS];
+  __shared__ gain_t s_pkey[RD_MEMBERS];      // the picks' keys
+  __shared__ gain_t s_best[RD_WARPS];
+  __shared__ gain_t s_tau;                   // one more than the largest gain outside S can be (0: none)
+  __shared__ int s_nm, s_ne, s_qn, s_np, s_cut, s_nv[2];
+
+  const int bl = blockIdx.x, b = a.scene0 + bl;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int N = a.N, fx = a.fx, S = a.S;
+  const float* v = a.v + (size_t)b * N;
+  const float* R = a.rows + (size_t)b * N * (LOCAL ? (size_t)a.g : (size_t)a.ldc);
+  const int32_t* NB = LOCAL ? a.nbr + (size_t)b * N * a.kk : nullptr;
+  uint2* span = a.span + (size_t)bl * N;
+  Entry* lists = LOCAL ? a.lists + (size_t)bl * a.list_step : a.lists;
+  unsigned long long my_ent = 0ull, my_row = 0ull, my_rounds = 0ull;
+
+  int step = LOCAL ? 0 : a.start[bl];
+  for (int j = threadIdx.x; j < N; j += RD_THREADS)
+    sm_m[j] = LOCAL ? a.m0 : a.m_in[(size_t)bl * N + j];
+  for (int p = threadIdx.x; p < 32 * S; p += RD_THREADS) {
+    const int t = ((p % S) << 5) | (p / S);
+    const gain_t x = t < N ? a.gains0[(size_t)b * N + t] : ~0ull;
+    g_lo[p] = (uint32_t)x;
+    g_hi[p] = (uint32_t)(x >> 32);
+  }
+  for (int i = threadIdx.x; i < (N + 31) / 32; i += RD_THREADS) bits[i] = 0u;
+  for (int i = threadIdx.x; i <= a.tmask; i += RD_THREADS) tab[i] = NO_RANK;
+  if (threadIdx.x == 0) s_np = 0;
+  __syncthreads();
+
+  while (step < a.K) {
+    ++my_rounds;
+#pragma unroll 1
+    for (int i = lane; i < s_np; i += 32) {  // the last round's picks are no candidates any more
+      const int t = s_pick[i];
+      if ((t & 31) == w) g_hi[w * S + (t >> 5)] = 0xFFFFFFFFu;
+    }
+    __syncwarp();
+    // ---- the slice's best candidates, by their gains' high words with the
+    // place in the lane's run in the low 5 bits (negative: selected, or
+    // none): each lane its three best, then the warp's best of those heads
+    // in turn; a lane whose three are used up bounds its rest by the third
+    int cnt = 0, left = -1;
+    {
+      int v1 = -1, v2 = -1, v3 = -1;
+#pragma unroll 4
+      for (int i = lane, q = 0; i < S; i += 32, ++q) {
+        const int x = (int)((g_hi[w * S + i] & 0xFFFFFFE0u) | (uint32_t)q);
+        v3 = max(v3, min(v2, x));
+        v2 = max(v2, min(v1, x));
+        v1 = max(v1, x);
+      }
+      const int third = v3;
+      bool real = true;  // the head is a candidate, not a bound
+#pragma unroll 1
+      for (; cnt < RD_TOP; ++cnt) {
+        const int best = __reduce_max_sync(0xFFFFFFFFu, v1);
+        const uint32_t who = __ballot_sync(0xFFFFFFFFu, v1 == best && real);
+        if (best < 0 || who == 0u) break;  // warp-uniform
+        if (lane == __ffs(who) - 1) {
+          s_top[cnt][w] = (((best & 31) * 32 + lane) << 5) | w;
+          v1 = v2;
+          v2 = v3;
+          v3 = -1;
+          if (v1 < 0) {
+            v1 = third;
+            real = false;
+          }
+        }
+      }
+      left = __reduce_max_sync(0xFFFFFFFFu, v1);
+      if (left >= 0) left |= 31;
+      if (lane == 0) s_left[w] = left;
+    }
+    if (threadIdx.x == 0) {
+      s_nm = 0;
+      s_ne = 0;
+      s_qn = 0;
+      s_nv[0] = s_nv[1] = 0;
+      s_tau = 0ull;
+    }
+    __syncthreads();  // every slice's bound is in
+    // ---- S: the slices' candidates above every high word left out
+    left = __reduce_max_sync(0xFFFFFFFFu, s_left[lane]);
+    if (threadIdx.x == 0) {
+      s_np = 0;
+      if (left >= 0) atomicMax(&s_tau, (gain_t)(left + 1) << 32);
+    }
+    if (cnt > 0) {
+      const int t = lane < cnt ? s_top[lane][w] : 0;
+      const uint32_t hi = lane < cnt ? g_hi[w * S + (t >> 5)] : 0u;
+      const uint32_t in = __ballot_sync(0xFFFFFFFFu, lane < cnt && (int)hi > left);
+      if (in) {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(&s_nm, __popc(in));
+        i = __shfl_sync(0xFFFFFFFFu, i, 0) + lane;
+        if ((in >> lane) & 1u) {  // in order, so lanes 0 .. popc - 1
+          s_mtok[i] = t;
+          s_mlo[i] = g_lo[w * S + (t >> 5)];
+          s_mhi[i] = hi;
+        }
+      }
+    }
+    __syncthreads();
+    // ---- the members' live targets (packed to the row's front on the dense
+    // path): rows of up to 64 entries are held in registers between the count
+    // and the write, longer ones are read twice
+    const int nm = s_nm, rr = row_room(N);
+#pragma unroll 1
+    for (int i = w; i < nm; i += RD_WARPS) {
+      const int t = s_mtok[i];
+      Entry* rw = LOCAL ? nullptr : a.row_ent + ((size_t)bl * N + t) * rr;
+      // entry q of the row of n, dead past it
+      auto fetch = [&](int q, int n) -> Entry {
+        Entry e = make_uint2(0u, 0x7F800000u);
+        if (q < n) {
+          if (LOCAL) {
+            e.x = q == 0 ? (uint32_t)t : (uint32_t)__ldg(NB + (size_t)t * a.kk + q - 1);
+            e.y = __float_as_uint(__ldg(R + (size_t)t * a.g + q));
+          } else {
+            e = __ldcg(rw + q);
+          }
+        }
+        return e;
+      };
+      Entry x[2];
+      x[0] = fetch(lane, LOCAL ? a.g : rr);
+      x[1] = fetch(32 + lane, LOCAL ? a.g : rr);
+      const int len = LOCAL ? a.g : (int)__ldcg(a.row_len + (size_t)bl * N + t);
+      const bool stored = LOCAL || len <= rr;  // a longer row is not kept
+      const uint32_t lt = (1u << lane) - 1u;
+      uint32_t mask[2];
+      float m[2];
+      int n = 0, n2;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int q = 32 * u + lane;
+        const bool in = stored && q < len;
+        m[u] = sm_m[in ? x[u].x : 0u];
+        mask[u] = __ballot_sync(0xFFFFFFFFu, in && __uint_as_float(x[u].y) < m[u]);
+        const int p = n + __popc(mask[u] & lt);
+        if (!LOCAL && ((mask[u] >> lane) & 1u) && p != q) __stcg(rw + p, x[u]);
+        n += __popc(mask[u]);
+      }
+      n2 = n;
+      if (stored)
+#pragma unroll 1
+        for (int k0 = 64; k0 < len; k0 += 64) {
+          Entry y[2];
+          y[0] = fetch(k0 + lane, len);
+          y[1] = fetch(k0 + 32 + lane, len);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int q = k0 + 32 * u + lane;
+            const bool live = __uint_as_float(y[u].y) < sm_m[y[u].x];
+            const uint32_t mk = __ballot_sync(0xFFFFFFFFu, live);
+            const int p = n2 + __popc(mk & lt);
+            if (!LOCAL && live && p != q) __stcg(rw + p, y[u]);
+            n2 += __popc(mk);
+          }
+        }
+      int at = 0;
+      if (lane == 0 && n2) at = atomicAdd(&s_ne, n2);
+      at = __shfl_sync(0xFFFFFFFFu, at, 0);
+      const bool fits = stored && at + n2 <= a.emax;
+      // the last places are filled even when the row does not fit
+      auto put = [&](const Entry& e, float mj, bool live, uint32_t mk) {
+        const int p = at + __popc(mk & lt);
+        if (live && p < a.emax) {
+          ent[p] = make_uint2(fits ? ((uint32_t)i << 16) | e.x : NO_ENTRY, e.y);
+          ent_m[p] = mj;
+        }
+        at += __popc(mk);
+      };
+#pragma unroll
+      for (int u = 0; u < 2; ++u) put(x[u], m[u], (mask[u] >> lane) & 1u, mask[u]);
+      if (n2 > n) {
+        __syncwarp();  // the packed row is visible to the whole warp
+        const int rn = LOCAL ? len : n2;
+#pragma unroll 1
+        for (int q = (LOCAL ? 64 : n) + lane; q - lane < rn; q += 32) {
+          const Entry e = fetch(q, rn);
+          const float mj = sm_m[e.x];
+          const bool live = __uint_as_float(e.y) < mj;
+          put(e, mj, live, __ballot_sync(0xFFFFFFFFu, live));
+        }
+      }
+      if (lane == 0) {
+        my_row += (unsigned long long)(stored ? len : 0);
+        if (!LOCAL && stored && n2 != len) __stcg(a.row_len + (size_t)bl * N + t, (uint32_t)n2);
+        if (!fits) {
+          s_mtok[i] = -1;
+          atomicMax(&s_tau, (((gain_t)s_mhi[i] << 32) | s_mlo[i]) + 1ull);
+        }
+      }
+    }
+    __syncthreads();
+    // ---- picks from S while its best stays above what is outside, by the
+    // first nw warps
+    const int ne = min(s_ne, a.emax);
+    const int nw = min(RD_WARPS, max(4, (ne + 31) / 32)), nt = 32 * nw;
+    if (w < nw) {
+      // a thread's entries
+      float ec[RD_EPT], em[RD_EPT];
+      uint32_t ej[RD_EPT];
+#pragma unroll
+      for (int u = 0; u < RD_EPT; ++u) {
+        const int e = threadIdx.x + u * nt;
+        const Entry x = e < ne ? ent[e] : make_uint2(NO_ENTRY, 0u);
+        const bool on = x.x != NO_ENTRY;
+        ej[u] = on ? x.x : 0u;
+        ec[u] = on ? __uint_as_float(x.y) : INFINITY;
+        em[u] = on ? ent_m[e] : -INFINITY;  // m never falls below that
+      }
+      // 24 bits of the largest gain outside S, + 1 (0: none)
+      const uint32_t out = s_tau ? gain_bits(s_tau - 1ull, fx) + 1u : 0u;
+      const int mi = threadIdx.x;  // a thread's member (nt >= RD_MEMBERS)
+      for (int it = 0;; ++it) {
+        // the members' keys, of those whose 24 bits are above the bound
+        if (mi < RD_MEMBERS) {
+          gain_t key = 0ull;
+          const int t = mi < nm ? s_mtok[mi] : -1;
+          if (t >= 0) {
+            const uint32_t f = gain_bits(((gain_t)s_mhi[mi] << 32) | s_mlo[mi], fx) + 1u;
+            if (f > out) key = gain_key(f - 1u, t);
+          }
+          s_mkey[mi] = key;
+          s_held[mi] = 0u;
+          const int n = __popc(__ballot_sync(0xFFFFFFFFu, key != 0ull));
+          if (lane == 0 && n) atomicAdd(&s_nv[it & 1], n);
+          if (mi == 0) {
+            s_cut = RD_MEMBERS;
+            s_nv[(it + 1) & 1] = 0;
+          }
+        }
+        warps_sync(nw);
+        const int nv = s_nv[it & 1], room = a.K - step - s_np;
+        if (nv == 0 || room == 0) break;  // the same in every warp
+        // their ranks, four lanes a member
+        for (int i0 = 0; i0 < nm; i0 += nt / 4) {
+          const int i = i0 + (int)(threadIdx.x >> 2);
+          const gain_t mine = i < nm ? s_mkey[i] : 0ull;
+          int r = 0;
+#pragma unroll 4
+          for (int o = lane & 3; o < nm; o += 4) r += s_mkey[o] > mine ? 1 : 0;
+          r += __shfl_xor_sync(0xFFFFFFFFu, r, 1);
+          r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
+          if ((lane & 3) == 0 && i < nm) s_rank[i] = mine ? r : (int)NO_RANK;
+        }
+        warps_sync(nw);
+        // the least rank on each target ...
+        int er[RD_EPT];
+#pragma unroll
+        for (int u = 0; u < RD_EPT; ++u) {
+          er[u] = (int)NO_RANK;
+          if (u * nt < ne && ec[u] < em[u]) er[u] = s_rank[ej[u] >> 16];
+          if (er[u] != (int)NO_RANK) atomicMin(tab + (ej[u] & (uint32_t)a.tmask), (uint32_t)er[u]);
+        }
+        warps_sync(nw);
+        // ... holds back the members that are not it
+#pragma unroll
+        for (int u = 0; u < RD_EPT; ++u) {
+          if (er[u] != (int)NO_RANK && tab[ej[u] & (uint32_t)a.tmask] < (uint32_t)er[u]) {
+            s_held[ej[u] >> 16] = 1u;
+            if (nv > room) atomicMin(&s_cut, er[u]);
+          }
+        }
+        warps_sync(nw);
+        // S <- S u {t*} (Eq. sgs_update) for the others: their live entries,
+        // one a target, lower m
+        const int lim = nv > room ? min(s_cut, room) : RD_MEMBERS;
+#pragma unroll
+        for (int u = 0; u < RD_EPT; ++u) {
+          if (er[u] != (int)NO_RANK) {
+            tab[ej[u] & (uint32_t)a.tmask] = NO_RANK;
+            if (er[u] < lim && s_held[ej[u] >> 16] == 0u) {
+              const int j = (int)(ej[u] & 0xFFFFu);
+              sm_m[j] = ec[u];
+              const uint32_t bit = 1u << (j & 31);
+              if (!(atomicOr(bits + (j >> 5), bit) & bit)) {
+                const int q = atomicAdd(&s_qn, 1);
+                q_j[q] = (uint16_t)j;
+                q_m[q] = em[u];
+              }
+            }
+          }
+        }
+        if (mi < nm && s_rank[mi] < lim && s_held[mi] == 0u) {
+          const int p = atomicAdd(&s_np, 1);
+          s_pick[p] = s_mtok[mi];
+          s_pkey[p] = s_mkey[mi];
+          s_mtok[mi] = -1;
+        }
+        warps_sync(nw);
+        // a lowered target takes off the members that still covered it
+#pragma unroll
+        for (int u = 0; u < RD_EPT; ++u) {
+          const float mj = u * nt < ne ? sm_m[ej[u] & 0xFFFFu] : INFINITY;
+          if (mj < em[u]) {
+            const uint32_t i = ej[u] >> 16;
+            uint32_t old;
+            const gain_t d = chunk_low(s_mlo, i, true, __ldg(v + (ej[u] & 0xFFFFu)), em[u],
+                                             mj, ec[u], fx, old);
+            chunk_high(s_mhi, i, d, old);
+            em[u] = mj;
+          }
+        }
+        warps_sync(nw);
+      }
+      // the picks in order, four lanes each
+      const int np = s_np;
+      for (int i0 = 0; i0 < np; i0 += nt / 4) {
+        const int i = i0 + (int)(threadIdx.x >> 2);
+        const gain_t mine = i < np ? s_pkey[i] : 0ull;
+        int r = 0;
+#pragma unroll 4
+        for (int o = lane & 3; o < np; o += 4) r += s_pkey[o] > mine ? 1 : 0;
+        r += __shfl_xor_sync(0xFFFFFFFFu, r, 1);
+        r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
+        if ((lane & 3) == 0 && i < np) {
+          a.order32[(size_t)b * a.K + step + r] = s_pick[i];
+          if (a.out_gains) a.out_gains[(size_t)b * a.K + step + r] = key_gain(mine);
+        }
+      }
+    }
+    __syncthreads();
+    const int np = s_np;
+    int pick = -1, len = 0;
+    if (np == 0) {
+      // ---- no pick from S: the best candidate alone, by its exact key
+      gain_t best = 0ull;
+#pragma unroll 1
+      for (int i = lane; i < S; i += 32) {
+        const uint32_t hi = g_hi[w * S + i];
+        if ((int)hi < 0) continue;
+        const gain_t key =
+            gain_key(gain_bits(((gain_t)hi << 32) | g_lo[w * S + i], fx), (i << 5) | w);
+        best = key > best ? key : best;
+      }
+      best = warp_max_key(best);
+      if (lane == 0) s_best[w] = best;
+      __syncthreads();
+      best = warp_max_key(s_best[lane]);
+      pick = best ? key_token(best) : -1;
+      if (pick < 0) {  // never expected: no candidate left (block-uniform)
+        if (threadIdx.x == 0 && atomicCAS(a.status, 0, CP_EDEVICE) == 0) {
+          a.status[4] = step;
+          a.status[5] = b;
+          a.status[6] = 0;
+          a.status[7] = pick;
+        }
+        return;
+      }
+      len = LOCAL ? a.g : N;
+      if (threadIdx.x == 0) {
+        a.order32[(size_t)b * a.K + step] = pick;
+        if (a.out_gains) a.out_gains[(size_t)b * a.K + step] = key_gain(best);
+        s_pick[0] = pick;
+        s_np = 1;
+        my_row += (unsigned long long)len;
+      }
+    }
+    // ---- the lists of the lowered targets; a lone pick's row in pieces
+    int k0 = 0;
+#pragma unroll 1
+    do {
+      if (pick >= 0) {
+        if (threadIdx.x == 0) s_qn = 0;
+        __syncthreads();
+#pragma unroll 1
+        for (int q = k0 + threadIdx.x; q < min(len, k0 + a.emax); q += RD_THREADS) {
+          const int j = LOCAL ? (q == 0 ? pick : __ldg(NB + (size_t)pick * a.kk + q - 1)) : q;
+          const float c = __ldg(R + (size_t)pick * (LOCAL ? (size_t)a.g : (size_t)a.ldc) + q);
+          const float mj = sm_m[j];
+          if (c < mj) {
+            const int at = atomicAdd(&s_qn, 1);
+            q_j[at] = (uint16_t)j;
+            q_m[at] = mj;
+            sm_m[j] = c;
+          }
+        }
+        __syncthreads();
+        k0 += a.emax;
+      }
+      // every live candidate of target q_j loses what the drop from q_m to m
+      // took; the entries that stay live are packed to the list's front.  A
+      // turn of this loop is a chain of latencies: 8 lanes take a list, 128
+      // lists a turn of the block, while lists are short (4 to 30 entries for
+      // most of a selection), 16 while they are long
+      const int qn = s_qn;
+      auto push = [&](auto width) {
+        constexpr int W = decltype(width)::value;   // lanes a list
+        constexpr int U = W == 16 ? 4 : 2;          // entries a lane has in flight
+        const int gl = lane & (W - 1), gs = lane & (32 - W);
+        constexpr uint32_t gm = (1u << W) - 1u;
+#pragma unroll 1
+        for (int q0 = (32 / W) * w; q0 < qn; q0 += RD_THREADS / W) {
+          const int q = q0 + lane / W;
+          const bool on = q < qn;
+          const int j = (int)q_j[on ? q : q0];
+          const uint2 sp = __ldcg(span + j);
+          const float vj = __ldg(v + j);
+          const float mo = q_m[on ? q : q0], mn = sm_m[j];
+          if (on && gl == 0) bits[j >> 5] = 0u;
+          Entry* L = lists + sp.x;
+          const int n = on ? (int)sp.y : 0;
+          int out = 0;
+#pragma unroll 1
+          for (int i0 = gl; __any_sync(0xFFFFFFFFu, i0 - gl < n); i0 += U * W) {
+            Entry x[U];
+            gain_t d[U];
+            uint32_t old[U], at[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+              x[u] = i0 + W * u < n ? __ldcg(L + i0 + W * u) : make_uint2(0u, 0x7F800000u);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              at[u] = (x[u].x & 31u) * (uint32_t)S + (x[u].x >> 5);
+              d[u] = chunk_low(g_lo, at[u], true, vj, mo, mn, __uint_as_float(x[u].y), fx,
+                                     old[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              chunk_high(g_hi, at[u], d[u], old[u]);
+              const bool stay = __uint_as_float(x[u].y) < mn;
+              const uint32_t mask = (__ballot_sync(0xFFFFFFFFu, stay) >> gs) & gm;
+              const int p = out + __popc(mask & ((1u << gl) - 1u));
+              if (stay && p != i0 + W * u) __stcg(L + p, x[u]);
+              out += __popc(mask);
+            }
+          }
+          if (gl == 0 && n) {
+            my_ent += (unsigned long long)n;
+            if (out != n) __stcg(&span[j].y, (uint32_t)out);
+          }
+        }
+      };
+      if (pick >= 0 || s_ne > 24 * s_nm)
+        push(Lanes<16>{});
+      else
+        push(Lanes<8>{});
+      __syncthreads();  // gains are settled
+    } while (k0 < len);
+    step += max(np, 1);
+  }
+
+  unsigned long long* cstats = reinterpret_cast<unsigned long long*>(
+      reinterpret_cast<unsigned char*>(a.status) + kCallStatsOffset);
+  if ((lane & 7) == 0) {
+    if (my_ent) atomicAdd(&cstats[0], my_ent);
+    atomicAdd(&cstats[2], 8ull * (my_ent + my_row));
+  }
+  if (threadIdx.x == 0) atomicAdd(&cstats[1], my_rounds);
+  if (a.objective) {
+    const double F = objective_sum(sm_m, v, N);
+    if (threadIdx.x == 0) a.objective[b] = F;
+  }
+}
+
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Scenes whose lists are held at once.  A dense scene's lists take 8 N^2
-// bytes at their largest (twice its cost), so a large batch runs in waves:
-// as many scenes as fit 24 GB less a twelfth of the whole cost, at least one.
+// bytes at their largest (twice its cost), its joined lists and rows up to
+// 16 RD_ROW N more, so a large batch runs in waves: as many scenes as fit 24
+// GB less a twelfth of the whole cost, at least one (entries are then
+// numbered in 32 bits).
 int64_t push_wave(int64_t B, int64_t N, int64_t ldc) {
-  const double per = 8.0 * (double)N * (double)(N + PUSH_CMAX);
+  const double per = 8.0 * (double)N * (double)(N + PUSH_CMAX + 2 * row_room(N));
   const double room = 24.0e9 - 4.0 * (double)B * (double)N * (double)ldc / 12.0;
   const int64_t w = room > per ? (int64_t)(room / per) : 1;
   return w < B ? w : B;
 }
 
 struct PushPlan {
-  size_t gains, first, max_bits, zero_bytes, sums, lens, lists, total;
+  size_t gains, first, max_bits, zero_bytes, sums, lens, span, lists, m, stop, row_len,
+      row_ent, total;
+  size_t join0;  // dense: entries before the joined lists
   int64_t wave;
 };
 PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t ldc) {
@@ -720,7 +1339,7 @@ PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t ldc) {
   p.gains = take(sizeof(gain_t) * BN);
   if (g < N) {
     p.wave = B;
-    p.lens = take(sizeof(uint2) * BN * PUSH_CMAX);
+    p.span = take(sizeof(uint2) * BN);
     p.lists = take(sizeof(Entry) * (BN * (size_t)g + LIST_PAD));
   } else {
     p.first = take(sizeof(gain_t) * (size_t)B);
@@ -728,9 +1347,15 @@ PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t ldc) {
     p.zero_bytes = off;
     p.sums = take(sizeof(float) * BN);
     p.wave = push_wave(B, N, ldc);
-    p.lens = take(sizeof(uint32_t) * (size_t)p.wave * (size_t)N * PUSH_CMAX);
-    p.lists =
-        take(sizeof(Entry) * ((size_t)p.wave * (size_t)N * (size_t)(N + PUSH_CMAX) + LIST_PAD));
+    const size_t WN = (size_t)p.wave * (size_t)N;
+    p.lens = take(sizeof(uint32_t) * WN * PUSH_CMAX);
+    p.join0 = WN * (size_t)(N + PUSH_CMAX);
+    p.lists = take(sizeof(Entry) * (p.join0 + WN * (size_t)row_room(N) + LIST_PAD));
+    p.span = take(sizeof(uint2) * WN);
+    p.m = take(sizeof(float) * WN);
+    p.stop = take(sizeof(int) * (size_t)p.wave);
+    p.row_len = take(sizeof(uint32_t) * (WN + (size_t)p.wave));  // and the joined lists' cursors
+    p.row_ent = take(sizeof(Entry) * (WN * (size_t)row_room(N) + LIST_PAD));
   }
   p.total = off;
   return p;
@@ -750,20 +1375,18 @@ size_t push_shape(PushArgs& a, int C, int64_t ncols) {
   const int per = (a.NC + PUSH_WARPS - 1) / PUSH_WARPS;
   a.lgS = lg2(per < 32 ? 32 : per);
   a.off_q = (uint32_t)(sizeof(float) * ncols);
-  a.off_lo = a.off_q + (uint32_t)(sizeof(uint32_t) * (size_t)(a.g < a.N ? a.g : a.N));
-  a.off_lo = (a.off_lo + 15u) & ~15u;
+  a.off_lo = a.off_q + (uint32_t)(sizeof(uint32_t) * (size_t)a.N);
   a.off_hi = a.off_lo + (uint32_t)(sizeof(uint32_t) * (size_t)a.NC);
   return a.off_hi + sizeof(uint32_t) * (size_t)a.NC;
 }
 
 // The largest cluster, C0 halved as often as needed, that the device can
 // hold; its launch configuration in cfg (attr must outlive it).
-template <bool LOCAL>
-int push_config(PushArgs& a, int C0, int64_t scenes, int64_t ncols, const DeviceInfo& di,
-                cudaStream_t s, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
-  auto fn = k_sgs_push<LOCAL>;
+template <typename Fn>
+int push_config(Fn fn, PushArgs& a, int C0, int64_t scenes, const DeviceInfo& di, cudaStream_t s,
+                cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   for (int C = C0; C >= 1; C >>= 1) {
-    const size_t smem = push_shape(a, C, ncols);
+    const size_t smem = push_shape(a, C, a.ldc);
     if (smem + 2048 > (size_t)di.max_smem_optin) continue;
     if (cuda_status(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem),
@@ -796,35 +1419,96 @@ int push_config(PushArgs& a, int C0, int64_t scenes, int64_t ncols, const Device
   return CP_EUNSUPPORTED;
 }
 
-}  // namespace
-
-// One size for every neighbourhood: a workspace of these sizes serves the
-// dense path and each local one.
-size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc) {
-  const size_t dense = push_plan(B, N, N, ldc).total;
-  const size_t local = g < N ? push_plan(B, N, g, ldc).total : 0;
-  return local > dense ? local : dense;
+// The rounds' launch: one block per scene, the row entries a round holds as
+// many as the shared memory beside m and the gains takes.
+template <typename Fn>
+int launch_rounds(Fn fn, RoundArgs& a, int64_t scenes, const DeviceInfo& di, cudaStream_t s) {
+  const int N = a.N;
+  a.S = ((N + 31) / 32) | 1;
+  a.off_lo = (uint32_t)((sizeof(float) * (size_t)N + 15) & ~(size_t)15);
+  a.off_hi = a.off_lo + 128u * (uint32_t)a.S;
+  a.off_ent = a.off_hi + 128u * (uint32_t)a.S;
+  size_t smem = 0;
+  const int tab = N > 12288 ? 2048 : 4096;
+  a.tmask = tab - 1;
+  for (a.emax = RD_EMAX;; a.emax >>= 1) {
+    a.off_em = a.off_ent + (uint32_t)(sizeof(Entry) * (size_t)a.emax);
+    a.off_qm = a.off_em + (uint32_t)(sizeof(float) * (size_t)a.emax);
+    a.off_qj = a.off_qm + (uint32_t)(sizeof(float) * (size_t)a.emax);
+    a.off_bits = a.off_qj + (uint32_t)(sizeof(uint16_t) * (size_t)a.emax);
+    a.off_tab = a.off_bits + (uint32_t)(sizeof(uint32_t) * (size_t)a.S);
+    smem = a.off_tab + sizeof(uint32_t) * (size_t)tab;
+    if (smem + 7168 <= (size_t)di.max_smem_optin) break;
+    if (a.emax <= 256) return CP_EUNSUPPORTED;
+  }
+  CP_TRY_STATUS(cuda_status(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem),
+                            "launch_sgs_push: rounds smem attribute"));
+  fn<<<(unsigned)scenes, RD_THREADS, smem, s>>>(a);
+  return launch_status("launch_sgs_push: rounds");
 }
 
-int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
-                    const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
-                    int32_t* order32, float* gains, double* objective, int* status,
-                    cudaStream_t s, const float* g0, void* ws) {
+int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
+                const float* v, const DevParams& P, int fx, int64_t B, int64_t N, int64_t K, int32_t* order32, float* gains, double* objective,
+                int* status, cudaStream_t s, const float* g0, void* ws) {
   DeviceInfo di;
   if (device_info(&di) != CP_OK) return CP_ECUDA;
   const bool local = P.g < N;
   const PushPlan pl = push_plan(B, N, P.g, ldc);
   unsigned char* base = static_cast<unsigned char*>(ws);
   gain_t* gains64 = reinterpret_cast<gain_t*>(base + pl.gains);
-  const int fx = gain_fx(P.m0);
+  RoundArgs r{};
+  r.rows = local ? slab : cost;
+  r.nbr = nbr;
+  r.v = v;
+  r.gains0 = gains64;
+  r.lists = reinterpret_cast<Entry*>(base + pl.lists);
+  r.span = reinterpret_cast<uint2*>(base + pl.span);
+  r.order32 = order32;
+  r.out_gains = gains;
+  r.objective = objective;
+  r.status = status;
+  r.ldc = ldc;
+  r.m0 = P.m0;
+  r.fx = fx;
+  r.N = (int)N;
+  r.K = (int)K;
+  r.g = P.g;
+  r.kk = P.kk;
+  if (local) {
+    const size_t rsmem = sizeof(int) * (size_t)N;
+    if (rsmem > 40 * 1024 &&
+        cuda_status(cudaFuncSetAttribute(k_rev_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)rsmem),
+                    "launch_sgs_push: reverse-list smem attribute") != CP_OK)
+      return CP_ECUDA;
+    k_rev_lists<<<(unsigned)B, 1024, rsmem, s>>>(nbr, slab, (int)N, P.g, P.kk, r.span,
+                                                 r.lists);
+    CP_TRY_STATUS(last_launch_status());
+    k_local_gains<<<dim3((unsigned)((N + 7) / 8), (unsigned)B), 256, 0, s>>>(
+        slab, nbr, v, (int)N, P.g, P.kk, P.m0, fx, gains64);
+    CP_TRY_STATUS(last_launch_status());
+    r.list_step = (size_t)N * (size_t)P.g;
+    return launch_rounds(k_sgs_rounds<true>, r, B, di, s);
+  }
+  gain_t* first = reinterpret_cast<gain_t*>(base + pl.first);
+  uint32_t* max_bits = reinterpret_cast<uint32_t*>(base + pl.max_bits);
+  float* sums = g0 ? reinterpret_cast<float*>(base + pl.sums) : nullptr;
+  r.row_len = reinterpret_cast<uint32_t*>(base + pl.row_len);
+  r.row_ent = reinterpret_cast<Entry*>(base + pl.row_ent);
+  r.m_in = reinterpret_cast<float*>(base + pl.m);
+  r.start = reinterpret_cast<int*>(base + pl.stop);
   PushArgs a{};
-  a.rows = local ? slab : cost;
-  a.nbr = nbr;
+  a.cost = cost;
   a.v = v;
-  a.gains0 = gains64;
+  a.gains = gains64;
+  a.first = first;
+  a.lists = r.lists;
+  a.lens = reinterpret_cast<uint32_t*>(base + pl.lens);
+  a.m_out = reinterpret_cast<float*>(base + pl.m);
+  a.stop = reinterpret_cast<int*>(base + pl.stop);
   a.order32 = order32;
   a.out_gains = gains;
-  a.objective = objective;
   a.status = status;
   a.ldc = ldc;
   a.timeout_ns = P.timeout_ns;
@@ -832,36 +1516,8 @@ int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int
   a.fx = fx;
   a.N = (int)N;
   a.K = (int)K;
-  a.g = P.g;
-  a.kk = P.kk;
-  a.lists = reinterpret_cast<Entry*>(base + pl.lists);
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  if (local) {
-    const int C0 = N > 12288 ? 2 : 1;
-    CP_TRY_STATUS(push_config<true>(a, C0, B, N, di, s, &cfg, attr));
-    a.span = reinterpret_cast<uint2*>(base + pl.lens);
-    const size_t rsmem = sizeof(int) * (size_t)N * (size_t)a.C;
-    if (rsmem > 40 * 1024 &&
-        cuda_status(cudaFuncSetAttribute(k_rev_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)rsmem),
-                    "launch_sgs_push: reverse-list smem attribute") != CP_OK)
-      return CP_ECUDA;
-    k_rev_lists<<<(unsigned)B, 1024, rsmem, s>>>(nbr, slab, (int)N, P.g, P.kk, a.C, a.lgC, a.span,
-                                                 a.lists);
-    CP_TRY_STATUS(last_launch_status());
-    k_local_gains<<<dim3((unsigned)((N + 7) / 8), (unsigned)B), 256, 0, s>>>(
-        slab, nbr, v, (int)N, P.g, P.kk, P.m0, fx, gains64);
-    CP_TRY_STATUS(last_launch_status());
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_sgs_push<true>, a);
-    note_launch();
-    return cuda_status(e, "launch_sgs_push: local");
-  }
-  gain_t* first = reinterpret_cast<gain_t*>(base + pl.first);
-  uint32_t* max_bits = reinterpret_cast<uint32_t*>(base + pl.max_bits);
-  float* sums = g0 ? reinterpret_cast<float*>(base + pl.sums) : nullptr;
-  a.first = first;
-  a.lens = reinterpret_cast<uint32_t*>(base + pl.lens);
   CP_TRY_STATUS(cuda_status(cudaMemsetAsync(base + pl.gains, 0, pl.zero_bytes, s),
                             "launch_sgs_push: gains"));
   if (g0) {
@@ -873,7 +1529,8 @@ int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int
   k_first_pick<<<dim3((unsigned)(groups < 512 ? groups : 512), (unsigned)B), 256, 0, s>>>(
       cost, ldc, v, (int)N, P.m0, fx, sums, max_bits, first);
   CP_TRY_STATUS(last_launch_status());
-  if (cuda_status(cudaFuncSetAttribute(k_live_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  auto lists_fn = k_live_lists;
+  if (cuda_status(cudaFuncSetAttribute(lists_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)LL_SMEM),
                   "launch_sgs_push: lists smem attribute") != CP_OK)
     return CP_ECUDA;
@@ -882,19 +1539,45 @@ int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int
     int C0 = PUSH_CMAX;
     while (C0 > 1 && ((int64_t)C0 * nb > di.sm_count || N / C0 < 256)) C0 >>= 1;
     if (C0 < 2 && N > 12288) C0 = 2;
-    CP_TRY_STATUS(push_config<false>(a, C0, nb, ldc, di, s, &cfg, attr));
+    auto push_fn = k_sgs_push;
+    CP_TRY_STATUS(push_config(push_fn, a, C0, nb, di, s, &cfg, attr));
     a.scene0 = (int)b0;
-    if (K > 1) {
-      k_live_lists<<<dim3((unsigned)((N + LL_COLS - 1) / LL_COLS), (unsigned)a.C, (unsigned)nb),
-                     32 * LL_WARPS, LL_SMEM, s>>>(cost, ldc, v, first, (int)N, a.C, a.lgC, a.NC,
-                                                  (int)b0, P.m0, fx, gains64, a.lists, a.lens);
-      CP_TRY_STATUS(last_launch_status());
-    }
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_sgs_push<false>, a);
+    lists_fn<<<dim3((unsigned)((N + LL_COLS - 1) / LL_COLS), (unsigned)a.C, (unsigned)nb),
+               32 * LL_WARPS, LL_SMEM, s>>>(cost, ldc, v, first, (int)N, a.C, a.lgC, a.NC,
+                                            (int)b0, P.m0, fx, gains64, a.lists, a.lens);
+    CP_TRY_STATUS(launch_status("launch_sgs_push: lists"));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, push_fn, a);
     note_launch();
-    CP_TRY_STATUS(cuda_status(e, "launch_sgs_push: dense"));
+    CP_TRY_STATUS(cuda_status(e, "launch_sgs_push: steps"));
+    uint32_t* cursor = r.row_len + (size_t)nb * (size_t)N;
+    CP_TRY_STATUS(cuda_status(
+        cudaMemsetAsync(r.row_len, 0, sizeof(uint32_t) * ((size_t)nb * (size_t)N + (size_t)nb), s),
+        "launch_sgs_push: rows"));
+    k_join_lists<<<dim3((unsigned)((N + 7) / 8), (unsigned)nb), 256, 0, s>>>(
+        a.lists, a.lens, (int)N, a.C, a.lgC, a.NC, pl.join0, (uint32_t)(N * row_room(N)), cursor, r.span,
+        r.row_len, r.row_ent);
+    CP_TRY_STATUS(last_launch_status());
+    r.scene0 = (int)b0;
+    CP_TRY_STATUS(launch_rounds(k_sgs_rounds<false>, r, nb, di, s));
   }
   return CP_OK;
+}
+
+}  // namespace
+
+// One size for every neighbourhood: a workspace of these sizes serves the
+// dense path and each local one.
+size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc) {
+  const size_t dense = push_plan(B, N, N, ldc).total;
+  const size_t local = g < N ? push_plan(B, N, g, ldc).total : 0;
+  return local > dense ? local : dense;
+}
+
+int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
+                    const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K, int32_t* order32, float* gains,
+                    double* objective, int* status, cudaStream_t s, const float* g0, void* ws) {
+  return launch_push(cost, ldc, slab, nbr, v, P, gain_fx(P.m0), B, N, K, order32, gains, objective,
+                     status, s, g0, ws);
 }
 
 }  // namespace cp
