@@ -570,7 +570,7 @@ int coverprune_select(const void* feats, int dtype, const float* pos, const int3
     if (slab && dtype != CP_BF16) CP_TRY(launch_slab(C, pl.ldc, nbr, d, B, N, slab, s));
     if (d.sgs_mode == 2)
       CP_TRY(launch_sgs_literal(C, pl.ldc, nbr, v, d, B, N, K, order32, gains, objective,
-                                at<void>(ws, pl.lit), s));
+                                at<void>(ws, pl.lit), status, s));
     else
       CP_TRY(launch_sgs(C, pl.ldc, slab, nbr, v, d, B, N, K, order32, gains, objective,
                         at<uint64_t>(ws, pl.partials), at<uint32_t>(ws, pl.counters), status, s,

@@ -185,7 +185,8 @@ int gain_fx(float m0);
 size_t sgs_literal_ws_bytes(int64_t B, int64_t N, int64_t K);
 int launch_sgs_literal(const float* cost, int64_t ldc, const int32_t* nbr, const float* v,
                        const DevParams& P, int64_t B, int64_t N, int64_t K, int32_t* order32,
-                       float* gains, double* objective, void* scratch, cudaStream_t s);
+                       float* gains, double* objective, void* scratch, int* status,
+                       cudaStream_t s);
 // Sort the B rows of K int32 indices ascending into int64 (and copy the
 // unsorted order out as int64 if order64 != NULL).
 int launch_sort_kept(const int32_t* idx32, int64_t B, int64_t K, int64_t* kept,

@@ -392,6 +392,35 @@ def test_sgs_literal_parity(orc, name, N, D, K, g):
           f"end to end equal for {first}/{K} steps, Jaccard {jac:.3f}")
 
 
+@pytest.mark.parametrize("N,D,K,g,eps,iters", [
+    (1, 64, 1, 0, 0.05, 20), (3, 64, 3, 0, 0.05, 20), (63, 64, 63, 0, 0.05, 20),
+    (129, 64, 65, 17, 0.05, 1), (130, 64, 33, 0, 0.2, 40),  # 2 blocks, the last not full
+    (1021, 64, 70, 24, 0.05, 20),                           # 16 blocks
+    (1030, 64, 40, 0, 0.02, 20), (517, 64, 50, 0, 1e-3, 20),  # C > 80 eps: on the potentials
+    (2500, 64, 250, 0, 0.05, 2)])                           # from 245 rows on: a launch a phase
+def test_sgs_literal_forms(orc, N, D, K, g, eps, iters):
+    """Every form of the iterations against the oracle along the GPU's own
+    picks.  A factor takes at most ~20 roundings of 2^-24 an iteration (a sum
+    in a tree, a division), a potential's exponent 2 x 3 / eps of them; a
+    score is off by at most that much of the score and of the score against
+    the full capacity, and so is a pick from the oracle's best."""
+    s = scene("long_video", 7, N=N, D=D)
+    prm = cp.Params(g=g, sgs_mode=2, sot_eps=eps, sot_iters=iters)
+    sel, cst = _select_case(orc, s, K, prm)
+    assert cp.coverprune_check(sel["ws"]) == cp.CP_OK
+    order, gains = host(sel["order"]), host(sel["gains"]).astype(np.float64)
+    assert len(set(order.tolist())) == K
+    C64 = host(cst["cost"]).astype(np.float64)
+    v64 = host(cst["capacity"]).astype(np.float64)
+    nbr = orc.knn_others(s["pos"], g - 1) if g else None
+    res = orc.sgs_literal(C64, v64, K, float(np.float32(eps)), iters, g, nbr, forced=order)
+    tol = iters * (20 + 6 / eps) * 2.0 ** -24
+    for l in range(K):
+        scale = res["picked_score"][l] + _full_capacity_score(C64, v64, int(order[l]), g, nbr)
+        assert abs(gains[l] - res["picked_score"][l]) <= tol * scale, l
+        assert res["picked_score"][l] - res["best_score"][l] <= 2 * tol * scale, l
+
+
 @pytest.mark.parametrize("name,N,D,K,g,seed", [("long_video", 2000, 512, 200, 64, 3),
                                                ("short_clip", 1500, 256, 150, 24, 4),
                                                ("long_video", 777, 128, 60, 17, 5)])
