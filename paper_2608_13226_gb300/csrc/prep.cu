@@ -436,12 +436,7 @@ int launch_knn(const float* pos, const float4* tok, int64_t B, int64_t N, int kk
 // as the brute-force kernels, but each query visits only the cells around
 // it.  The scene's bounding box is cut into cubic cells of side h =
 // (largest extent) / G with G = the least integer such that 4 G^3 >= N, so
-// at most G^3 cells; points are counting-sorted by cell.  A query scans the
-// shells of cells at Chebyshev distance r = 0, 1, 2, ... from its own cell;
-// every point outside the first r shells is more than r h away along some
-// axis, so once the kk-th best squared distance is below ((r - 1/1024) h)^2
-// (the margin covers the rounding of the cell coordinates) no later point
-// can enter the list.
+// at most G^3 cells; points are counting-sorted by cell.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int grid_side(int N) {
   int G = 1;
@@ -530,14 +525,246 @@ __global__ void __launch_bounds__(1024) k_grid_build(const float* __restrict__ p
   }
 }
 
-// One thread per query token.  The KK best keys are kept unsorted with the
+// One warp per query token, queries in cell order.  Three scans of candidate
+// ranges (a range is the cells of one (y, z) row, contiguous in the sorted
+// points; the ranges of 32 rows are scanned as one flat sequence):
+//  - the smallest block of cells around the query with more than kk points,
+//    at least 3 x 3 x 3: a histogram of the squared distances, 8 bins an
+//    octave, gives a bound U that at least kk of them are below;
+//  - every cell within sqrt(U) (rows and ends of rows by their distance, with
+//    a margin for the rounding of the cell coordinates): the keys below U are
+//    gathered, kk and usually a few more;
+//  - should more than KW_CAP be (coincident points, say), histograms over the
+//    range of those keys lower U until they fit.
+// The gathered keys are ranked by counting; the first kk go out in order.
+// Keys are (d^2 bits, index), as in the brute-force kernels.  Bound by
+// instruction issue (a point costs ~40 instructions a scan, of the warp), no
+// longer by the chain of one thread's scan and list: 56,000 queries (8 scenes
+// of 7000), kk = 63: 0.17 ms, a heap per thread took 0.62; 262,144 queries:
+// 0.82 (1.66); one scene of 8192, kk = 8: 0.024 (0.087), of 16384 0.076
+// (0.37).
+constexpr int KW_WARPS = 8, KW_CAP = 256;
+
+__global__ void __launch_bounds__(32 * KW_WARPS) k_knn_grid(
+    int N, int kk, int gmax, const GridInfo* __restrict__ info,
+    const int32_t* __restrict__ cell_start, const float4* __restrict__ sorted,
+    int32_t* __restrict__ nbr) {
+  __shared__ __align__(16) unsigned long long s_buf[KW_WARPS][KW_CAP];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, b = blockIdx.y;
+  const int jj = blockIdx.x * KW_WARPS + w;
+  if (jj >= N) return;
+  unsigned long long* buf = s_buf[w];
+  uint32_t* hist = reinterpret_cast<uint32_t*>(buf);  // [256]
+  const GridInfo g = info[b];
+  const int32_t* cs = cell_start + (size_t)b * (gmax + 1);
+  const float4* P = sorted + (size_t)b * N;
+  const float4 qp = P[jj];
+  const int self = __float_as_int(qp.w);
+  const int cx = grid_coord(g, qp.x, 0), cy = grid_coord(g, qp.y, 1), cz = grid_coord(g, qp.z, 2);
+  float span = 0.0f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) span = fmaxf(span, fabsf(g.lo[a]) + (float)g.dims[a] * g.h);
+  const float delta = 1e-3f * g.h + 1e-5f * span;
+
+  // The window of the next scan: rows [y0, y1] x [z0, z1], cells [x0, x1] of
+  // them; rad2 < infinity: only cells within that distance.
+  int x0, x1, y0, y1, z0, z1;
+  float rad2;
+  auto block = [&](int r) {
+    x0 = max(cx - r, 0);
+    x1 = min(cx + r, g.dims[0] - 1);
+    y0 = max(cy - r, 0);
+    y1 = min(cy + r, g.dims[1] - 1);
+    z0 = max(cz - r, 0);
+    z1 = min(cz + r, g.dims[2] - 1);
+    rad2 = INFINITY;
+  };
+  // distance from the query to the cells of coordinate c along one axis
+  auto gap = [&](int a, float q, int cq, int c) -> float {
+    const float edge = g.lo[a] + (float)(c < cq ? c + 1 : c) * g.h;
+    return c == cq ? 0.0f : fmaxf((c < cq ? q - edge : edge - q) - delta, 0.0f);
+  };
+  // Row q of the window: its first point and number of points.
+  auto row = [&](int q, int rows, int ny, int& start) -> int {
+    start = 0;
+    if (q >= rows) return 0;
+    const int z = z0 + q / ny, y = y0 + q % ny;
+    int xa = x0, xb = x1;
+    if (rad2 < INFINITY) {
+      const float gy = gap(1, qp.y, cy, y), gz = gap(2, qp.z, cz, z);
+      const float left = rad2 - (gy * gy + gz * gz);
+      if (left < 0.0f) return 0;
+      const float half = sqrtf(left) + delta;
+      xa = max(xa, grid_coord(g, qp.x - half, 0));
+      xb = min(xb, grid_coord(g, qp.x + half, 0));
+    }
+    const int base = (z * g.dims[1] + y) * g.dims[0];
+    start = cs[base + xa];
+    return cs[base + xb + 1] - start;
+  };
+  // visit(in, key) with the whole warp for every 32 points of the window
+  auto scan = [&](auto&& visit) {
+    const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
+    for (int q0 = 0; q0 < rows; q0 += 32) {
+      int start;
+      const int len = row(q0 + lane, rows, ny, start);
+      int incl = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const int total = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - len;
+      for (int c0 = 0; c0 < total; c0 += 32) {
+        const int c = min(c0 + lane, total - 1);
+        int r = 0;  // the row of the c-th point: the last that starts at or before c
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if (__shfl_sync(0xFFFFFFFFu, excl, r + o) <= c) r += o;
+        const float4 p =
+            P[__shfl_sync(0xFFFFFFFFu, start, r) + c - __shfl_sync(0xFFFFFFFFu, excl, r)];
+        const int k = __float_as_int(p.w);
+        const uint32_t bits = __float_as_uint(sqdist_rn(qp.x, qp.y, qp.z, p.x, p.y, p.z));
+        visit(c0 + lane < total && k != self, ((unsigned long long)bits << 32) | (uint32_t)k);
+      }
+    }
+  };
+  // the bin of hist in which the count reaches `want`, and the count before it
+  auto bin_of = [&](int want, int& before) -> int {
+    __syncwarp();
+    const uint4 h0 = reinterpret_cast<const uint4*>(hist)[2 * lane];
+    const uint4 h1 = reinterpret_cast<const uint4*>(hist)[2 * lane + 1];
+    const uint32_t h[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+    uint32_t sum = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum += h[i];
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const int first = __ffs(__ballot_sync(0xFFFFFFFFu, incl >= (uint32_t)want)) - 1;
+    int bin = 0;
+    uint32_t run = incl - sum, below = run;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      run += h[i];
+      if (run < (uint32_t)want) {
+        bin = i + 1;
+        below = run;
+      }
+    }
+    before = (int)__shfl_sync(0xFFFFFFFFu, below, first);
+    return 8 * first + __shfl_sync(0xFFFFFFFFu, bin, first);
+  };
+  auto clear = [&]() {
+    reinterpret_cast<uint4*>(hist)[2 * lane] = make_uint4(0u, 0u, 0u, 0u);
+    reinterpret_cast<uint4*>(hist)[2 * lane + 1] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+  };
+
+  // ---- a block with more than kk points (the query among them)
+  for (int r = 1;; ++r) {
+    block(r);
+    const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
+    int n = 0;
+    for (int q = lane; q < rows; q += 32) {
+      int start;
+      n += row(q, rows, ny, start);
+    }
+    n = __reduce_add_sync(0xFFFFFFFFu, n);
+    if (n > kk) break;  // N > kk: the whole grid at the latest
+  }
+  const float far = 64.0f * g.h;
+  const int off = (int)(__float_as_uint(far * far) >> 20) - 255;
+  clear();
+  scan([&](bool in, unsigned long long key) {
+    const int bin = min(max((int)(key >> 52) - off, 0), 255);
+    if (in) atomicAdd(hist + bin, 1u);
+  });
+  int below;
+  const int top = bin_of(kk, below);
+  // at least kk keys are below U
+  unsigned long long U = top == 255 ? ~0ull : (unsigned long long)(top + 1 + off) << 52;
+  // ---- the keys below U; `sure` of the kk are below L
+  unsigned long long L = 0ull;
+  int n = 0, sure = 0;
+  for (;;) {
+    const float d2 = __uint_as_float((uint32_t)(U >> 32));
+    if (d2 < 1e30f) {
+      const float rad = sqrtf(d2) * 1.000244140625f + delta;  // 1 + 2^-12
+      x0 = 0;
+      x1 = g.dims[0] - 1;
+      y0 = grid_coord(g, qp.y - rad, 1);
+      y1 = grid_coord(g, qp.y + rad, 1);
+      z0 = grid_coord(g, qp.z - rad, 2);
+      z1 = grid_coord(g, qp.z + rad, 2);
+      rad2 = rad * rad;
+    } else {  // infinite or not a number: everywhere
+      block(max(g.dims[0], max(g.dims[1], g.dims[2])));
+    }
+    n = 0;
+    unsigned long long lo = ~0ull, hi = 0ull;
+    scan([&](bool in, unsigned long long key) {
+      in = in && key < U;
+      const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
+      if (in) {
+        const int at = n + __popc(mask & ((1u << lane) - 1u));
+        if (at < KW_CAP) buf[at] = key;
+        if (key >= L) {
+          lo = key < lo ? key : lo;
+          hi = key > hi ? key : hi;
+        }
+      }
+      n += __popc(mask);
+    });
+    if (n <= KW_CAP) break;
+    // too many: a histogram of those from L on over their range [lo, hi];
+    // the bin with the kk-th is at most a 128th of it, down to a single key
+    lo = __shfl_sync(0xFFFFFFFFu, warp_min_u64(lo), 0);
+    hi = __shfl_sync(0xFFFFFFFFu, warp_max_u64(hi), 0);
+    const int shift = max(0, 56 - __clzll((long long)((hi - lo) | 1ull)));
+    __syncwarp();
+    clear();
+    scan([&](bool in, unsigned long long key) {
+      if (in && key >= lo && key <= hi) atomicAdd(hist + (int)((key - lo) >> shift), 1u);
+    });
+    const int bin = bin_of(kk - sure, below);
+    sure += below;
+    L = lo + ((unsigned long long)bin << shift);
+    U = L + (1ull << shift);
+  }
+  __syncwarp();
+  // ---- ranks
+  int32_t* out = nbr + ((size_t)b * N + self) * kk;
+  for (int i0 = 0; i0 < n; i0 += 64) {
+    const unsigned long long ka = i0 + lane < n ? buf[i0 + lane] : ~0ull;
+    const unsigned long long kb = i0 + 32 + lane < n ? buf[i0 + 32 + lane] : ~0ull;
+    int ra = 0, rb = 0;
+#pragma unroll 4
+    for (int t = 0; t < n; ++t) {
+      const unsigned long long o = buf[t];
+      ra += o < ka ? 1 : 0;
+      rb += o < kb ? 1 : 0;
+    }
+    if (i0 + lane < n && ra < kk) out[ra] = (int32_t)(uint32_t)ka;
+    if (i0 + 32 + lane < n && rb < kk) out[rb] = (int32_t)(uint32_t)kb;
+  }
+}
+
+// Few neighbours of very many queries (kk <= 8): one thread per query token
+// scans the shells of cells at Chebyshev distance r = 0, 1, 2, ... from its
+// own cell; every point outside the first r shells is more than r h away
+// along some axis, so once the kk-th best squared distance is below ((r -
+// 1/1024) h)^2 (the margin covers the rounding of the cell coordinates) no
+// later point can enter the list.  The KK best keys are kept unsorted with the
 // position of the worst: a closer point overwrites the worst (a select per
 // slot, so the list stays in registers) and the worst is found again; the
 // list is sorted once at the end.  Keys are (d^2 bits, index), as in the
 // brute-force kernels.
 template <int KK>
-__global__ void __launch_bounds__(128) k_knn_grid(const float* __restrict__ pos, int N, int kk,
-                                                  int gmax, const GridInfo* __restrict__ info,
+__global__ void __launch_bounds__(128) k_knn_grid_thread(int N, int kk, int gmax, const GridInfo* __restrict__ info,
                                                   const int32_t* __restrict__ cell_start,
                                                   const float4* __restrict__ sorted,
                                                   int32_t* __restrict__ nbr) {
@@ -613,109 +840,6 @@ __global__ void __launch_bounds__(128) k_knn_grid(const float* __restrict__ pos,
 #pragma unroll
   for (int i = 0; i < KK; ++i)
     if (i >= KK - kk) out[i - (KK - kk)] = (int32_t)(best[i] & 0xFFFFFFFFull);
-}
-
-// More neighbours (8 < kk <= kKnnGridMax): the same shell search, one thread
-// per query (queries in cell order), with the kk best keys in a max-heap in
-// shared memory (slot i of thread t at [i][t]: the threads of a warp touch
-// distinct banks); the root is the worst kept key.  A heapsort leaves them
-// ascending at the end.
-__global__ void __launch_bounds__(128) k_knn_grid_heap(const float* __restrict__ pos, int N, int kk,
-                                                       int gmax, const GridInfo* __restrict__ info,
-                                                       const int32_t* __restrict__ cell_start,
-                                                       const float4* __restrict__ sorted,
-                                                       int32_t* __restrict__ nbr) {
-  extern __shared__ unsigned long long s_heap[];  // [kk][blockDim.x]
-  const int jj = blockIdx.x * blockDim.x + threadIdx.x;  // the jj-th token in cell order
-  const int b = blockIdx.y;
-  if (jj >= N) return;
-  const int T = blockDim.x;
-  unsigned long long* H = s_heap + threadIdx.x;  // H[i * T] is slot i
-  const GridInfo g = info[b];
-  const int32_t* cs = cell_start + (size_t)b * (gmax + 1);
-  const float4* P = sorted + (size_t)b * N;
-  const float4 qp = P[jj];
-  const int j = __float_as_int(qp.w);
-  const float qx = qp.x, qy = qp.y, qz = qp.z;
-  const int cx = grid_coord(g, qx, 0), cy = grid_coord(g, qy, 1), cz = grid_coord(g, qz, 2);
-  int cnt = 0;
-  unsigned long long worst = ~0ull;  // the root once the heap is full
-  // the root replaced by key (smaller than it), sifted down within n slots
-  auto sift_down = [&](unsigned long long key, int n) {
-    int i = 0;
-    for (;;) {
-      const int l = 2 * i + 1;
-      if (l >= n) break;
-      const int r = l + 1;
-      unsigned long long ck = H[(size_t)l * T];
-      int c = l;
-      if (r < n) {
-        const unsigned long long rk = H[(size_t)r * T];
-        if (rk > ck) {
-          ck = rk;
-          c = r;
-        }
-      }
-      if (ck <= key) break;
-      H[(size_t)i * T] = ck;
-      i = c;
-    }
-    H[(size_t)i * T] = key;
-  };
-  const int rmax = max(g.dims[0], max(g.dims[1], g.dims[2]));
-  for (int r = 0; r <= rmax; ++r) {
-    for (int dz = -r; dz <= r; ++dz) {
-      const int z = cz + dz;
-      if (z < 0 || z >= g.dims[2]) continue;
-      for (int dy = -r; dy <= r; ++dy) {
-        const int y = cy + dy;
-        if (y < 0 || y >= g.dims[1]) continue;
-        const bool face = dz == -r || dz == r || dy == -r || dy == r;
-        for (int dx = -r; dx <= r; dx += (face || r == 0) ? 1 : 2 * r) {
-          const int x = cx + dx;
-          if (x < 0 || x >= g.dims[0]) continue;
-          const int c = (z * g.dims[1] + y) * g.dims[0] + x;
-          const int e = cs[c + 1];
-          for (int s = cs[c]; s < e; ++s) {
-            const float4 p = P[s];
-            const int k = __float_as_int(p.w);
-            const uint32_t bits = __float_as_uint(sqdist_rn(qx, qy, qz, p.x, p.y, p.z));
-            if (k == j || bits > (uint32_t)(worst >> 32)) continue;
-            const unsigned long long key = ((unsigned long long)bits << 32) | (uint32_t)k;
-            if (key >= worst) continue;
-            if (cnt < kk) {  // filling: sift the new key up
-              int i = cnt++;
-              while (i > 0) {
-                const int pi = (i - 1) >> 1;
-                const unsigned long long pk = H[(size_t)pi * T];
-                if (pk >= key) break;
-                H[(size_t)i * T] = pk;
-                i = pi;
-              }
-              H[(size_t)i * T] = key;
-              if (cnt == kk) worst = H[0];
-            } else {
-              sift_down(key, kk);
-              worst = H[0];
-            }
-          }
-        }
-      }
-    }
-    if (cnt == kk) {  // the heap is full: is anything closer still possible?
-      const float reach = ((float)r - 1.0f / 1024.0f) * g.h;
-      if (reach > 0.0f && __uint_as_float((uint32_t)(worst >> 32)) < reach * reach) break;
-    }
-  }
-  // heapsort: the largest to the end, repeatedly
-  for (int n = kk; n > 1; --n) {
-    const unsigned long long top = H[0];
-    const unsigned long long last = H[(size_t)(n - 1) * T];
-    H[(size_t)(n - 1) * T] = top;
-    sift_down(last, n - 1);
-  }
-  int32_t* out = nbr + ((size_t)b * N + j) * kk;
-  for (int i = 0; i < kk; ++i) out[i] = (int32_t)(H[(size_t)i * T] & 0xFFFFFFFFull);
 }
 
 // The largest pinned-fp32 squared distance over pairs, into stats.d2_max_bits,
@@ -902,20 +1026,18 @@ int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr
                                                                           stats);
   CP_TRY_STATUS(last_launch_status());
   if (kk <= 0) return CP_OK;
-  if (kk <= 8) {
-    dim3 grid((unsigned)((N + 127) / 128), (unsigned)B);
-    k_knn_grid<8><<<grid, 128, 0, s>>>(pos, (int)N, kk, gmax, info, cell_start, sorted, nbr);
+  // A thread a query needs fewer instructions, but only many queries hide its
+  // latency.  kk = 8, us, thread / warp (with k_grid_build and
+  // k_diameter_grid), scenes of 8192: 8 300 / 224, 12 346 / 283, 16 349 / 338,
+  // 20 356 / 400, 32 584 / 579; 32 of 4096 268 / 308, 128 of 1024 184 / 250,
+  // 8 of 16384 525 / 494; 32 long videos 300 / 491 for the search alone.
+  if (kk <= 8 && B * N >= 131072) {
+    k_knn_grid_thread<8><<<dim3((unsigned)((N + 127) / 128), (unsigned)B), 128, 0, s>>>(
+        (int)N, kk, gmax, info, cell_start, sorted, nbr);
     return last_launch_status();
   }
-  const int T = kk <= 64 ? 128 : 64;  // heaps of T x kk keys: at most 64 KB
-  const size_t hsmem = sizeof(unsigned long long) * (size_t)T * (size_t)kk;
-  if (hsmem > 48 * 1024 &&
-      cuda_status(cudaFuncSetAttribute(k_knn_grid_heap, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)hsmem),
-                  "launch_knn_grid: heap smem attribute") != CP_OK)
-    return CP_ECUDA;
-  dim3 grid((unsigned)((N + T - 1) / T), (unsigned)B);
-  k_knn_grid_heap<<<grid, T, hsmem, s>>>(pos, (int)N, kk, gmax, info, cell_start, sorted, nbr);
+  const dim3 grid((unsigned)((N + KW_WARPS - 1) / KW_WARPS), (unsigned)B);
+  k_knn_grid<<<grid, 32 * KW_WARPS, 0, s>>>((int)N, kk, gmax, info, cell_start, sorted, nbr);
   return last_launch_status();
 }
 

@@ -56,6 +56,36 @@ def test_knn_ties_and_duplicates(orc):
     np.testing.assert_array_equal(host(nbr), orc.knn_others(X, 11))
 
 
+@pytest.mark.parametrize("k", [1, 8, 9, 32, 33, 127, 128])
+def test_knn_grid_forms(k):
+    """The grid search against the brute-force kernels, bit for bit: lone far
+    points (blocks of many cells), more coincident points than the buffer of
+    gathered keys holds (with kk of them, with fewer), infinite and undefined
+    coordinates."""
+    rng = np.random.default_rng(k)
+    X = (rng.random((1, 1100, 3)) * 4).astype(np.float32)
+    X[0, 3] = 90.0
+    X[0, 100:420] = X[0, 7]
+    X[0, 500:510] = X[0, 8]
+    Y = X.copy()
+    Y[0, 5] = np.nan
+    Y[0, 6, 1] = np.inf
+    for P in (X, Y, X[:, :k + 1], X[:, 100:400], X[:, 95:395]):
+        pos = torch.from_numpy(np.ascontiguousarray(P)).cuda()
+        nbr, _ = cp.coverprune_knn(pos, k)
+        bf = torch.empty(1, P.shape[1], k, dtype=torch.int32, device="cuda")
+        cp.coverprune_knn_noalloc(pos, bf, torch.empty(1, dtype=torch.float32, device="cuda"))
+        assert torch.equal(nbr.view_as(bf), bf)
+
+
+def test_knn_very_many_queries():
+    """131,072 queries or more take a thread each, fewer a warp each."""
+    pos = torch.rand(33, 8192, 3, device="cuda") * 5
+    nbr, _ = cp.coverprune_knn(pos, 8)
+    one, _ = cp.coverprune_knn(pos[:2].contiguous(), 8)
+    assert torch.equal(nbr[:2], one)
+
+
 def _max_d2_fp32(X):
     """The largest squared distance over all pairs, every operation rounded
     in fp32 in the kernels' order ((dx dx + dy dy) + dz dz)."""
