@@ -17,12 +17,23 @@ __global__ void __launch_bounds__(512) k_scene_stats(const float* __restrict__ p
   const int32_t* T = frame ? frame + (size_t)b * N : nullptr;  // may be absent
   int tmin = INT32_MAX, tmax = INT32_MIN;
   float lo[3] = {INFINITY, INFINITY, INFINITY};
-  for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    const int t = T ? T[j] : 0;
-    tmin = min(tmin, t);
-    tmax = max(tmax, t);
+  for (int j0 = threadIdx.x; j0 < N; j0 += 4 * 512) {  // four tokens' loads in flight
+    int t[4];
+    float x[4][3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) lo[a] = fminf(lo[a], X[3 * j + a]);
+    for (int u = 0; u < 4; ++u) {
+      const int j = min(j0 + 512 * u, N - 1);
+      t[u] = T ? T[j] : 0;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[u][a] = X[3 * j + a];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      tmin = min(tmin, t[u]);
+      tmax = max(tmax, t[u]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) lo[a] = fminf(lo[a], x[u][a]);
+    }
   }
   __shared__ int s_tmin[16], s_tmax[16];
   __shared__ float s_lo[3][16];
@@ -444,7 +455,10 @@ __device__ __forceinline__ int grid_side(int N) {
   return G;
 }
 
-// One block per scene: bounding box, cell size, counting sort by cell.
+// One block per scene: bounding box, cell size, counting sort by cell.  Bound
+// by latency: three passes over the points, four points' loads in flight a
+// thread, and a scan of the cell counts by all threads (one thread's scan
+// was half of the time): 16384 points 21 us, 34 before; 1024 points 8 us.
 __global__ void __launch_bounds__(1024) k_grid_build(const float* __restrict__ pos, int N,
                                                      int gmax, GridInfo* __restrict__ info,
                                                      int32_t* __restrict__ cell_start,
@@ -454,12 +468,22 @@ __global__ void __launch_bounds__(1024) k_grid_build(const float* __restrict__ p
   const int b = blockIdx.x;
   const float* X = pos + (size_t)b * N * 3;
   float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  for (int j = threadIdx.x; j < N; j += blockDim.x)
+  for (int j0 = threadIdx.x; j0 < N; j0 += 4 * 1024) {
+    float x[4][3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      lo[a] = fminf(lo[a], X[3 * j + a]);
-      hi[a] = fmaxf(hi[a], X[3 * j + a]);
+    for (int u = 0; u < 4; ++u) {
+      const int j = min(j0 + 1024 * u, N - 1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[u][a] = X[3 * j + a];
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        lo[a] = fminf(lo[a], x[u][a]);
+        hi[a] = fmaxf(hi[a], x[u][a]);
+      }
+  }
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -503,25 +527,62 @@ __global__ void __launch_bounds__(1024) k_grid_build(const float* __restrict__ p
   }
   __syncthreads();
   const GridInfo g = s_g;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) atomicAdd(&s_cnt[grid_cell(g, X + 3 * j)], 1);
+  for (int j0 = threadIdx.x; j0 < N; j0 += 4 * 1024) {
+    float x[4][3];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = min(j0 + 1024 * u, N - 1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[u][a] = X[3 * j + a];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + 1024 * u < N) atomicAdd(&s_cnt[grid_cell(g, x[u])], 1);
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {  // exclusive scan; cells <= G^3 <= 13824
-    int run = 0;
-    for (int c = 0; c < g.ncells; ++c) {
+  // exclusive scan of the counts, a run of cells a thread
+  __shared__ int s_sum[32];
+  {
+    const int per = (g.ncells + 1023) >> 10;
+    const int c0 = min(g.ncells, (int)threadIdx.x * per), c1 = min(g.ncells, c0 + per);
+    int sum = 0;
+    for (int c = c0; c < c1; ++c) sum += s_cnt[c];
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (l >= o) incl += t;
+    }
+    if (l == 31) s_sum[w] = incl;
+    __syncthreads();
+    int run = __reduce_add_sync(0xFFFFFFFFu, l < w ? s_sum[l] : 0) + incl - sum;
+    for (int c = c0; c < c1; ++c) {
       const int n = s_cnt[c];
       s_cnt[c] = run;
       run += n;
     }
-    s_cnt[g.ncells] = run;
+    if (threadIdx.x == 0) s_cnt[g.ncells] = N;
   }
   __syncthreads();
   int32_t* cs = cell_start + (size_t)b * (gmax + 1);
   for (int c = threadIdx.x; c <= g.ncells; c += blockDim.x) cs[c] = s_cnt[c];
   __syncthreads();
   float4* out = sorted + (size_t)b * N;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    const int slot = atomicAdd(&s_cnt[grid_cell(g, X + 3 * j)], 1);
-    out[slot] = make_float4(X[3 * j], X[3 * j + 1], X[3 * j + 2], __int_as_float(j));
+  for (int j0 = threadIdx.x; j0 < N; j0 += 4 * 1024) {
+    float x[4][3];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = min(j0 + 1024 * u, N - 1);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[u][a] = X[3 * j + a];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + 1024 * u;
+      if (j < N)
+        out[atomicAdd(&s_cnt[grid_cell(g, x[u])], 1)] =
+            make_float4(x[u][0], x[u][1], x[u][2], __int_as_float(j));
+    }
   }
 }
 
@@ -844,159 +905,210 @@ __global__ void __launch_bounds__(128) k_knn_grid_thread(int N, int kk, int gmax
 
 // The largest pinned-fp32 squared distance over pairs, into stats.d2_max_bits,
 // from the neighbour grid (points sorted by cell).  A lower bound L is the
-// largest d^2 among the extreme points of 13 directions (an actual pair).
-// For two cells whose coordinates differ by (dx, dy, dz) cells, any two of
-// their points are at most (|d| + 1) h + delta apart along each axis (delta
-// covers the rounding of the cell assignment), so the pair of cells can hold
-// a pair above L only if sum ((|d| + 1) h + delta)^2, inflated for fp32
-// rounding, reaches L.  Cells that reach L with no cell of the grid's corners
-// are dropped; the pairs of the remaining cells that pass the test are
-// evaluated with the same arithmetic as every other kernel, so the result is
-// exactly the largest d^2.  Blocks (part, scene); part p takes every P-th
-// row of candidate-cell pairs.
-constexpr int DIA_THREADS = 512, DIA_PARTS = 4, DIA_DIRS = 13;
+// largest d^2 among the extreme points of 7 directions (the axes and the
+// space diagonals; an actual pair).  For two cells whose coordinates differ
+// by (dx, dy, dz) cells, any two of their points are at most (|d| + 1) h +
+// delta apart along each axis (delta covers the rounding of the cell
+// assignment), so the pair of cells can hold a pair above L only if
+// sum ((|d| + 1) h + delta)^2, inflated for fp32 rounding, reaches L.  Cells
+// that reach L with no cell of the grid's corners are dropped; the pairs of
+// the remaining cells that pass the test are evaluated with the same
+// arithmetic as every other kernel, so the result is exactly the largest d^2.
+//
+// A cluster of 8 blocks per scene: each finds the extremes of its eighth of
+// the points (the work is nearly all there; few dozen pairs of cells pass the
+// test), then takes the pairs whose lower cell c has c mod 8 = its rank, a
+// warp per cell; pairs of large cells are left to the whole block.  16384
+// points: 167 us before (13 directions over all points in each of 4 blocks,
+// a thread per pair of cells), 24 now; 32 scenes of 8192 88 and 38.
+constexpr int DIA_THREADS = 512, DIA_PARTS = 8, DIA_DIRS = 7, DIA_BIG = 64;
 
 __device__ __forceinline__ uint32_t warp_max_u32(uint32_t v) {
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  return v;
+  return __reduce_max_sync(0xFFFFFFFFu, v);
 }
 
-__device__ __forceinline__ float dia_dir_dot(int d, float x, float y, float z) {
-  switch (d) {
-    case 0: return x;
-    case 1: return y;
-    case 2: return z;
-    case 3: return x + y;
-    case 4: return x - y;
-    case 5: return x + z;
-    case 6: return x - z;
-    case 7: return y + z;
-    case 8: return y - z;
-    case 9: return x + y + z;
-    case 10: return x + y - z;
-    case 11: return x - y + z;
-    default: return -x + y + z;
-  }
-}
-
-__global__ void __launch_bounds__(DIA_THREADS) k_diameter_grid(
+__global__ void __cluster_dims__(DIA_PARTS, 1, 1) __launch_bounds__(DIA_THREADS) k_diameter_grid(
     int N, int gmax, const GridInfo* __restrict__ info, const int32_t* __restrict__ cell_start,
     const float4* __restrict__ sorted, SceneStats* stats) {
   extern __shared__ int s_cand[];  // candidate cells, [gmax]
-  __shared__ unsigned long long s_ext[2 * DIA_DIRS];
-  __shared__ int s_ncand, s_wcnt[DIA_THREADS / 32];
-  __shared__ uint32_t s_m[DIA_THREADS / 32];
-  const int b = blockIdx.y;
+  __shared__ unsigned long long s_ext[2 * DIA_DIRS];   // this block's extremes: (key, point)
+  __shared__ uint32_t s_pt[2 * DIA_DIRS];              // the scene's
+  __shared__ int4 s_big[DIA_BIG];
+  __shared__ int s_ncand, s_nbig;
+  __shared__ uint32_t s_m;
+  const int b = blockIdx.y, part = (int)cluster_ctarank();
   const GridInfo g = info[b];
   const int32_t* cs = cell_start + (size_t)b * (gmax + 1);
   const float4* P = sorted + (size_t)b * N;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  constexpr int NW = DIA_THREADS / 32;
   if (threadIdx.x < 2 * DIA_DIRS) s_ext[threadIdx.x] = 0ull;
-  if (threadIdx.x == 0) s_ncand = 0;
-  __syncthreads();
-
-  // extreme points of 13 directions (max of +u and of -u), as (key, slot)
-  for (int d = 0; d < DIA_DIRS; ++d) {
-    unsigned long long hi = 0ull, lo = 0ull;
-    for (int i = threadIdx.x; i < N; i += DIA_THREADS) {
-      const float4 p = P[i];
-      const float v = dia_dir_dot(d, p.x, p.y, p.z);
-      const unsigned long long kh = ((unsigned long long)f2key(v) << 32) | (uint32_t)i;
-      const unsigned long long kl = ((unsigned long long)f2key(-v) << 32) | (uint32_t)i;
-      hi = kh > hi ? kh : hi;
-      lo = kl > lo ? kl : lo;
-    }
-    hi = warp_max_u64(hi);
-    lo = warp_max_u64(lo);
-    if (lane == 0) {
-      atomicMax(&s_ext[2 * d], hi);
-      atomicMax(&s_ext[2 * d + 1], lo);
-    }
+  if (threadIdx.x == 0) {
+    s_ncand = 0;
+    s_nbig = 0;
+    s_m = 0u;
   }
   __syncthreads();
+
   uint32_t m = 0u;  // the largest d^2 bits this thread has seen
-  for (int e = threadIdx.x; e < 2 * DIA_DIRS * 2 * DIA_DIRS; e += DIA_THREADS) {
-    const int u = e / (2 * DIA_DIRS), v = e % (2 * DIA_DIRS);
-    const float4 a = P[(uint32_t)(s_ext[u] & 0xFFFFFFFFull)];
-    const float4 c = P[(uint32_t)(s_ext[v] & 0xFFFFFFFFull)];
+  {
+    float hi[DIA_DIRS], lo[DIA_DIRS];
+    int ih[DIA_DIRS], il[DIA_DIRS];
+#pragma unroll
+    for (int d = 0; d < DIA_DIRS; ++d) {
+      hi[d] = -INFINITY;
+      lo[d] = INFINITY;
+      ih[d] = il[d] = 0;
+    }
+#pragma unroll 2
+    for (int i = part * DIA_THREADS + threadIdx.x; i < N; i += DIA_PARTS * DIA_THREADS) {
+      const float4 p = P[i];
+      const float v[DIA_DIRS] = {p.x, p.y, p.z, p.x + p.y + p.z, p.x + p.y - p.z,
+                                 p.x - p.y + p.z, -p.x + p.y + p.z};
+      if (!(v[3] == v[3])) m = 0x7FFFFFFFu;  // an undefined point: so is the diameter
+#pragma unroll
+      for (int d = 0; d < DIA_DIRS; ++d) {
+        if (v[d] > hi[d]) {
+          hi[d] = v[d];
+          ih[d] = i;
+        }
+        if (v[d] < lo[d]) {
+          lo[d] = v[d];
+          il[d] = i;
+        }
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < DIA_DIRS; ++d) {
+      const uint32_t kh = f2key(hi[d]), kl = f2key(-lo[d]);
+      const uint32_t mh = warp_max_u32(kh), ml = warp_max_u32(kl);
+      const int sh = __ffs(__ballot_sync(0xFFFFFFFFu, kh == mh)) - 1;
+      const int sl = __ffs(__ballot_sync(0xFFFFFFFFu, kl == ml)) - 1;
+      if (lane == sh) atomicMax(&s_ext[2 * d], ((unsigned long long)mh << 32) | (uint32_t)ih[d]);
+      if (lane == sl) atomicMax(&s_ext[2 * d + 1], ((unsigned long long)ml << 32) | (uint32_t)il[d]);
+    }
+  }
+  hw_cluster_sync();  // every block's extremes are complete
+  if (threadIdx.x < 2 * DIA_DIRS) {
+    unsigned long long x[DIA_PARTS];
+#pragma unroll
+    for (int r = 0; r < DIA_PARTS; ++r)
+      asm volatile("ld.shared::cluster.u64 %0, [%1];"
+                   : "=l"(x[r])
+                   : "r"(map_rank(smem_addr(&s_ext[threadIdx.x]), (uint32_t)r))
+                   : "memory");
+    unsigned long long m = x[0];
+#pragma unroll
+    for (int r = 1; r < DIA_PARTS; ++r) m = x[r] > m ? x[r] : m;
+    s_pt[threadIdx.x] = (uint32_t)m;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4 * DIA_DIRS * DIA_DIRS) {
+    const float4 a = P[s_pt[threadIdx.x / (2 * DIA_DIRS)]];
+    const float4 c = P[s_pt[threadIdx.x % (2 * DIA_DIRS)]];
     m = max(m, __float_as_uint(sqdist_rn(a.x, a.y, a.z, c.x, c.y, c.z)));
   }
   m = warp_max_u32(m);
-  if (lane == 0) s_m[w] = m;
+  if (lane == 0) atomicMax(&s_m, m);
   __syncthreads();
-  uint32_t Lb = s_m[0];
-  for (int i = 1; i < DIA_THREADS / 32; ++i) Lb = max(Lb, s_m[i]);
-  const float L = __uint_as_float(Lb);
+  const float L = __uint_as_float(s_m);
 
   // bound of two cells' d^2 from their coordinate differences
   float span = 0.0f;
   for (int a = 0; a < 3; ++a) span = fmaxf(span, fabsf(g.lo[a]) + (float)g.dims[a] * g.h);
   const float delta = 1e-3f * g.h + 1e-5f * span;
-  auto bound = [&](int ax, int ay, int az, int bx, int by, int bz) -> float {
-    const float ex = (float)(abs(ax - bx) + 1) * g.h + delta;
-    const float ey = (float)(abs(ay - by) + 1) * g.h + delta;
-    const float ez = (float)(abs(az - bz) + 1) * g.h + delta;
+  auto bound = [&](int dx, int dy, int dz) -> float {
+    const float ex = (float)(dx + 1) * g.h + delta;
+    const float ey = (float)(dy + 1) * g.h + delta;
+    const float ez = (float)(dz + 1) * g.h + delta;
     return (ex * ex + ey * ey + ez * ez) * 1.000244140625f;  // 1 + 2^-12
   };
-  // the candidate cells in ascending order (every block of the scene lists
-  // them alike, so the parts split the pairs without gaps or overlaps)
+  // the candidate cells, in any order
   const int d0 = g.dims[0], d1 = g.dims[1], d2 = g.dims[2];
   for (int base = 0; base < g.ncells; base += DIA_THREADS) {
     const int c = base + threadIdx.x;
     bool cand = false;
     if (c < g.ncells && cs[c + 1] > cs[c]) {
       const int cx = c % d0, cy = (c / d0) % d1, cz = c / (d0 * d1);
-      float far = 0.0f;
-      for (int k = 0; k < 8; ++k)
-        far = fmaxf(far, bound(cx, cy, cz, (k & 1) ? d0 - 1 : 0, (k & 2) ? d1 - 1 : 0,
-                               (k & 4) ? d2 - 1 : 0));
-      cand = far >= L;
+      cand = bound(max(cx, d0 - 1 - cx), max(cy, d1 - 1 - cy), max(cz, d2 - 1 - cz)) >= L;
     }
     const uint32_t bal = __ballot_sync(0xFFFFFFFFu, cand);
-    if (lane == 0) s_wcnt[w] = __popc(bal);
-    __syncthreads();
-    int off = s_ncand;
-    for (int i = 0; i < w; ++i) off += s_wcnt[i];
-    if (cand) s_cand[off + __popc(bal & ((1u << lane) - 1u))] = c;
-    __syncthreads();  // every thread has read s_ncand and s_wcnt
-    if (threadIdx.x == 0) {
-      int tot = 0;
-      for (int i = 0; i < DIA_THREADS / 32; ++i) tot += s_wcnt[i];
-      s_ncand += tot;
+    if (bal) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&s_ncand, __popc(bal));
+      at = __shfl_sync(0xFFFFFFFFu, at, 0);
+      if (cand) s_cand[at + __popc(bal & ((1u << lane) - 1u))] = c;
     }
-    __syncthreads();
   }
+  __syncthreads();
   const int M = s_ncand;
 
-  // rows of candidate-cell pairs: warp (part, w) takes rows r = part + P*w, ...
-  const int nw = DIA_THREADS / 32;
-  for (int r = blockIdx.x + DIA_PARTS * w; r < M; r += DIA_PARTS * nw) {
+  auto pair_max = [&](const float4& p, const float4& q) {
+    m = max(m, __float_as_uint(sqdist_rn(p.x, p.y, p.z, q.x, q.y, q.z)));
+  };
+  // pairs of candidate cells A <= B
+  for (int r = w; r < M; r += NW) {
     const int A = s_cand[r];
+    if (A % DIA_PARTS != part) continue;
     const int ax = A % d0, ay = (A / d0) % d1, az = A / (d0 * d1);
-    const int a0 = cs[A], a1 = cs[A + 1];
-    for (int t = r + lane; t < M; t += 32) {
-      const int Bc = s_cand[t];
-      const int bx = Bc % d0, by = (Bc / d0) % d1, bz = Bc / (d0 * d1);
-      if (bound(ax, ay, az, bx, by, bz) < L) continue;
-      const int b0 = cs[Bc], b1 = cs[Bc + 1];
-      for (int i = a0; i < a1; ++i) {
-        const float4 p = P[i];
-        for (int j = b0; j < b1; ++j) {
-          const float4 q = P[j];
-          m = max(m, __float_as_uint(sqdist_rn(p.x, p.y, p.z, q.x, q.y, q.z)));
+    const int a0 = cs[A], na = cs[A + 1] - a0;
+    for (int t0 = 0; t0 < M; t0 += 32) {
+      const int t = t0 + lane;
+      int b0 = 0, nb = 0;
+      if (t < M) {
+        const int B = s_cand[t];
+        const int bx = B % d0, by = (B / d0) % d1, bz = B / (d0 * d1);
+        if (B >= A && bound(abs(ax - bx), abs(ay - by), abs(az - bz)) >= L) {
+          b0 = cs[B];
+          nb = cs[B + 1] - b0;
+        }
+      }
+      uint32_t todo = __ballot_sync(0xFFFFFFFFu, nb > 0);
+      while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int q0 = __shfl_sync(0xFFFFFFFFu, b0, src), nq = __shfl_sync(0xFFFFFFFFu, nb, src);
+        if ((int64_t)na * nq > 4096) {  // for the whole block, while there is room
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&s_nbig, 1);
+          at = __shfl_sync(0xFFFFFFFFu, at, 0);
+          if (at < DIA_BIG) {
+            if (lane == 0) s_big[at] = make_int4(a0, na, q0, nq);
+            continue;
+          }
+        }
+        if (nq >= 16) {
+          for (int i = 0; i < na; ++i) {
+            const float4 p = P[a0 + i];
+            for (int j = lane; j < nq; j += 32) pair_max(p, P[q0 + j]);
+          }
+        } else {  // a lane a point of A
+          for (int i = lane; i < na; i += 32) {
+            const float4 p = P[a0 + i];
+            for (int j = 0; j < nq; ++j) pair_max(p, P[q0 + j]);
+          }
         }
       }
     }
   }
-  m = warp_max_u32(m);
-  __syncthreads();  // every warp has read s_m above
-  if (lane == 0) s_m[w] = m;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t mm = s_m[0];
-    for (int i = 1; i < nw; ++i) mm = max(mm, s_m[i]);
-    atomicMax(&stats[b].d2_max_bits, mm);
+  for (int k = 0; k < min(s_nbig, DIA_BIG); ++k) {
+    const int4 e = s_big[k];
+    for (int i = 4 * w; i < e.y; i += 4 * NW) {  // four points of A a warp
+      float4 p[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) p[u] = P[e.x + min(i + u, e.y - 1)];
+#pragma unroll 2
+      for (int j = lane; j < e.w; j += 32) {
+        const float4 q = P[e.z + j];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) pair_max(p[u], q);
+      }
+    }
   }
+  m = warp_max_u32(m);
+  if (lane == 0) atomicMax(&stats[b].d2_max_bits, m);
+  hw_cluster_sync();  // nobody leaves while a peer may still read its extremes
 }
 
 int grid_cells_max(int64_t N) {
