@@ -121,15 +121,27 @@ __global__ void __launch_bounds__(256) k_capacity_r_cos(
 }
 
 // v_j = r_j / sum_l r_l (phi = identity), uniform when the sum is 0 or the
-// uniform-capacity ablation is on.  One block per scene; the sum is taken in
-// fp64 in a fixed order.
+// uniform-capacity ablation is on.  The sum is taken in fp64 in a fixed order
+// (thread r adds j = r, r + 1024, ...).  Bound by the few fp64 units of an SM,
+// a division taking ~15 of their operations: every block adds up the whole
+// scene and divides `chunk` tokens of it.  One scene of 8192 / 16384 tokens
+// 10 / 15 us; one block dividing all of them took 34 / 64.  32 scenes of 8192
+// 26 (34).
 __global__ void __launch_bounds__(1024) k_capacity_v(const float* __restrict__ r_all, int N,
-                                                     int mode, float* __restrict__ v_all,
+                                                     int mode, int chunk,
+                                                     float* __restrict__ v_all,
                                                      float* __restrict__ v_out) {
-  const int b = blockIdx.x;
+  const int b = blockIdx.y;
   const float* r = r_all + (size_t)b * N;
   double part = 0.0;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) part += (double)r[j];
+  for (int j0 = threadIdx.x; j0 < N; j0 += 4 * 1024) {
+    float x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = j0 + 1024 * u < N ? r[j0 + 1024 * u] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + 1024 * u < N) part += (double)x[u];
+  }
   part = warp_sum(part);
   __shared__ double s_part[32];
   __shared__ double s_total;
@@ -143,7 +155,8 @@ __global__ void __launch_bounds__(1024) k_capacity_v(const float* __restrict__ r
   __syncthreads();
   const double total = s_total;
   const bool uniform = mode == 1 || !(total > 0.0);
-  for (int j = threadIdx.x; j < N; j += blockDim.x) {
+  const int end = min(N, (int)(blockIdx.x + 1) * chunk);
+  for (int j = blockIdx.x * chunk + threadIdx.x; j < end; j += blockDim.x) {
     const float vj = uniform ? (float)(1.0 / (double)N) : (float)((double)r[j] / total);
     v_all[(size_t)b * N + j] = vj;
     if (v_out) v_out[(size_t)b * N + j] = vj;
@@ -169,7 +182,13 @@ int launch_capacity(const void* feats, int dtype, const float* inv, const float*
                                                         nbr, P, (int)N, (int)D, r);
   int st = last_launch_status();
   if (st != CP_OK) return st;
-  k_capacity_v<<<(unsigned)B, 1024, 0, s>>>(r, (int)N, P.cap_mode, v, v_out);
+  // chunks of 128 tokens while few scenes leave SMs idle, up to 1024
+  DeviceInfo di;
+  if (device_info(&di) != CP_OK) return CP_ECUDA;
+  int chunk = 128;
+  while (chunk < 1024 && B * ((N + chunk - 1) / chunk) > 2 * di.sm_count) chunk <<= 1;
+  k_capacity_v<<<dim3((unsigned)((N + chunk - 1) / chunk), (unsigned)B), 1024, 0, s>>>(
+      r, (int)N, P.cap_mode, chunk, v, v_out);
   return last_launch_status();
 }
 
