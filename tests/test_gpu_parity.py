@@ -674,6 +674,22 @@ def test_capacity_from_features(orc, n_cap, N, D, seed):
     np.testing.assert_array_equal(host(lt["group_start"]), b)
 
 
+@pytest.mark.parametrize("voxel", [100.0, 0.2, 0.004])  # codes of 0, ~18 and 30 bits
+@pytest.mark.parametrize("N", [1, 31, 33, 257, 1025, 6272, 16384])
+def test_morton_order(orc, N, voxel):
+    """The group starts depend on the whole order: equal to the oracle's, for
+    every number of passes and at the edges of the warps' runs of tokens."""
+    s = scene("long_video", 11, N=N, D=64)
+    s["pos"][: N // 3] = s["pos"][N // 3]  # equal codes
+    prm = cp.Params(voxel_m=voxel, norm_mode=1)
+    K = (N + 2) // 3
+    f, pos, fr = to_dev(s)
+    lt = cp.coverprune_lite_select(f, pos, fr, K, prm)
+    vg = host(cp.coverprune_cost(f, pos, fr, prm, cost=False)["capacity"])
+    b, _ = orc.lite_groups(vg, orc.morton(s["pos"], prm.voxel_m)[1], K)
+    np.testing.assert_array_equal(host(lt["group_start"]), b)
+
+
 @pytest.mark.parametrize("name,N,D,K", [("tiny", 1024, 256, 102), ("long_video", 1500, 512, 150),
                                         ("short_clip", 333, 256, 100)])
 def test_lite_parity(orc, name, N, D, K):
