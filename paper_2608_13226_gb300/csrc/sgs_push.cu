@@ -16,7 +16,7 @@
 // N^2); a whole selection of a long-video scene (N = 8192, K = 1229) then
 // touches 21 M entries, and steps past 410 change ~8 targets and ~150
 // entries.  On the local path the live candidates of j start as the t with j
-// in M_g(t) (k_rev_lists).
+// in M_g(t) (k_rev_fill).
 //
 // The work is little; what bounds it is chains of dependent latencies --
 // argmax, the winner's row, the lowered targets' lists, the gain updates --
@@ -264,74 +264,76 @@ __global__ void __launch_bounds__(32 * LL_WARPS) k_live_lists(
 
 // ---------------------------------------------------------------------------
 // The local path's lists: the candidates t with j in M_g(t) and their costs.
-// One block per scene: counts, an exclusive scan and a fill, with counts and
-// cursors in shared memory [N] (0.67 ms of 32 scenes, N = 8192, g = 64).  span[b N + j] = (offset into the scene's
-// entries, length); the order within a list is arbitrary (no result depends
-// on it).
+// Counts (a warp a candidate), an exclusive scan (a block a scene) and the
+// fill, which also sums the candidates' first gains (m = m0).  span[b N + j] =
+// (offset into the scene's entries, length); the order within a list is
+// arbitrary (no result depends on it).  Bound by L2 atomics: 4 scenes of
+// 6272, g = 64, 63 us (one block a scene doing all of it: 489), 32 of 8192
+// 419 (728).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_rev_lists(const int32_t* __restrict__ nbr_all,
-                                                    const float* __restrict__ slab, int N, int g,
-                                                    int kk, uint2* __restrict__ span_all,
-                                                    Entry* __restrict__ ent_all) {
-  extern __shared__ int s_c[];  // [N]
-  __shared__ int s_sum[1024];
-  const int b = blockIdx.x;
-  const int32_t* NB = nbr_all + (size_t)b * N * kk;
-  const float* S = slab + (size_t)b * N * g;
-  uint2* span = span_all + (size_t)b * N;
-  Entry* ent = ent_all + (size_t)b * N * g;
-  const int64_t ng = (int64_t)N * g;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) s_c[j] = 0;
-  __syncthreads();
-  for (int64_t i = threadIdx.x; i < ng; i += blockDim.x) {
-    const int t = (int)(i / g), k = (int)(i % g);
-    atomicAdd(&s_c[k == 0 ? t : NB[(size_t)t * kk + (k - 1)]], 1);
-  }
-  __syncthreads();
-  // exclusive prefix of the counts: each thread a contiguous chunk, then a
-  // scan of the 1024 chunk sums
-  const int chunk = (N + blockDim.x - 1) / blockDim.x;
-  const int c0 = min(N, (int)threadIdx.x * chunk), c1 = min(N, c0 + chunk);
-  int part = 0;
-  for (int j = c0; j < c1; ++j) part += s_c[j];
-  s_sum[threadIdx.x] = part;
-  __syncthreads();
-  for (int d = 1; d < (int)blockDim.x; d <<= 1) {
-    const int x = threadIdx.x >= (unsigned)d ? s_sum[threadIdx.x - d] : 0;
+__global__ void __launch_bounds__(256) k_rev_count(const int32_t* __restrict__ nbr, int N, int g,
+                                                   int kk, uint2* __restrict__ span) {
+  const int t = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y, lane = threadIdx.x & 31;
+  if (t >= N) return;
+  const int32_t* nb = nbr + ((size_t)b * N + t) * kk;
+  for (int k = lane; k < g; k += 32)
+    atomicAdd(&span[(size_t)b * N + (k == 0 ? t : __ldg(nb + k - 1))].y, 1u);
+}
+
+__global__ void __launch_bounds__(1024) k_rev_scan(int N, uint2* __restrict__ span_all) {
+  __shared__ uint32_t s_w[32];
+  uint2* span = span_all + (size_t)blockIdx.x * N;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t carry = 0u;
+  for (int j0 = 0; j0 < N; j0 += 4096) {  // four a thread
+    const int j = j0 + 4 * (int)threadIdx.x;
+    uint32_t n[4], sum = 0u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      n[u] = j + u < N ? span[j + u].y : 0u;
+      sum += n[u];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    __syncthreads();  // the last turn's sums are read
+    if (lane == 31) s_w[w] = incl;
     __syncthreads();
-    s_sum[threadIdx.x] += x;
-    __syncthreads();
-  }
-  int run = s_sum[threadIdx.x] - part;  // the exclusive prefix of this chunk
-  for (int j = c0; j < c1; ++j) {
-    const int n = s_c[j];
-    span[j] = make_uint2((uint32_t)run, (uint32_t)n);
-    s_c[j] = run;  // from here on: the next free slot
-    run += n;
-  }
-  __syncthreads();
-  for (int64_t i = threadIdx.x; i < ng; i += blockDim.x) {
-    const int t = (int)(i / g), k = (int)(i % g);
-    const int j = k == 0 ? t : NB[(size_t)t * kk + (k - 1)];
-    ent[atomicAdd(&s_c[j], 1)] = make_uint2((uint32_t)t, __float_as_uint(S[i]));
+    const uint32_t x = s_w[lane];
+    uint32_t run = carry + __reduce_add_sync(0xFFFFFFFFu, lane < w ? x : 0u) + incl - sum;
+    carry += __reduce_add_sync(0xFFFFFFFFu, x);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (j + u < N) span[j + u] = make_uint2(run, 0u);  // the fill counts again
+      run += n[u];
+    }
   }
 }
 
-// The local path's first gains (m = m0), one warp per candidate.
-__global__ void __launch_bounds__(256) k_local_gains(const float* __restrict__ slab,
-                                                     const int32_t* __restrict__ nbr,
-                                                     const float* __restrict__ v_all,
-                                                     int N, int g, int kk, float m0, int fx,
-                                                     gain_t* __restrict__ gains) {
+__global__ void __launch_bounds__(256) k_rev_fill(const float* __restrict__ slab,
+                                                  const int32_t* __restrict__ nbr,
+                                                  const float* __restrict__ v_all, int N, int g,
+                                                  int kk, float m0, int fx,
+                                                  uint2* __restrict__ span_all,
+                                                  Entry* __restrict__ ent_all,
+                                                  gain_t* __restrict__ gains) {
   const int t = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y, lane = threadIdx.x & 31;
   if (t >= N) return;
   const float* v = v_all + (size_t)b * N;
   const float* srow = slab + ((size_t)b * N + t) * g;
   const int32_t* nb = nbr + ((size_t)b * N + t) * kk;
+  uint2* span = span_all + (size_t)b * N;
+  Entry* ent = ent_all + (size_t)b * N * g;
   gain_t acc = 0ull;
   for (int k = lane; k < g; k += 32) {
     const int j = k == 0 ? t : __ldg(nb + k - 1);
-    acc += gain_term(__ldg(v + j), m0, __ldg(srow + k), fx);
+    const float c = __ldg(srow + k);
+    const uint32_t at = atomicAdd(&span[j].y, 1u);
+    ent[span[j].x + at] = make_uint2((uint32_t)t, __float_as_uint(c));
+    acc += gain_term(__ldg(v + j), m0, c, fx);
   }
   acc = warp_sum_gain(acc);
   if (lane == 0) gains[(size_t)b * N + t] = acc;
@@ -1439,17 +1441,15 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
   r.g = P.g;
   r.kk = P.kk;
   if (local) {
-    const size_t rsmem = sizeof(int) * (size_t)N;
-    if (rsmem > 40 * 1024 &&
-        cuda_status(cudaFuncSetAttribute(k_rev_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)rsmem),
-                    "launch_sgs_push: reverse-list smem attribute") != CP_OK)
-      return CP_ECUDA;
-    k_rev_lists<<<(unsigned)B, 1024, rsmem, s>>>(nbr, slab, (int)N, P.g, P.kk, r.span,
-                                                 r.lists);
+    const dim3 per_token((unsigned)((N + 7) / 8), (unsigned)B);
+    CP_TRY_STATUS(cuda_status(cudaMemsetAsync(r.span, 0, sizeof(uint2) * (size_t)(B * N), s),
+                              "launch_sgs_push: lists"));
+    k_rev_count<<<per_token, 256, 0, s>>>(nbr, (int)N, P.g, P.kk, r.span);
     CP_TRY_STATUS(last_launch_status());
-    k_local_gains<<<dim3((unsigned)((N + 7) / 8), (unsigned)B), 256, 0, s>>>(
-        slab, nbr, v, (int)N, P.g, P.kk, P.m0, fx, gains64);
+    k_rev_scan<<<(unsigned)B, 1024, 0, s>>>((int)N, r.span);
+    CP_TRY_STATUS(last_launch_status());
+    k_rev_fill<<<per_token, 256, 0, s>>>(slab, nbr, v, (int)N, P.g, P.kk, P.m0, fx, r.span,
+                                         r.lists, gains64);
     CP_TRY_STATUS(last_launch_status());
     r.list_step = (size_t)N * (size_t)P.g;
     return launch_rounds(k_sgs_rounds<true>, r, B, di, s);
