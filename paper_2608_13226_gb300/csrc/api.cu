@@ -304,6 +304,11 @@ static T* at(void* ws, size_t off) {
     if (_st != CP_OK) return _st;  \
   } while (0)
 
+// The neighbour grid's sorted points, where the neighbours came from it.
+static const float4* grid_order(const DevParams& d, void* ws, const Plan& pl) {
+  return d.kk <= kKnnGridMax ? at<float4>(ws, pl.grid_pts) : nullptr;
+}
+
 // Stats, inverse norms, neighbours and normalisers: the shared front of
 // every entry point.
 // cos_out (bf16 features only, may be null): the normaliser pass also stores
@@ -482,7 +487,8 @@ int coverprune_cost(const void* feats, int dtype, const float* pos, const int32_
     Stage st(CP_STAGE_CAPACITY, s);
     CP_TRY(launch_capacity(feats, dtype, at<float>(ws, pl.inv), pos, frame, nm,
                            at<int32_t>(ws, pl.nbr), d, B, N, D, at<float>(ws, pl.r),
-                           at<float>(ws, pl.v), capacity, s, cosines, N));
+                           at<float>(ws, pl.v), capacity, s, cosines, N, nullptr,
+                           grid_order(d, ws, pl)));
   }
   if (cost) {
     Stage st(CP_STAGE_COST, s);
@@ -606,7 +612,8 @@ int coverprune_lite_select(const void* feats, int dtype, const float* pos, const
   {
     Stage st(CP_STAGE_CAPACITY, s);
     CP_TRY(launch_capacity(feats, dtype, inv, pos, frame, nm, at<int32_t>(ws, pl.nbr), d, B, N,
-                           D, at<float>(ws, pl.r), v, nullptr, s));
+                           D, at<float>(ws, pl.r), v, nullptr, s, nullptr, 0, nullptr,
+                           grid_order(d, ws, pl)));
   }
   int32_t* perm = at<int32_t>(ws, pl.perm);
   int32_t* gs = group_start ? group_start : at<int32_t>(ws, pl.gs);

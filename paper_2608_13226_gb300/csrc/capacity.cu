@@ -78,6 +78,72 @@ __global__ void __launch_bounds__(32 * CAP_WARPS) k_capacity_r(
   if (threadIdx.x == 0) r_all[(size_t)b * N + j] = P.n_cap > 0 ? acc / (float)P.n_cap : 0.0f;
 }
 
+// The same r_j for bf16 features, a warp a token: its row against eight of its
+// neighbours' at a time.  A block's 8 tokens are neighbours themselves (their
+// places follow the neighbour grid's order), so at any moment its warps read
+// the same columns of few distinct rows, most of them from L1; a block a
+// token, a warp a neighbour, brought every row from L2 each time it was a
+// neighbour.  32 scenes of 8192, D = 3584, 8 neighbours: 15 GB of such rows,
+// 1.31 ms, now 1.00; one scene of 16384 87 us, now 74.  Three blocks an SM:
+// at the registers the compiler takes by itself one fits, and 1.99 ms.  Every
+// dot product and sum keeps its order.
+__global__ void __launch_bounds__(256, 3) k_capacity_r_near(
+    const __nv_bfloat16* __restrict__ F_all, const float* __restrict__ inv_all,
+    const float* __restrict__ pos_all, const int32_t* __restrict__ frame_all,
+    const SceneNorms* __restrict__ norms, const int32_t* __restrict__ nbr_all,
+    const float4* __restrict__ order_all, DevParams P, int N, int D, float* __restrict__ r_all) {
+  const int slot = blockIdx.x * 8 + (threadIdx.x >> 5), b = blockIdx.y, lane = threadIdx.x & 31;
+  if (slot >= N) return;
+  const int j = __float_as_int(order_all[(size_t)b * N + slot].w);
+  const __nv_bfloat16* F = F_all + (size_t)b * N * D;
+  const float* inv = inv_all + (size_t)b * N;
+  const float* X = pos_all + (size_t)b * N * 3;
+  const int32_t* TAU = frame_all + (size_t)b * N;
+  const int32_t* nb = nbr_all + ((size_t)b * N + j) * P.kk;
+  const SceneNorms nm = norms[b];
+  const __nv_bfloat16* fj = F + (size_t)j * D;
+  float acc = 0.0f;
+  for (int q0 = 0; q0 < P.n_cap; q0 += 8) {
+    const int mine = nb[min(q0 + (lane & 7), P.n_cap - 1)];
+    const __nv_bfloat16* fk[8];
+    float dot[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      fk[i] = F + (size_t)__shfl_sync(0xFFFFFFFFu, mine, i) * D;
+      dot[i] = 0.0f;
+    }
+    for (int c = lane * 8; c < D; c += 256) {
+      const uint4 x = __ldg(reinterpret_cast<const uint4*>(fj + c));
+      uint4 y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) y[i] = __ldg(reinterpret_cast<const uint4*>(fk[i] + c));
+#pragma unroll
+      for (int i = 0; i < 8; ++i) dot[i] = dot8_bf16(x, y[i], dot[i]);
+    }
+    float own = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float t = warp_sum(dot[i]);
+      own = (lane & 7) == i ? t : own;
+    }
+    const int k = mine;
+    const float cosv = clamp_cos(own * inv[j] * inv[k]);
+    const float tf = ((1.0f - cosv) - nm.f_lo) * nm.f_rinv;
+    const float dx = sqrtf(
+        sqdist_rn(X[3 * j], X[3 * j + 1], X[3 * j + 2], X[3 * k], X[3 * k + 1], X[3 * k + 2]));
+    const float tx = (dx - nm.x_lo) * nm.x_rinv;
+    const int dt = TAU[j] - TAU[k];
+    const float tt = dt > 0 ? (float)dt * nm.t_rinv : 0.0f;
+    const float term = P.alpha_f * tf + P.alpha_x * tx + P.alpha_tau * tt;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float t = __shfl_sync(0xFFFFFFFFu, term, i);
+      if (q0 + i < P.n_cap) acc += t;
+    }
+  }
+  if (lane == 0) r_all[(size_t)b * N + j] = P.n_cap > 0 ? acc / (float)P.n_cap : 0.0f;
+}
+
 // The same r_j from stored cosines in place of the dot product, the rest
 // identical: the normaliser Gram's output, the upper triangle of
 // [B][N][ldc] (cos(j, k) at [min(j, k)][max(j, k)]); or, given pos_of, the
@@ -167,13 +233,16 @@ int launch_capacity(const void* feats, int dtype, const float* inv, const float*
                     const int32_t* frame, const SceneNorms* norms, const int32_t* nbr,
                     const DevParams& P, int64_t B, int64_t N, int64_t D, float* r, float* v,
                     float* v_out, cudaStream_t s, const float* cos, int64_t ldc,
-                    const int32_t* pos_of) {
+                    const int32_t* pos_of, const float4* order) {
   // one block per token, a warp per neighbour (at most CAP_WARPS)
   const dim3 grid((unsigned)N, (unsigned)B);
   const int warps = P.n_cap < 1 ? 1 : (P.n_cap < CAP_WARPS ? P.n_cap : CAP_WARPS);
   if (cos)
     k_capacity_r_cos<<<dim3((unsigned)((N + 255) / 256), (unsigned)B), 256, 0, s>>>(
         cos, ldc, pos, frame, norms, nbr, P, (int)N, pos_of, r);
+  else if (dtype == CP_BF16 && order)
+    k_capacity_r_near<<<dim3((unsigned)((N + 7) / 8), (unsigned)B), 256, 0, s>>>(
+        (const __nv_bfloat16*)feats, inv, pos, frame, norms, nbr, order, P, (int)N, (int)D, r);
   else if (dtype == CP_BF16)
     k_capacity_r<__nv_bfloat16><<<grid, 32 * warps, 0, s>>>(
         (const __nv_bfloat16*)feats, inv, pos, frame, norms, nbr, P, (int)N, (int)D, r);

@@ -132,11 +132,13 @@ int launch_cost(const void* feats, int dtype, const float* inv, const float4* to
 // K4: capacity score r and capacity v (Eqs. fst_capacity_score, fst_capacity).
 // cos (may be null): every cosine, [B][N][ldc], as the normaliser pass
 // stores it; the pairs' cosines are then read from it, not recomputed.
+// order (may be null): the neighbour grid's sorted points.
 int launch_capacity(const void* feats, int dtype, const float* inv, const float* pos,
                     const int32_t* frame, const SceneNorms* norms, const int32_t* nbr,
                     const DevParams& P, int64_t B, int64_t N, int64_t D, float* r, float* v,
                     float* v_out, cudaStream_t s, const float* cos = nullptr,
-                    int64_t ldc = 0, const int32_t* pos_of = nullptr);
+                    int64_t ldc = 0, const int32_t* pos_of = nullptr,
+                    const float4* order = nullptr);
 // Local SGS, bf16 features: the same slab computed from the stored cosines
 // (cos [B][N][ldc], as the normaliser pass writes them), without a dense cost.
 // (pos_of given: cos(t, j) at [min(pos)][max(pos)] of the flagged Morton tiles).
