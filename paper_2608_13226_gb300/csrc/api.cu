@@ -16,10 +16,11 @@ namespace cp {
 
 // Tensor-core (bf16) and SIMT (fp32) variants of the Gram kernels.
 int launch_gram_minmax_simt(const void* feats, int dtype, const float* inv, int64_t B, int64_t N,
-                            int64_t D, SceneStats* stats, cudaStream_t s);
-int launch_cost_simt(const void* feats, int dtype, const float* inv, const float* pos,
-                     const int32_t* frame, const SceneNorms* norms, const DevParams& P, int64_t B,
-                     int64_t N, int64_t D, float* cost, int64_t ldc, cudaStream_t s);
+                            int64_t D, SceneStats* stats, cudaStream_t s, float* dots,
+                            int64_t ldc);
+int launch_fst_simt(float* cost, int64_t ldc, int64_t B, int64_t N, const float* inv,
+                    const float* pos, const int32_t* frame, const SceneNorms* norms,
+                    const DevParams& P, cudaStream_t s);
 int64_t sgs_partials_count(int64_t B, int64_t N);
 int launch_gram_minmax_tc(const void* feats, const float4* tok, int64_t B, int64_t N, int64_t D,
                           SceneStats* stats, int* status, uint64_t timeout_ns, cudaStream_t s,
@@ -112,27 +113,15 @@ int device_info(DeviceInfo* out) {
 }
 
 // bf16 features: tcgen05 tensor cores; fp32 features: fp32 FMA tiles (TF32
-// would round the features to 10 mantissa bits).  cos_out (bf16 only; may
-// be null): every cosine stored [B][N][ldc] for the elementwise cost pass.
+// would round the features to 10 mantissa bits).  cos_out (may be null):
+// every cosine (bf16) or dot product (fp32) of a pair i <= j stored
+// [B][N][ldc] for the elementwise cost pass.
 int launch_gram_minmax(const void* feats, int dtype, const float* inv, const float4* tok,
                        int64_t B, int64_t N, int64_t D, SceneStats* stats, int* status,
                        uint64_t timeout_ns, cudaStream_t s, float* cos_out, int64_t ldc) {
   if (dtype == CP_BF16)
     return launch_gram_minmax_tc(feats, tok, B, N, D, stats, status, timeout_ns, s, cos_out, ldc);
-  return launch_gram_minmax_simt(feats, dtype, inv, B, N, D, stats, s);
-}
-
-// fp32 features: the FST cost on the SIMT cores (bf16 features take the
-// stored cosines and launch_fst_apply instead).
-int launch_cost(const void* feats, int dtype, const float* inv, const float4* tok,
-                const float* pos, const int32_t* frame, const SceneNorms* norms,
-                const DevParams& P, int64_t B, int64_t N, int64_t D, float* cost, int64_t ldc,
-                cudaStream_t s) {
-  if (dtype == CP_BF16) {
-    note_message("launch_cost: bf16 features take the stored-cosine cost pass");
-    return CP_EUNSUPPORTED;
-  }
-  return launch_cost_simt(feats, dtype, inv, pos, frame, norms, P, B, N, D, cost, ldc, s);
+  return launch_gram_minmax_simt(feats, dtype, inv, B, N, D, stats, s, cos_out, ldc);
 }
 
 // ---------------------------------------------------------------------------
@@ -311,8 +300,8 @@ static const float4* grid_order(const DevParams& d, void* ws, const Plan& pl) {
 
 // Stats, inverse norms, neighbours and normalisers: the shared front of
 // every entry point.
-// cos_out (bf16 features only, may be null): the normaliser pass also stores
-// every cosine there, [B][N][ldc], for launch_fst_apply.
+// cos_out (may be null): the normaliser pass also stores every cosine (bf16)
+// or dot product (fp32) there, [B][N][ldc], for the elementwise cost pass.
 static int run_front(const void* feats, int dtype, const float* pos, const int32_t* frame,
                      int64_t B, int64_t N, int64_t D, const DevParams& d, const Plan& pl, void* ws,
                      float* norms_out, cudaStream_t s, float* cos_out = nullptr,
@@ -333,10 +322,8 @@ static int run_front(const void* feats, int dtype, const float* pos, const int32
       CP_TRY(launch_knn(pos, at<float4>(ws, pl.tok), B, N, d.kk, at<int32_t>(ws, pl.nbr), stats,
                         s));
   }
-  // the Gram gives the min-max feature normaliser and, for bf16 inputs, the
-  // stored cosines; with the bounded normaliser and no cosines to store
-  // (Lite, or fp32 inputs) it does not run
-  cos_out = dtype == CP_BF16 ? cos_out : nullptr;
+  // the Gram gives the min-max feature normaliser and the stored products;
+  // with the bounded normaliser and none to store (Lite) it does not run
   if (d.norm_mode == 0 || cos_out) {
     Stage st(CP_STAGE_GRAM, s);
     CP_TRY(launch_gram_minmax(feats, dtype, at<float>(ws, pl.inv), at<float4>(ws, pl.tok), B, N,
@@ -477,9 +464,9 @@ int coverprune_cost(const void* feats, int dtype, const float* pos, const int32_
   Plan pl;
   CP_TRY(check_ws(CP_OP_COST, B, N, D, 0, dtype, d, ws, ws_bytes, &pl));
   cudaStream_t s = (cudaStream_t)stream;
-  // bf16: the normaliser pass stores the cosines into the output (the
-  // capacity reads its pairs there), then one elementwise pass turns them
-  // into the cost
+  // the normaliser pass stores the cosines (bf16: the capacity reads its
+  // pairs there) or dot products (fp32) into the output, then one elementwise
+  // pass turns them into the cost
   CP_TRY(run_front(feats, dtype, pos, frame, B, N, D, d, pl, ws, norms, s, cost, N));
   const SceneNorms* nm = at<SceneNorms>(ws, pl.norms);
   const float* cosines = dtype == CP_BF16 ? cost : nullptr;
@@ -496,8 +483,7 @@ int coverprune_cost(const void* feats, int dtype, const float* pos, const int32_
       CP_TRY(launch_fst_apply(cost, N, B, N, at<float4>(ws, pl.tok), frame, nm, d, nullptr,
                               nullptr, s));
     else
-      CP_TRY(launch_cost(feats, dtype, at<float>(ws, pl.inv), at<float4>(ws, pl.tok), pos, frame,
-                         nm, d, B, N, D, cost, N, s));
+      CP_TRY(launch_fst_simt(cost, N, B, N, at<float>(ws, pl.inv), pos, frame, nm, d, s));
   }
   return record_inputs_done(p, s);
 }
@@ -520,7 +506,7 @@ int coverprune_select(const void* feats, int dtype, const float* pos, const int3
   cudaStream_t s = (cudaStream_t)stream;
   int* status = at<int>(ws, pl.hdr);
   float* C = at<float>(ws, pl.cost);
-  // the all-pairs Gram stores every cosine into C for the cost pass; the
+  // the all-pairs Gram stores every pair's product into C for the cost pass; the
   // local path with the bounded normaliser stores only the Morton tiles it
   // needs (below), so the front runs no Gram for it
   const bool tiles = local_tiles_path(CP_OP_SELECT, dtype, N, d);
@@ -565,8 +551,7 @@ int coverprune_select(const void* feats, int dtype, const float* pos, const int3
     else if (dtype == CP_BF16)
       CP_TRY(launch_fst_apply(C, pl.ldc, B, N, at<float4>(ws, pl.tok), frame, nm, d, v, g0, s));
     else
-      CP_TRY(launch_cost(feats, dtype, inv, at<float4>(ws, pl.tok), pos, frame, nm, d, B, N, D, C,
-                         pl.ldc, s));
+      CP_TRY(launch_fst_simt(C, pl.ldc, B, N, inv, pos, frame, nm, d, s));
   }
   // the greedy selection reads none of feats, pos, frame
   CP_TRY(record_inputs_done(p, s));

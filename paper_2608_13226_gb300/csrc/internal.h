@@ -122,13 +122,6 @@ int launch_diameter(const SceneStats* stats, int64_t B, float* out, cudaStream_t
 // the Gram's extremes).  Optionally also the public [B, 6] float copy.
 int launch_finalize_norms(const SceneStats* stats, int64_t B, int norm_mode, SceneNorms* norms,
                           float* norms_out, cudaStream_t s);
-// K3 for fp32 features: the FST cost C[b][s][t] into cost + b*N*ldc + s*ldc
-// + t for t < N; columns N <= t < ldc are written as 0.  (bf16 features:
-// launch_gram_minmax stores the cosines, then launch_fst_apply.)
-int launch_cost(const void* feats, int dtype, const float* inv, const float4* tok,
-                const float* pos, const int32_t* frame, const SceneNorms* norms,
-                const DevParams& P, int64_t B, int64_t N, int64_t D, float* cost, int64_t ldc,
-                cudaStream_t s);
 // K4: capacity score r and capacity v (Eqs. fst_capacity_score, fst_capacity).
 // cos (may be null): every cosine, [B][N][ldc], as the normaliser pass
 // stores it; the pairs' cosines are then read from it, not recomputed.
