@@ -1123,7 +1123,7 @@ int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr
   const int gmax = grid_cells_max(N);
   if (kk > kKnnGridMax) return CP_EINVAL;
   const size_t smem = sizeof(int) * (size_t)(gmax + 1);
-  if (smem > 48 * 1024 &&
+  if (smem > 40 * 1024 &&  // beside ~1 KB of static shared memory
       (cuda_status(cudaFuncSetAttribute(k_grid_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)smem),
                    "launch_knn_grid: smem attribute") != CP_OK ||
