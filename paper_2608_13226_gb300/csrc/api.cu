@@ -192,7 +192,7 @@ struct Plan {
   size_t cost, slab, partials, order32, g0, push;  // select
   size_t lit;                                     // literal SGS (sgs_mode 2) scratch
   size_t lfeats, ltok, lperm, lpos, lflags, lunits, lnunits;  // local Morton tiles
-  size_t perm, prefix, gs, proto, score;          // lite
+  size_t perm, gs, proto, score;                  // lite
   size_t total;
   int64_t ldc;
 };
@@ -261,7 +261,6 @@ static void plan_ws(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtyp
     pl->g0 = take(sizeof(float) * BN * (size_t)fst_apply_slots(pl->ldc));
   } else if (op == CP_OP_LITE) {
     pl->perm = take(sizeof(int32_t) * BN);
-    pl->prefix = take(sizeof(uint64_t) * BN);
     pl->gs = take(sizeof(int32_t) * (size_t)B * (size_t)(K + 1));
     pl->proto = take(sizeof(int32_t) * (size_t)B * (size_t)K);
     pl->score = take(sizeof(double) * (size_t)B * (size_t)K);
@@ -605,7 +604,7 @@ int coverprune_lite_select(const void* feats, int dtype, const float* pos, const
   {
     Stage st(CP_STAGE_LITE_ORDER, s);
     CP_TRY(launch_morton(pos, at<SceneStats>(ws, pl.stats), d, B, N, perm, s));
-    CP_TRY(launch_groups(v, perm, B, N, K, at<uint64_t>(ws, pl.prefix), gs, s));
+    CP_TRY(launch_groups(v, perm, B, N, K, gs, s));
   }
   int32_t* proto = at<int32_t>(ws, pl.proto);
   {

@@ -191,7 +191,7 @@ int launch_morton(const float* pos, const SceneStats* stats, const DevParams& P,
                   int64_t N, int32_t* perm, cudaStream_t s);
 // K7: capacity-guided group starts gs[b*(K+1) + q] (int32).
 int launch_groups(const float* v, const int32_t* perm, int64_t B, int64_t N, int64_t K,
-                  uint64_t* prefix, int32_t* gs, cudaStream_t s);
+                  int32_t* gs, cudaStream_t s);
 // K8: per-group prototype and its score; objective = sum of scores.
 int launch_lite_proto(const void* feats, int dtype, const float* inv, const float* pos,
                       const int32_t* frame, const SceneNorms* norms, const float* v,

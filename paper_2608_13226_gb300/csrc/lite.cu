@@ -158,34 +158,7 @@ int launch_morton(const float* pos, const SceneStats* stats, const DevParams& P,
   return last_launch_status();
 }
 
-// Block-wide inclusive scans over blockDim.x == 1024 values.
-__device__ __forceinline__ unsigned long long block_incl_sum_u64(unsigned long long x,
-                                                                 unsigned long long* s_w,
-                                                                 unsigned long long* total) {
-  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (l >= o) x += y;
-  }
-  if (l == 31) s_w[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    unsigned long long y = s_w[l];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      unsigned long long z = __shfl_up_sync(0xFFFFFFFFu, y, o);
-      if (l >= o) y += z;
-    }
-    s_w[l] = y;
-  }
-  __syncthreads();
-  const unsigned long long r = x + (w > 0 ? s_w[w - 1] : 0ull);
-  *total = s_w[31];
-  __syncthreads();
-  return r;
-}
-
+// Block-wide inclusive scan over blockDim.x == 1024 values.
 __device__ __forceinline__ int block_incl_max_int(int x, int* s_w, int* total) {
   const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
@@ -215,52 +188,85 @@ __device__ __forceinline__ int block_incl_max_int(int x, int* s_w, int* total) {
 //   Q_j = rint(v_j 2^40); P(p) = inclusive running mass in Morton order;
 //   ideal start of group q >= 1: 1 + min{p : P(p) K >= q P(N-1)};
 //   b_q = q + min(N - K, max_{q' <= q} (ideal_q' - q')), b_0 = 0, b_K = N.
-// One block of 1024 threads per scene.
+// One block of 1024 threads per scene.  Each warp sums a contiguous run of the
+// order, kept in shared memory; a group's start is searched there (all
+// products fit 64 bits: P(N-1) is 2^40 and a little, K at most 2^14).
+// Latency-bound: 16384 tokens 16 us; with the masses in global memory, a
+// block scan per 1024 tokens and 128-bit products 43.
 __global__ void __launch_bounds__(1024) k_groups(const float* __restrict__ v_all,
                                                  const int32_t* __restrict__ perm_all, int N, int K,
-                                                 unsigned long long* __restrict__ prefix_all,
                                                  int32_t* __restrict__ gs_all) {
-  __shared__ unsigned long long s_w[32];
+  extern __shared__ unsigned long long s_P[];  // [N] masses within a warp's run, inclusive
+  __shared__ unsigned long long s_off[33];     // mass before each warp's run; [32]: all of it
   __shared__ int s_wi[32];
-  const int b = blockIdx.x;
+  const int b = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float* v = v_all + (size_t)b * N;
   const int32_t* perm = perm_all + (size_t)b * N;
-  unsigned long long* P = prefix_all + (size_t)b * N;
   int32_t* gs = gs_all + (size_t)b * (K + 1);
+  const int run = ((N + 31) / 32 + 31) & ~31;  // tokens a warp
+  const int p0 = min(N, w * run), p1 = min(N, p0 + run);
   unsigned long long carry = 0ull;
-  for (int c0 = 0; c0 < N; c0 += 1024) {
-    const int p = c0 + threadIdx.x;
-    unsigned long long q = 0ull;
-    if (p < N) {
-      const float vj = v[perm[p]];
-      q = vj > 0.0f ? __double2ull_rn((double)vj * 1099511627776.0) : 0ull;  // 2^40
+  for (int p = p0; p < p1; p += 128) {  // four chunks' loads in flight
+    float x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = p + 32 * u + lane;
+      x[u] = i < p1 ? v[perm[i]] : 0.0f;
     }
-    unsigned long long tot;
-    const unsigned long long incl = block_incl_sum_u64(q, s_w, &tot);
-    if (p < N) P[p] = carry + incl;
-    carry += tot;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      // rint(v 2^40), the product exact
+      unsigned long long q = x[u] > 0.0f ? __float2ull_rn(x[u] * 1099511627776.0f) : 0ull;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, q, o);
+        if (lane >= o) q += t;
+      }
+      q += carry;
+      carry = __shfl_sync(0xFFFFFFFFu, q, 31);
+      const int i = p + 32 * u + lane;
+      if (i < p1) s_P[i] = q;
+    }
+  }
+  if (lane == 0) s_off[w] = carry;
+  __syncthreads();
+  if (w == 0) {
+    unsigned long long q = s_off[lane];
+    const unsigned long long own = q;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, q, o);
+      if (lane >= o) q += t;
+    }
+    s_off[lane] = q - own;
+    if (lane == 31) s_off[32] = q;
   }
   __syncthreads();
-  const unsigned long long total = carry;
+  const unsigned long long total = s_off[32];
   // ideal_q - q for q = 1..K-1, staged in gs[q]
   for (int q = 1 + threadIdx.x; q < K; q += 1024) {
-    const unsigned __int128 target = (unsigned __int128)q * total;
-    int lo = 0, hi = N - 1;  // smallest p with P[p] * K >= target (exists: P[N-1]*K >= target)
+    const unsigned long long target = (unsigned long long)q * total;
+    // smallest p with P(p) K >= target (exists: P(N-1) K >= target): the run
+    // first, then within it
+    int r = 0;
+    while (r < 31 && (r + 1) * run < N && s_off[r + 1] * (unsigned)K < target) ++r;
+    const unsigned long long before = s_off[r];
+    int lo = r * run, hi = min(N, lo + run) - 1;
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      if ((unsigned __int128)__ldcg(P + mid) * (unsigned)K >= target) hi = mid; else lo = mid + 1;
+      if ((before + s_P[mid]) * (unsigned)K >= target) hi = mid; else lo = mid + 1;
     }
     gs[q] = (lo + 1) - q;
   }
   __syncthreads();
-  int run = INT32_MIN;
+  int top = INT32_MIN;
   for (int c0 = 1; c0 < K; c0 += 1024) {
     const int q = c0 + threadIdx.x;
-    const int d = q < K ? gs[q] : INT32_MIN;
+    const int x = q < K ? gs[q] : INT32_MIN;
     int tot;
-    const int m = max(run, block_incl_max_int(d, s_wi, &tot));
+    const int m = max(top, block_incl_max_int(x, s_wi, &tot));
     if (q < K) gs[q] = q + min(N - K, m);
-    run = max(run, tot);
+    top = max(top, tot);
   }
   if (threadIdx.x == 0) {
     gs[0] = 0;
@@ -269,9 +275,14 @@ __global__ void __launch_bounds__(1024) k_groups(const float* __restrict__ v_all
 }
 
 int launch_groups(const float* v, const int32_t* perm, int64_t B, int64_t N, int64_t K,
-                  uint64_t* prefix, int32_t* gs, cudaStream_t s) {
-  k_groups<<<(unsigned)B, 1024, 0, s>>>(v, perm, (int)N, (int)K,
-                                        reinterpret_cast<unsigned long long*>(prefix), gs);
+                  int32_t* gs, cudaStream_t s) {
+  const size_t smem = sizeof(unsigned long long) * (size_t)N;
+  if (smem > 40 * 1024 &&
+      cuda_status(cudaFuncSetAttribute(k_groups, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem),
+                  "launch_groups: smem attribute") != CP_OK)
+    return CP_ECUDA;
+  k_groups<<<(unsigned)B, 1024, smem, s>>>(v, perm, (int)N, (int)K, gs);
   return last_launch_status();
 }
 
