@@ -339,26 +339,28 @@ def run_ours(args, rank, world, local_rank, raw):
     ms_step = max_over_ranks(ev0.elapsed_time(ev1) / args.steps)
     value = whole_job_rate(B, world, ms_step)
 
-    # roofline of the SGS kernel from its own events and its counted reads:
-    # the cost bytes its gain evaluations and coverage updates read (the
-    # kernel counts them; row blocks known to hold only zero terms are
-    # skipped)
+    # roofline of the selection (its kernels together) from the stage's events
+    # and the bytes it reads: the cost once, for the live lists and the gains
+    # after the first pick, and what the steps count (winners' rows, live
+    # entries of the lowered targets' lists)
     hbm, tf_burst, tf_sust, peak_kind = measured_peaks()
     cstats = cp.coverprune_call_stats(ws)
     sgs_ms, sgs_launches = prof["sgs"]
-    launches_per_step = max(sgs_launches // args.steps, 1)
     ldc = (N + 3) // 4 * 4
-    sgs_bytes_per_step = cstats["cost_bytes_read"]
-    sgs_launch_ms = sgs_ms / max(sgs_launches, 1)
-    sgs_gbs = (sgs_bytes_per_step / launches_per_step) / (sgs_launch_ms / 1000.0) / 1e9
-    roofline_sgs = {"bound": "hbm", "kernel": "k_sgs_push", "achieved": round(sgs_gbs, 1),
+    sgs_bytes_per_step = cstats["cost_bytes_read"] + 4 * B * N * ldc
+    sgs_step_ms = sgs_ms / args.steps
+    sgs_gbs = sgs_bytes_per_step / (sgs_step_ms / 1000.0) / 1e9
+    roofline_sgs = {"bound": "hbm",
+                    "kernel": "k_live_lists + k_sgs_push + k_join_lists + k_sgs_rounds",
+                    "achieved": round(sgs_gbs, 1),
                     "peak": hbm, "unit": "GB/s", "frac": round(sgs_gbs / hbm, 4),
                     "frac_of_nominal": round(sgs_gbs / HBM_NOMINAL_GBS, 4),
-                    "traffic": read_traffic("k_sgs_push", sgs_bytes_per_step // launches_per_step),
+                    "traffic": read_traffic("sgs_selection", sgs_bytes_per_step),
                     "peak_source": peak_kind,
-                    "algorithmic_bytes_per_launch": sgs_bytes_per_step // launches_per_step,
-                    "avg_launch_ms": round(sgs_launch_ms, 3),
-                    "gain_evaluations_per_step": cstats["gain_evaluations"],
+                    "algorithmic_bytes_per_step": sgs_bytes_per_step,
+                    "ms_per_step": round(sgs_step_ms, 3),
+                    "launches_per_step": sgs_launches // args.steps,
+                    "terms_updated_per_step": cstats["gain_evaluations"],
                     "rounds_per_step": cstats["rounds"],
                     "cost_bytes_read_per_step": cstats["cost_bytes_read"],
                     "full_sweep_evaluations_per_step": B * (K * N - K * (K - 1) // 2)}
