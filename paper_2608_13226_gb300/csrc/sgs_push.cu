@@ -26,9 +26,9 @@
 //  - k_sgs_rounds, one block per scene, many picks a round, for the rest
 //    (and all of a local selection): late picks lower few targets each,
 //    mostly different ones, so dozens of them are independent of one another.
-// Selection of 1229 of 8192 tokens: 2.95 ms (re-evaluating candidate rows
+// Selection of 1229 of 8192 tokens: 2.7 ms (re-evaluating candidate rows
 // behind bounds, the approach before these: 11.9; one pick a step to the end:
-// 5.9); 410 of 4096: 1.14 (3.8, 2.1); 32 scenes of 8192: 8.6 (19.9, 12.0).
+// 5.9); 410 of 4096: 1.05 (3.8, 2.1); 32 scenes of 8192: 8.5 (19.9, 12.0).
 #include <string.h>
 
 #include "bf16_dot.cuh"
@@ -42,7 +42,8 @@ constexpr int PUSH_WARPS = 32;
 // The single-pick steps end once the running mean of the targets a pick
 // lowers is below this: a step costs ~2 us whatever it lowers, a pick of a
 // round costs its lists' share of one block, and where rows are still longer
-// than RD_ROW rounds pick one at a time.  Selection, ms, at 16 / 24 / 32 / 40
+// than RD_ROW rounds pick one at a time.  Selection, ms, with a warp a list, at
+// 16 / 24 / 32 / 40
 // / 48 / 64: N = 1024 0.34 / 0.32 / 0.32 / 0.31 / 0.31 / 0.30, N = 4096 1.22 /
 // 1.20 / 1.15 / 1.14 / 1.13 / 1.12, N = 8192 3.00 / 2.97 / 2.96 / 2.95 / 3.22 /
 // 3.21, 32 scenes of N = 8192 8.65 / 8.52 / 8.54 / 8.61 / 9.17 / 9.23.
@@ -390,17 +391,7 @@ __device__ __forceinline__ void chunk_high(uint32_t* hi, uint32_t at, gain_t d, 
     if (dh) atomicAdd(hi + at, 0u - dh);
   }
 }
-// The chunk's entries that stay live (c < mn; infinite past the list), packed
-// from place `out` of the list on.
-__device__ __forceinline__ void chunk_pack(Entry* L, const Entry& x, int i, float mn, int lane,
-                                           int& out) {
-  const bool stay = __uint_as_float(x.y) < mn;
-  const uint32_t mask = __ballot_sync(0xFFFFFFFFu, stay);
-  const int p = out + __popc(mask & ((1u << lane) - 1u));
-  if (stay && p != i) __stcg(L + p, x);
-  out += __popc(mask);
-}
-
+template <int LW>
 __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_constant__ PushArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   float* sm_m = reinterpret_cast<float*>(smem);                     // [ldc] coverage cost
@@ -567,14 +558,16 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
       ok = false;
       break;
     }
-    // ---- a warp per lowered target: its live candidates lose what the drop
+    // ---- LW lanes per lowered target: its live candidates lose what the drop
     // took; the entries that stay live are packed to the list's front.  Four
-    // chunks of 32 entries are in flight, and the next target's length and
-    // costs load meanwhile.
-    const int qn = s_qn;
+    // entries a lane are in flight, and the next target's length and costs
+    // load meanwhile.
+    constexpr int PER = 32 / LW;  // targets a warp takes at a time
+    const int qn = s_qn, sub = lane / LW, gl = lane & (LW - 1);
     int j = 0, len = 0;
     float mn = 0.0f, vj = 0.0f;
     auto next = [&](int q) {
+      len = 0;
       if (q < qn) {
         j = (int)queue[q];
         len = (int)__ldcg(a.lens + ((size_t)bl * N + j) * a.C + rank);
@@ -582,47 +575,40 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
         vj = __ldg(v + j);
       }
     };
-    next(w);
+    next(PER * w + sub);
 #pragma unroll 1
-    for (int q = w; q < qn; q += PUSH_WARPS) {
+    for (int q = PER * w; q < qn; q += PER * PUSH_WARPS) {
       const int jc = j, lenc = len;
       const float mnc = mn, mo = sm_m[j], vc = vj;
       const size_t lj = ((size_t)bl * N + jc) * a.C + rank;
       Entry* L = a.lists + lj * a.NC;
-      next(q + PUSH_WARPS);
-      int out = 0, i0 = 0;
+      const bool on = q + sub < qn;
+      next(q + PER * PUSH_WARPS + sub);
+      int out = 0;
 #pragma unroll 1
-      for (; i0 + 96 < lenc; i0 += 128) {  // four chunks, the last perhaps not full
+      for (int i0 = gl; __any_sync(0xFFFFFFFFu, i0 - gl < lenc); i0 += 4 * LW) {
         Entry x[4];
         gain_t d[4];
         uint32_t old[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + 32 * u + lane;
-          x[u] = i < lenc ? __ldcg(L + i) : make_uint2(0u, 0x7F800000u);
-        }
+        for (int u = 0; u < 4; ++u)
+          x[u] = i0 + LW * u < lenc ? __ldcg(L + i0 + LW * u) : make_uint2(0u, 0x7F800000u);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          d[u] = chunk_low(g_lo, x[u].x, true, vc, mo, mnc, __uint_as_float(x[u].y), fx,
-                                 old[u]);
+          d[u] = chunk_low(g_lo, x[u].x, true, vc, mo, mnc, __uint_as_float(x[u].y), fx, old[u]);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           chunk_high(g_hi, x[u].x, d[u], old[u]);
           if (d[u] != 0ull) s_dirty[x[u].x >> a.lgS] = 1u;
-          chunk_pack(L, x[u], i0 + 32 * u + lane, mnc, lane, out);
+          const bool stay = __uint_as_float(x[u].y) < mnc;
+          uint32_t mask = __ballot_sync(0xFFFFFFFFu, stay);
+          if (LW < 32) mask = (mask >> (lane & (32 - LW))) & ((1u << (LW & 31)) - 1u);
+          const int p = out + __popc(mask & ((1u << gl) - 1u));
+          if (stay && p != i0 + LW * u) __stcg(L + p, x[u]);
+          out += __popc(mask);
         }
       }
-#pragma unroll 1
-      for (; i0 < lenc; i0 += 32) {
-        const Entry x = i0 + lane < lenc ? __ldcg(L + i0 + lane) : make_uint2(0u, 0x7F800000u);
-        uint32_t old;
-        const gain_t d = chunk_low(g_lo, x.x, true, vc, mo, mnc, __uint_as_float(x.y), fx,
-                                         old);
-        chunk_high(g_hi, x.x, d, old);
-        if (d != 0ull) s_dirty[x.x >> a.lgS] = 1u;
-        chunk_pack(L, x, i0 + lane, mnc, lane, out);
-      }
-      if (lane == 0) {
+      if (gl == 0 && on) {
         my_ent += (unsigned long long)lenc;
         if (out != lenc) __stcg(a.lens + lj, (uint32_t)out);
         sm_m[jc] = mnc;
@@ -635,7 +621,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
 
   unsigned long long* cstats = reinterpret_cast<unsigned long long*>(
       reinterpret_cast<unsigned char*>(a.status) + kCallStatsOffset);
-  if (lane == 0 && my_ent) {
+  if ((lane & (LW - 1)) == 0 && my_ent) {
     atomicAdd(&cstats[0], my_ent);
     atomicAdd(&cstats[2], 8ull * my_ent);
   }
@@ -1505,7 +1491,16 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
     int C0 = PUSH_CMAX;
     while (C0 > 1 && ((int64_t)C0 * nb > di.sm_count || N / C0 < 128)) C0 >>= 1;
     if (C0 < 2 && N > 12288) C0 = 2;
-    auto push_fn = k_sgs_push;
+    // lanes a list (its part in one block: N / C candidates at most): short
+    // parts leave most of a warp idle, and a list is a chain of latencies;
+    // many blocks with long parts are bound by the shared-memory atomics.
+    // Selection, ms, at 8 / 16 / 32: one scene of 1024 (C = 8) 0.304 / 0.317 /
+    // 0.354, of 8192 (16) 2.87 / 2.92 / 3.25, of 16384 (16) 11.3 / 11.2 / 11.7;
+    // 8 of 8192 (16) 4.45 / 4.32 / 4.46, 16 (8) 7.15 / 7.05 / 7.40, 32 (4) 8.71
+    // / 8.24 / 7.99; 32 of 2048 (4) 0.99 / 0.98 / 1.03.
+    const int64_t part = N / C0;
+    auto push_fn = part >= 2048 ? k_sgs_push<32>
+                                : (nb == 1 && part <= 512 ? k_sgs_push<8> : k_sgs_push<16>);
     CP_TRY_STATUS(push_config(push_fn, a, C0, nb, di, s, &cfg, attr));
     a.scene0 = (int)b0;
     lists_fn<<<dim3((unsigned)((N + LL_COLS - 1) / LL_COLS), (unsigned)a.C, (unsigned)nb),
