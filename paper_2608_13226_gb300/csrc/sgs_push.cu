@@ -42,11 +42,11 @@ constexpr int PUSH_WARPS = 32;
 // The single-pick steps end once the running mean of the targets a pick
 // lowers is below this: a step costs ~2 us whatever it lowers, a pick of a
 // round costs its lists' share of one block, and where rows are still longer
-// than RD_ROW rounds pick one at a time.  Selection, ms, with a warp a list, at
-// 16 / 24 / 32 / 40
-// / 48 / 64: N = 1024 0.34 / 0.32 / 0.32 / 0.31 / 0.31 / 0.30, N = 4096 1.22 /
-// 1.20 / 1.15 / 1.14 / 1.13 / 1.12, N = 8192 3.00 / 2.97 / 2.96 / 2.95 / 3.22 /
-// 3.21, 32 scenes of N = 8192 8.65 / 8.52 / 8.54 / 8.61 / 9.17 / 9.23.
+// than RD_ROW rounds pick one at a time.  Selection, ms, with a warp a list,
+// at 16 / 24 / 32 / 40 / 48 / 64: N = 1024 0.34 / 0.32 / 0.32 / 0.31 / 0.31 /
+// 0.30, N = 4096 1.22 / 1.20 / 1.15 / 1.14 / 1.13 / 1.12, N = 8192 3.00 / 2.97
+// / 2.96 / 2.95 / 3.22 / 3.21, 32 scenes of N = 8192 8.65 / 8.52 / 8.54 / 8.61
+// / 9.17 / 9.23.
 constexpr int PUSH_STOP = 36;
 constexpr int PUSH_THREADS = 32 * PUSH_WARPS;
 
