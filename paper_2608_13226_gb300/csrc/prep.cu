@@ -1121,7 +1121,7 @@ int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr
                     SceneStats* stats, GridInfo* info, int32_t* cell_start, float4* sorted,
                     cudaStream_t s) {
   const int gmax = grid_cells_max(N);
-  if (kk > kKnnGridMax) return CP_EINVAL;
+  if (kk > kKnnGridMax || (kk > 0 && kk >= N)) return CP_EINVAL;  // the search needs kk others
   const size_t smem = sizeof(int) * (size_t)(gmax + 1);
   if (smem > 40 * 1024 &&  // beside ~1 KB of static shared memory
       (cuda_status(cudaFuncSetAttribute(k_grid_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
