@@ -589,9 +589,13 @@ __global__ void __launch_bounds__(1024) k_grid_build(const float* __restrict__ p
 // One warp per query token, queries in cell order.  Three scans of candidate
 // ranges (a range is the cells of one (y, z) row, contiguous in the sorted
 // points; the ranges of 32 rows are scanned as one flat sequence):
-//  - the smallest block of cells around the query with more than kk points,
-//    at least 3 x 3 x 3: a histogram of the squared distances, 8 bins an
-//    octave, gives a bound U that at least kk of them are below;
+//  - the query's own cell if it has more than 2 kk points, else the smallest
+//    block of 3, 5, ... cells a side around it with more than kk: a histogram
+//    of the squared distances, 8 bins an octave, gives a bound U that at least
+//    kk of them are below (16384 tokens, 8 neighbours: the whole preparation
+//    124 us, 159 with blocks of 3 cells a side at least, 122 / 130 with the
+//    own cell from kk / 4 kk points on; 64 neighbours of 32 scenes 1.16 ms,
+//    1.16, 1.28 / 1.17);
 //  - every cell within sqrt(U) (rows and ends of rows by their distance, with
 //    a margin for the rounding of the cell coordinates): the keys below U are
 //    gathered, kk and usually a few more;
@@ -602,7 +606,7 @@ __global__ void __launch_bounds__(1024) k_grid_build(const float* __restrict__ p
 // instruction issue (a point costs ~40 instructions a scan, of the warp), no
 // longer by the chain of one thread's scan and list: 56,000 queries (8 scenes
 // of 7000), kk = 63: 0.17 ms, a heap per thread took 0.62; 262,144 queries:
-// 0.82 (1.66); one scene of 8192, kk = 8: 0.024 (0.087), of 16384 0.076
+// 0.82 (1.66); one scene of 8192, kk = 8: 0.017 (0.087), of 16384 0.041
 // (0.37).
 constexpr int KW_WARPS = 8, KW_CAP = 256;
 
@@ -726,7 +730,7 @@ __global__ void __launch_bounds__(32 * KW_WARPS) k_knn_grid(
   };
 
   // ---- a block with more than kk points (the query among them)
-  for (int r = 1;; ++r) {
+  for (int r = 0;; ++r) {
     block(r);
     const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
     int n = 0;
@@ -735,7 +739,7 @@ __global__ void __launch_bounds__(32 * KW_WARPS) k_knn_grid(
       n += row(q, rows, ny, start);
     }
     n = __reduce_add_sync(0xFFFFFFFFu, n);
-    if (n > kk) break;  // N > kk: the whole grid at the latest
+    if (n > (r == 0 ? 2 * kk : kk)) break;  // N > kk: the whole grid at the latest
   }
   const float far = 64.0f * g.h;
   const int off = (int)(__float_as_uint(far * far) >> 20) - 255;
@@ -814,7 +818,7 @@ __global__ void __launch_bounds__(32 * KW_WARPS) k_knn_grid(
   }
 }
 
-// Few neighbours of very many queries (kk <= 8): one thread per query token
+// Few neighbours (kk <= 8) of very many small scenes: one thread per query token
 // scans the shells of cells at Chebyshev distance r = 0, 1, 2, ... from its
 // own cell; every point outside the first r shells is more than r h away
 // along some axis, so once the kk-th best squared distance is below ((r -
@@ -1138,12 +1142,12 @@ int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr
                                                                           stats);
   CP_TRY_STATUS(last_launch_status());
   if (kk <= 0) return CP_OK;
-  // A thread a query needs fewer instructions, but only many queries hide its
-  // latency.  kk = 8, us, thread / warp (with k_grid_build and
-  // k_diameter_grid), scenes of 8192: 8 300 / 224, 12 346 / 283, 16 349 / 338,
-  // 20 356 / 400, 32 584 / 579; 32 of 4096 268 / 308, 128 of 1024 184 / 250,
-  // 8 of 16384 525 / 494; 32 long videos 300 / 491 for the search alone.
-  if (kk <= 8 && B * N >= 131072) {
+  // A thread a query needs fewer instructions where cells hold few points, but
+  // only many queries hide its latency.  kk = 8, us, thread / warp (with
+  // k_grid_build and k_diameter_grid): 128 scenes of 1024 176 / 223, 32 of 4096
+  // 227 / 219, of 8192 8 252 / 143, 16 303 / 219, 32 508 / 383, 8 of 16384
+  // 374 / 245; 32 long videos (the whole preparation) 655 / 657.
+  if (kk <= 8 && N <= 2048 && B * N >= 131072) {
     k_knn_grid_thread<8><<<dim3((unsigned)((N + 127) / 128), (unsigned)B), 128, 0, s>>>(
         (int)N, kk, gmax, info, cell_start, sorted, nbr);
     return last_launch_status();
