@@ -333,14 +333,14 @@ __global__ void __launch_bounds__(LS_THREADS, 1) k_lit_sinkhorn(const __grid_con
   float* cap = reinterpret_cast<float*>(all + (size_t)2 * a.CB * lp);  // [W] v, or eps log v
   float* f = cap + W;                                                // [l] F, or f
   __shared__ __align__(8) uint64_t s_bar[2];
-  __shared__ int s_fail, s_bad, s_again;
+  __shared__ int s_fail, s_bad, s_again, s_abort;
   const int rank = (int)cluster_ctarank(), b = blockIdx.x / a.CB;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c0 = rank * W, nc = max(0, min(W, a.N - c0));
   const unsigned long long* keys = a.keys + (size_t)b * a.K;
   if (threadIdx.x == 0) {
     if (rank == 0) a.chosen[(size_t)b * a.N + key_index(keys[l - 1])] = 1;
-    s_fail = s_bad = s_again = 0;
+    s_fail = s_bad = s_again = s_abort = 0;
     mbar_init(&s_bar[0], 1);
     mbar_init(&s_bar[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -530,13 +530,16 @@ __global__ void __launch_bounds__(LS_THREADS, 1) k_lit_sinkhorn(const __grid_con
       }
     }
     __syncthreads();
-    if (factors && s_bad && threadIdx.x < a.CB)  // one block's step again is everybody's
+    // one block's step again is everybody's, and so is its giving up: a block
+    // may have passed the wait that another one gave up in
+    if ((!ok || (factors && s_bad)) && threadIdx.x < a.CB)
       asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
-                       map_rank(smem_addr(&s_again), threadIdx.x)),
+                       map_rank(smem_addr(ok ? &s_again : &s_abort), threadIdx.x)),
                    "r"(1)
                    : "memory");
     // nobody leaves while a copy of its own sums or into it may be under way
     hw_cluster_sync();
+    ok = s_abort == 0;  // the same in every block of the cluster
     if (factors && s_again && ok) continue;
     if (ok)
       for (int j = threadIdx.x; j < nc; j += LS_THREADS)

@@ -47,3 +47,27 @@ def test_select_reports_ok_status():
         assert cp.coverprune_check(r["ws"]) == cp.CP_OK
     lt = cp.coverprune_lite_select(f, pos, fr, 30)
     assert cp.coverprune_check(lt["ws"]) == cp.CP_OK
+
+
+@pytest.mark.parametrize("eps", [0.05, 1e-3])  # the factors alone; both forms of the iterations
+def test_literal_rule_gives_up_as_a_cluster(eps):
+    """Waits of the transport rule's iterations limited to a nanosecond: a
+    block may give up where its peers did not have to wait, and then none of
+    the cluster may go on to the second form.  The call returns, its status is
+    one of the two, and the context and the workspace work afterwards."""
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    f = torch.randn(5, 1024, 64, generator=gen, device="cuda")
+    pos = torch.rand(5, 1024, 3, generator=gen, device="cuda") * 6
+    fr = (torch.arange(1024, device="cuda") // 128).to(torch.int32).expand(5, 1024).contiguous()
+    ref = cp.coverprune_select(f, pos, fr, 12, cp.Params(sgs_mode=2, sot_eps=eps))
+    assert cp.coverprune_check(ref["ws"]) == cp.CP_OK
+    t0 = time.time()
+    for _ in range(3):
+        r = cp.coverprune_select(f, pos, fr, 12, cp.Params(sgs_mode=2, sot_eps=eps, timeout_ms=1e-6),
+                                 ws=ref["ws"])
+        assert cp.coverprune_check(r["ws"]) in (cp.CP_OK, cp.CP_ETIMEOUT)
+    assert time.time() - t0 < 5.0
+    r = cp.coverprune_select(f, pos, fr, 12, cp.Params(sgs_mode=2, sot_eps=eps), ws=ref["ws"])
+    assert cp.coverprune_check(r["ws"]) == cp.CP_OK
+    for k in ("kept", "order", "gains", "objective"):
+        assert torch.equal(r[k], ref[k]), k
