@@ -492,7 +492,9 @@ __global__ void __launch_bounds__(LS_THREADS, 1) k_lit_sinkhorn(const __grid_con
                    !(p >= 7.7037198e-34f || vj == 0.0f);
             g[j] = p;
             if (it == a.iters - 1) {
-              a.resid[gj] = fmaxf(vj - p * s, 0.0f);
+              // a column at its capacity leaves nothing (v - (v / s) s would
+              // leave its rounding)
+              a.resid[gj] = p < 1.0f ? 0.0f : fmaxf(vj - s, 0.0f);
               cap[j] = p > 0.0f ? a.eps * logf(p) : -INFINITY;  // the potential to carry on
             }
           }
@@ -514,9 +516,8 @@ __global__ void __launch_bounds__(LS_THREADS, 1) k_lit_sinkhorn(const __grid_con
             const float p = ev > -INFINITY ? fminf(0.0f, ev - lv) : -INFINITY;
             g[j] = p;
             if (it == a.iters - 1) {
-              const float sum =
-                  lv > -INFINITY && p > -INFINITY ? expf((p + lv) * a.inv_eps) : 0.0f;
-              a.resid[gj] = fmaxf(__ldg(a.v + gj) - sum, 0.0f);
+              const float sum = lv > -INFINITY ? expf(lv * a.inv_eps) : 0.0f;
+              a.resid[gj] = p < 0.0f ? 0.0f : fmaxf(__ldg(a.v + gj) - sum, 0.0f);
             }
           }
         }

@@ -451,6 +451,21 @@ def test_sgs_literal_forms(orc, N, D, K, g, eps, iters):
         assert res["picked_score"][l] - res["best_score"][l] <= 2 * tol * scale, l
 
 
+@pytest.mark.parametrize("eps", [0.05, 1e-3])  # the factors; the potentials
+def test_sgs_literal_saturated_columns_leave_nothing(orc, eps):
+    """A target at its capacity has no residual, so a candidate whose whole
+    neighbourhood is served scores 0, not the rounding of v - (v / s) s."""
+    N, K, g, iters = 700, 70, 24, 20
+    s = scene("short_clip", 0, N=N, D=256)
+    sel, cst = _select_case(orc, s, K, cp.Params(g=g, sgs_mode=2, sot_eps=eps, sot_iters=iters))
+    res = orc.sgs_literal(host(cst["cost"]).astype(np.float64),
+                          host(cst["capacity"]).astype(np.float64), K, float(np.float32(eps)),
+                          iters, g, orc.knn_others(s["pos"], g - 1), forced=host(sel["order"]))
+    served = np.asarray(res["picked_score"]) < 1e-13  # nothing but the oracle's own rounding
+    assert served.sum() >= K // 4
+    assert np.all(host(sel["gains"])[served] == 0.0)
+
+
 @pytest.mark.parametrize("name,N,D,K,g,seed", [("long_video", 2000, 512, 200, 64, 3),
                                                ("short_clip", 1500, 256, 150, 24, 4),
                                                ("long_video", 777, 128, 60, 17, 5)])
