@@ -172,8 +172,10 @@ int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int
                     const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                     int32_t* order32, float* gains, double* objective, int* status,
                     cudaStream_t s, const float* g0, void* ws);
-// The fixed-point scale of the gains for a coverage cost m0 (sgs_gain.cuh).
+// The fixed-point scale of the gains while targets cost m0 at most, and once
+// every target is covered (sgs_gain.cuh).
 int gain_fx(float m0);
+int gain_fx_covered(const DevParams& P);
 // K5 as Sec. 3.5 prints it (sgs_mode 2): entropic semi-relaxed OT residual
 // and the residual-weighted local cost; needs the dense cost [B][N][ldc]
 // and sgs_literal_ws_bytes(B, N, K) bytes of scratch (256-byte aligned).

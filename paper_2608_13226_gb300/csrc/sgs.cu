@@ -37,11 +37,18 @@ int gain_fx(float m0) {
   return 130 + e < 64 ? 64 : 130 + e;
 }
 
+// A cost is at most the sum of its weights, up to rounding (which the scale's
+// spare bit takes).
+int gain_fx_covered(const DevParams& P) {
+  const float c = P.lambda_f + P.lambda_x + P.lambda_tau;
+  return gain_fx(c < P.m0 ? c : P.m0);
+}
+
 template <bool LOCAL>
 __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
     const float* __restrict__ cost, int64_t ldc, const float* __restrict__ slab,
     const int32_t* __restrict__ nbr, const float* __restrict__ v_all, DevParams P, int N, int K,
-    int cps, int scene0, int fx, int32_t* __restrict__ order32, float* __restrict__ gains,
+    int cps, int scene0, int fx, int fx1, int32_t* __restrict__ order32, float* __restrict__ gains,
     double* __restrict__ objective, unsigned long long* partials, uint32_t* counters,
     int* status) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -50,7 +57,7 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
   float* sm_v = sm_m + ncols;                                    // [ncols] capacity v_j
   uint32_t* chosen = reinterpret_cast<uint32_t*>(sm_v + ncols);  // [ceil(N/32)] bitset
   __shared__ unsigned long long s_best[SGS_WARPS];
-  __shared__ int s_pick, s_bad;
+  __shared__ int s_pick, s_bad, s_fx;
   __shared__ float s_gain;
 
   const int b = scene0 + blockIdx.x / cps;
@@ -75,7 +82,8 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
   bool alive = true;
   unsigned long long my_evals = 0ull;  // rows this warp evaluated (lane 0 counts)
   unsigned long long my_update_bytes = 0ull;  // coverage-update reads (thread 0 of block 0)
-  for (int step = 0; step < K && alive; ++step) {
+  uint32_t turn = 0;  // sweeps: one a step, one more where the scale is refitted
+  for (int step = 0; step < K && alive;) {
     unsigned long long best = 0ull;
     for (int t = gw; t < N; t += nw) {
       if (chosen[t >> 5] & (1u << (t & 31))) continue;
@@ -89,13 +97,14 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
     }
     if (lane == 0) s_best[w] = best;
     __syncthreads();
-    const int par = step & 1;
+    const int par = (int)(turn & 1u);
+    ++turn;
     if (threadIdx.x == 0) {
       unsigned long long m = s_best[0];
       for (int i = 1; i < SGS_WARPS; ++i) m = s_best[i] > m ? s_best[i] : m;
       part[((size_t)par * nscenes + (b - scene0)) * cps + c] = m;
     }
-    if (!grid_barrier(counters + b, (uint32_t)(step + 1) * (uint32_t)cps, status, P.timeout_ns)) {
+    if (!grid_barrier(counters + b, turn * (uint32_t)cps, status, P.timeout_ns)) {
       alive = false;
       break;
     }
@@ -114,6 +123,9 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
         s_gain = key_gain(m);
         // decided once, before anyone updates the state: a winner must be an
         // unselected token (never expected to fail)
+        s_fx = fx;
+        if (m != 0ull && (LOCAL || step > 0) && (uint32_t)(m >> 32) <= gain_floor(fx))
+          s_fx = gain_refit((uint32_t)(m >> 32) - 1u, fx, 32 - __clz(N));
         s_bad = m == 0ull || pk < 0 || pk >= N || (chosen[pk >> 5] & (1u << (pk & 31))) != 0u;
       }
     }
@@ -128,6 +140,11 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
       }
       alive = false;
       break;
+    }
+    if (s_fx != fx) {  // every block's answer is the same
+      fx = s_fx;
+      __syncthreads();  // before it is written again
+      continue;
     }
     if (threadIdx.x == 0) {
       chosen[pick >> 5] |= 1u << (pick & 31);
@@ -149,6 +166,8 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
         sm_m[j] = fminf(sm_m[j], srow[k]);
       }
     }
+    ++step;
+    fx = step == 1 ? fx1 : fx;
     __syncthreads();
   }
 
@@ -202,9 +221,11 @@ static int sgs_launch_impl(const float* cost, int64_t ldc, const float* slab, co
   for (int64_t b0 = 0; b0 < B; b0 += per_launch) {
     const int64_t nb = (B - b0) < per_launch ? (B - b0) : per_launch;
     int Ni = (int)N, Ki = (int)K, scene0 = (int)b0, fx = gain_fx(P.m0);
+    int fx1 = LOCAL ? fx : gain_fx_covered(P);  // from the second step on
     DevParams Pc = P;
     void* args[] = {(void*)&cost, (void*)&ldc, (void*)&slab, (void*)&nbr, (void*)&v, (void*)&Pc,
-                    (void*)&Ni, (void*)&Ki, (void*)&cps, (void*)&scene0, (void*)&fx, (void*)&order32,
+                    (void*)&Ni, (void*)&Ki, (void*)&cps, (void*)&scene0, (void*)&fx, (void*)&fx1,
+                    (void*)&order32,
                     (void*)&gains, (void*)&objective, (void*)&partials, (void*)&counters,
                     (void*)&status};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)fn, dim3((unsigned)(nb * cps)),

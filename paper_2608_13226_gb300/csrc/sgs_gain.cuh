@@ -4,13 +4,19 @@
 //
 // A term is v_j * max(m_j - C, 0) in fp32, each operation rounded once, and
 // the terms add up in 64-bit fixed point: term -> floor(term 2^S), with 2^S
-// chosen so that the largest possible gain (m0, as sum v = 1) stays below
-// 2^62.  Integer addition has no rounding and no order, so a gain is the
-// same number however it is computed: summed over a row, over a list, over
-// several blocks, or kept up to date by subtracting what a pick took away
-// from single terms.  Every term is non-increasing in m, so gains are
-// non-increasing too.  A term loses at most 2^-60 m0, far below the fp32
-// rounding of the term itself (2^-24 of it) for every term above 2^-36 m0.
+// chosen so that the largest possible gain stays below 2^62.  Integer
+// addition has no rounding and no order, so a gain is the same number however
+// it is computed: summed over a row, over a list, over several blocks, or
+// kept up to date by subtracting what a pick took away from single terms.
+// Every term is non-increasing in m, so gains are non-increasing too.
+//
+// The scale follows the gains, not m0, which may be any number: it starts
+// from m0 (sum v = 1), on the dense path from the largest cost once the first
+// pick has covered every target (fx in launch_sgs), and whenever the best
+// gain left is below 2^-24 of it, it is fitted to that gain and the gains are
+// summed afresh before the pick (gain_floor, gain_refit; at most 8 times in a
+// selection, as it falls by 2^24 or more each time).  A term loses at most
+// 2^-60 of the scale, so n terms 2^-36 n of the best gain.
 //
 // Decisions and recorded gains use the sum rounded to 24 bits, an fp32 number
 // (equal sums give equal numbers and larger sums never smaller ones); the
@@ -53,6 +59,18 @@ __device__ __forceinline__ uint32_t gain_bits(gain_t g, int fx) {
   if (g == 0ull) return 0u;
   const int lz = __clzll((long long)g);
   return ((uint32_t)(fx - lz - 1) << 23) + (((uint32_t)((g << lz) >> 39) + 1u) >> 1);
+}
+
+// The refit of the scale, a rule on the best gain left that every selection
+// kernel applies at the same step.  gain_floor: its 24 bits below which the
+// scale no longer fits; gain_refit: the scale that does.  Before their cut
+// the sums of up to 2^lgN terms are below that gain and 2^lgN units together.
+__device__ __forceinline__ uint32_t gain_floor(int fx) {
+  return fx > 64 ? (uint32_t)(fx - 27) << 23 : 0u;
+}
+__device__ __forceinline__ int gain_refit(uint32_t bits, int fx, int lgN) {
+  const int of_gain = bits ? (int)(bits >> 23) + 4 : 64, of_cut = fx - 60 + lgN;
+  return max(64, max(of_gain, of_cut));
 }
 
 // (gain, index) as one key: the largest gain wins, the lowest index among

@@ -372,15 +372,15 @@ struct PushArgs {
   uint32_t off_q, off_lo, off_hi;  // dynamic shared memory offsets
 };
 
-// One chunk of 32 list entries against a target lowered from mo to mn: the
-// gains of the live candidates lose what the drop took.  Gains are kept as
-// two 32-bit words (32-bit shared atomics are native): the low word's update
-// goes out first and `old` carries what it saw, so that chunk_high, called
-// once every chunk's low words are on their way, takes the borrow off the
-// high word; the pair is right once every update has run.
-__device__ __forceinline__ gain_t chunk_low(uint32_t* lo, uint32_t at, bool on, float v, float mo,
-                                            float mn, float c, int fx, uint32_t& old) {
-  const gain_t d = on ? gain_drop(v, mo, mn, c, fx) : 0ull;
+// One live candidate of a target lowered from mo to mn: its gain loses what
+// the drop took.  Gains are kept as two 32-bit words (32-bit shared atomics
+// are native): the low word's update goes out first and `old` carries what it
+// saw, so that chunk_high, called once the low words of all entries in flight
+// are on their way, takes the borrow off the high word; the pair is right once
+// every update has run.
+__device__ __forceinline__ gain_t chunk_low(uint32_t* lo, uint32_t at, float v, float mo, float mn,
+                                            float c, int fx, uint32_t& old) {
+  const gain_t d = gain_drop(v, mo, mn, c, fx);
   old = 0u;
   if (d != 0ull) old = atomicAdd(lo + at, 0u - (uint32_t)d);
   return d;
@@ -439,6 +439,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
   hw_cluster_sync();  // every block initialised before any peer writes to it
   const int lo0 = w << a.lgS, lo1 = min(nown, lo0 + (1 << a.lgS));  // this warp's candidates
 
+  const uint32_t low = gain_floor(fx);
   bool ok = true;
   int pref = -1;  // the row last prefetched
   int step = 1;
@@ -466,10 +467,11 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
       }
       const uint32_t mf = __reduce_max_sync(0xFFFFFFFFu, bf);
       const int mt = __reduce_min_sync(0xFFFFFFFFu, bf == mf ? bt : 0x7FFFFFFF);
-      if (lane == 0) s_key[w] = mf ? gain_key(mf - 1u, (mt << lgC) | rank) : 0ull;
+      if (lane == 0) s_key[w] = mf > low ? gain_key(mf - 1u, (mt << lgC) | rank) : 0ull;
     }
     __syncthreads();  // every warp's key is in
     gain_t W = 0ull;
+    int good = 1;
     if (a.C == 1 || w < 2) W = warp_max_key(lane < PUSH_WARPS ? s_key[lane] : 0ull);
     if (a.C > 1) {
       if (w == 0 && lane < a.C)
@@ -480,7 +482,6 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
         if (t != pref && lane == 0) prefetch_l2(R + (size_t)t * a.ldc, (uint32_t)(4 * a.ldc));
         pref = t;
       }
-      int good = 1;
       if (lane == 0 && !mbar_test(&s_bar[par], (uint32_t)((step - 1) >> 1) & 1u)) {
         const uint64_t t0 = globaltimer_ns();
         uint32_t spins = 0;
@@ -500,14 +501,10 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
       W = good ? warp_max_key(lane < a.C ? *(volatile gain_t*)&s_res[par][lane] : 0ull) : 0ull;
     }
     const int pick = W ? key_token(W) : -1;
-    if (pick < 0 || pick >= N) {  // never expected: no candidate left
-      if (lane == 0) s_fail = 1;
-      if (threadIdx.x == 0 && atomicCAS(a.status, 0, CP_EDEVICE) == 0) {
-        a.status[4] = step;
-        a.status[5] = b;
-        a.status[6] = rank;
-        a.status[7] = pick;
-      }
+    if (pick < 0) {
+      // no gain within the scale's reach: the rounds that follow fit it (or a
+      // wait that ran out)
+      if (lane == 0 && good) s_qn = -1;
     } else {
       if (rank == 0 && threadIdx.x == 0) {
         a.order32[(size_t)b * a.K + step] = pick;
@@ -552,12 +549,12 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
         }
       }
     }
-    last = pick;
     __syncthreads();  // the lowered targets are listed
-    if (s_fail) {     // block-uniform
-      ok = false;
+    if (s_fail != 0 || s_qn < 0) {  // block-uniform; this step is not taken
+      ok = s_fail == 0;
       break;
     }
+    last = pick;
     // ---- LW lanes per lowered target: its live candidates lose what the drop
     // took; the entries that stay live are packed to the list's front.  Four
     // entries a lane are in flight, and the next target's length and costs
@@ -595,7 +592,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
           x[u] = i0 + LW * u < lenc ? __ldcg(L + i0 + LW * u) : make_uint2(0u, 0x7F800000u);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          d[u] = chunk_low(g_lo, x[u].x, true, vc, mo, mnc, __uint_as_float(x[u].y), fx, old[u]);
+          d[u] = chunk_low(g_lo, x[u].x, vc, mo, mnc, __uint_as_float(x[u].y), fx, old[u]);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           chunk_high(g_hi, x[u].x, d[u], old[u]);
@@ -777,6 +774,34 @@ __device__ __forceinline__ void warps_sync(int n) {
   asm volatile("bar.sync 1, %0;" ::"r"(32 * n) : "memory");
 }
 
+// How far a gain of this key, and so any smaller one, can be shifted up
+// without reaching the sign.
+__device__ __forceinline__ int gains_shift(gain_t key, int fx) {
+  const uint32_t bits = (uint32_t)(key >> 32) - 1u;
+  return bits ? min(31, fx - 2 - (int)(bits >> 23)) : 31;
+}
+
+// The gains (all 0 before) from the lists, a warp per target.
+__device__ __noinline__ void sum_lists(const Entry* lists, const uint2* span, const float* v,
+                                       const float* m, int N, int S, int fx, uint32_t* g_lo,
+                                       uint32_t* g_hi) {
+#pragma unroll 1
+  for (int j = threadIdx.x >> 5; j < N; j += RD_WARPS) {
+    const uint2 sp = __ldcg(span + j);
+    const float vj = __ldg(v + j), mj = m[j];
+#pragma unroll 1
+    for (uint32_t i = threadIdx.x & 31; i < sp.y; i += 32) {
+      const Entry x = __ldcg(lists + sp.x + i);
+      const uint32_t at = (x.x & 31u) * (uint32_t)S + (x.x >> 5);
+      const gain_t d = gain_term(vj, mj, __uint_as_float(x.y), fx);
+      if (d == 0ull) continue;
+      const uint32_t old = atomicAdd(g_lo + at, (uint32_t)d);
+      const uint32_t dh = (uint32_t)(d >> 32) + (old > ~(uint32_t)d ? 1u : 0u);
+      if (dh) atomicAdd(g_hi + at, dh);
+    }
+  }
+}
+
 template <bool LOCAL>
 __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_constant__ RoundArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -803,11 +828,13 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
   __shared__ gain_t s_pkey[RD_MEMBERS];      // the picks' keys
   __shared__ gain_t s_best[RD_WARPS];
   __shared__ gain_t s_tau;                   // one more than the largest gain outside S can be (0: none)
+  __shared__ int s_fx;                       // the gains' scale (sgs_gain.cuh)
+  __shared__ int s_sh;                       // every gain left is below 2^(63 - sh)
   __shared__ int s_nm, s_ne, s_qn, s_np, s_cut, s_nv[2];
 
   const int bl = blockIdx.x, b = a.scene0 + bl;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int N = a.N, fx = a.fx, S = a.S;
+  const int N = a.N, S = a.S;
   const float* v = a.v + (size_t)b * N;
   const float* R = a.rows + (size_t)b * N * (LOCAL ? (size_t)a.g : (size_t)a.ldc);
   const int32_t* NB = LOCAL ? a.nbr + (size_t)b * N * a.kk : nullptr;
@@ -826,7 +853,11 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
   }
   for (int i = threadIdx.x; i < (N + 31) / 32; i += RD_THREADS) bits[i] = 0u;
   for (int i = threadIdx.x; i <= a.tmask; i += RD_THREADS) tab[i] = NO_RANK;
-  if (threadIdx.x == 0) s_np = 0;
+  if (threadIdx.x == 0) {
+    s_np = 0;
+    s_fx = a.fx;
+    s_sh = 0;
+  }
   __syncthreads();
 
   while (step < a.K) {
@@ -837,16 +868,23 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
       if ((t & 31) == w) g_hi[w * S + (t >> 5)] = 0xFFFFFFFFu;
     }
     __syncwarp();
-    // ---- the slice's best candidates, by their gains' high words with the
-    // place in the lane's run in the low 5 bits (negative: selected, or
-    // none): each lane its three best, then the warp's best of those heads
-    // in turn; a lane whose three are used up bounds its rest by the third
+    // ---- the slice's best candidates, by the 31 bits of their gains that
+    // start at the last picks' leading one (no gain left is above those) with
+    // the place in the lane's run in the low 5 (negative: selected, or none):
+    // each lane its three best, then the warp's best of those heads in turn;
+    // a lane whose three are used up bounds its rest by the third.  Fixed bits
+    // of the scale, ranked by before, did not tell late gains apart: rounds of
+    // a selection and ms, then / now, 4096 of 16384 tokens 972 / 534 and 29.3 /
+    // 15.0; 1229 of 8192 at m0 = 1000 1002 / 199 and 12.4 / 4.0; at the default
+    // m0 190 / 189 and 3.25 / 3.28 (the shift and the variable scale)
     int cnt = 0, left = -1;
     {
+      const int sh = s_sh;
       int v1 = -1, v2 = -1, v3 = -1;
 #pragma unroll 4
       for (int i = lane, q = 0; i < S; i += 32, ++q) {
-        const int x = (int)((g_hi[w * S + i] & 0xFFFFFFE0u) | (uint32_t)q);
+        const uint32_t top = __funnelshift_l(g_lo[w * S + i], g_hi[w * S + i], sh);
+        const int x = (int)((top & 0xFFFFFFE0u) | (uint32_t)q);
         v3 = max(v3, min(v2, x));
         v2 = max(v2, min(v1, x));
         v1 = max(v1, x);
@@ -881,23 +919,26 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
       s_tau = 0ull;
     }
     __syncthreads();  // every slice's bound is in
-    // ---- S: the slices' candidates above every high word left out
+    // ---- S: the slices' candidates above the leading bits of all left out
+    const int sh = s_sh;
     left = __reduce_max_sync(0xFFFFFFFFu, s_left[lane]);
     if (threadIdx.x == 0) {
       s_np = 0;
-      if (left >= 0) atomicMax(&s_tau, (gain_t)(left + 1) << 32);
+      if (left >= 0) atomicMax(&s_tau, (gain_t)(left + 1) << (32 - sh));
     }
     if (cnt > 0) {
       const int t = lane < cnt ? s_top[lane][w] : 0;
+      const uint32_t lo = lane < cnt ? g_lo[w * S + (t >> 5)] : 0u;
       const uint32_t hi = lane < cnt ? g_hi[w * S + (t >> 5)] : 0u;
-      const uint32_t in = __ballot_sync(0xFFFFFFFFu, lane < cnt && (int)hi > left);
+      const uint32_t in = __ballot_sync(
+          0xFFFFFFFFu, lane < cnt && (int)__funnelshift_l(lo, hi, sh) > left);
       if (in) {
         int i = 0;
         if (lane == 0) i = atomicAdd(&s_nm, __popc(in));
         i = __shfl_sync(0xFFFFFFFFu, i, 0) + lane;
         if ((in >> lane) & 1u) {  // in order, so lanes 0 .. popc - 1
           s_mtok[i] = t;
-          s_mlo[i] = g_lo[w * S + (t >> 5)];
+          s_mlo[i] = lo;
           s_mhi[i] = hi;
         }
       }
@@ -1001,6 +1042,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
     const int ne = min(s_ne, a.emax);
     const int nw = min(RD_WARPS, max(4, (ne + 31) / 32)), nt = 32 * nw;
     if (w < nw) {
+      const int fx = s_fx;
       // a thread's entries
       float ec[RD_EPT], em[RD_EPT];
       uint32_t ej[RD_EPT];
@@ -1013,8 +1055,9 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
         ec[u] = on ? __uint_as_float(x.y) : INFINITY;
         em[u] = on ? ent_m[e] : -INFINITY;  // m never falls below that
       }
-      // 24 bits of the largest gain outside S, + 1 (0: none)
-      const uint32_t out = s_tau ? gain_bits(s_tau - 1ull, fx) + 1u : 0u;
+      // 24 bits of the largest gain outside S, + 1 (0: none), or those from
+      // which on the scale fits
+      const uint32_t out = max(s_tau ? gain_bits(s_tau - 1ull, fx) + 1u : 0u, gain_floor(fx));
       const int mi = threadIdx.x;  // a thread's member (nt >= RD_MEMBERS)
       for (int it = 0;; ++it) {
         // the members' keys, of those whose 24 bits are above the bound
@@ -1100,8 +1143,8 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
           if (mj < em[u]) {
             const uint32_t i = ej[u] >> 16;
             uint32_t old;
-            const gain_t d = chunk_low(s_mlo, i, true, __ldg(v + (ej[u] & 0xFFFFu)), em[u],
-                                             mj, ec[u], fx, old);
+            const gain_t d = chunk_low(s_mlo, i, __ldg(v + (ej[u] & 0xFFFFu)), em[u], mj, ec[u], fx,
+                                       old);
             chunk_high(s_mhi, i, d, old);
             em[u] = mj;
           }
@@ -1120,6 +1163,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
         r += __shfl_xor_sync(0xFFFFFFFFu, r, 2);
         if ((lane & 3) == 0 && i < np) {
           a.order32[(size_t)b * a.K + step + r] = s_pick[i];
+          if (r == np - 1) s_sh = gains_shift(mine, fx);
           if (a.out_gains) a.out_gains[(size_t)b * a.K + step + r] = key_gain(mine);
         }
       }
@@ -1129,6 +1173,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
     int pick = -1, len = 0;
     if (np == 0) {
       // ---- no pick from S: the best candidate alone, by its exact key
+      const int fx = s_fx;
       gain_t best = 0ull;
 #pragma unroll 1
       for (int i = lane; i < S; i += 32) {
@@ -1152,8 +1197,24 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
         }
         return;
       }
+      if ((uint32_t)(best >> 32) <= gain_floor(fx)) {  // block-uniform
+        // ---- the scale no longer fits: the gains afresh at one that does,
+        // a warp per target's list
+        const int fit = gain_refit((uint32_t)(best >> 32) - 1u, fx, 32 - __clz(N));
+        for (int p = threadIdx.x; p < 32 * S; p += RD_THREADS)
+          if ((int)g_hi[p] >= 0) g_lo[p] = g_hi[p] = 0u;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          s_fx = fit;
+          s_sh = 0;
+        }
+        sum_lists(lists, span, v, sm_m, N, S, fit, g_lo, g_hi);
+        __syncthreads();
+        continue;
+      }
       len = LOCAL ? a.g : N;
       if (threadIdx.x == 0) {
+        s_sh = gains_shift(best, fx);
         a.order32[(size_t)b * a.K + step] = pick;
         if (a.out_gains) a.out_gains[(size_t)b * a.K + step] = key_gain(best);
         s_pick[0] = pick;
@@ -1189,6 +1250,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
       // lists a turn of the block, while lists are short (4 to 30 entries for
       // most of a selection), 16 while they are long
       const int qn = s_qn;
+      const int fx = s_fx;
       auto push = [&](auto width) {
         constexpr int W = decltype(width)::value;   // lanes a list
         constexpr int U = W == 16 ? 4 : 2;          // entries a lane has in flight
@@ -1217,8 +1279,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
 #pragma unroll
             for (int u = 0; u < U; ++u) {
               at[u] = (x[u].x & 31u) * (uint32_t)S + (x[u].x >> 5);
-              d[u] = chunk_low(g_lo, at[u], true, vj, mo, mn, __uint_as_float(x[u].y), fx,
-                                     old[u]);
+              d[u] = chunk_low(g_lo, at[u], vj, mo, mn, __uint_as_float(x[u].y), fx, old[u]);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -1400,14 +1461,17 @@ int launch_rounds(Fn fn, RoundArgs& a, int64_t scenes, const DeviceInfo& di, cud
 }
 
 int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
-                const float* v, const DevParams& P, int fx, int64_t B, int64_t N, int64_t K, int32_t* order32, float* gains, double* objective,
-                int* status, cudaStream_t s, const float* g0, void* ws) {
+                const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
+                int32_t* order32, float* gains, double* objective, int* status, cudaStream_t s,
+                const float* g0, void* ws) {
   DeviceInfo di;
   if (device_info(&di) != CP_OK) return CP_ECUDA;
   const bool local = P.g < N;
   const PushPlan pl = push_plan(B, N, P.g, ldc);
   unsigned char* base = static_cast<unsigned char*>(ws);
   gain_t* gains64 = reinterpret_cast<gain_t*>(base + pl.gains);
+  const int fx0 = gain_fx(P.m0);                    // uncovered targets cost m0,
+  const int fx = local ? fx0 : gain_fx_covered(P);  // covered ones no more than the largest cost
   RoundArgs r{};
   r.rows = local ? slab : cost;
   r.nbr = nbr;
@@ -1434,7 +1498,7 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
     CP_TRY_STATUS(last_launch_status());
     k_rev_scan<<<(unsigned)B, 1024, 0, s>>>((int)N, r.span);
     CP_TRY_STATUS(last_launch_status());
-    k_rev_fill<<<per_token, 256, 0, s>>>(slab, nbr, v, (int)N, P.g, P.kk, P.m0, fx, r.span,
+    k_rev_fill<<<per_token, 256, 0, s>>>(slab, nbr, v, (int)N, P.g, P.kk, P.m0, fx0, r.span,
                                          r.lists, gains64);
     CP_TRY_STATUS(last_launch_status());
     r.list_step = (size_t)N * (size_t)P.g;
@@ -1476,7 +1540,7 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
   }
   const int64_t groups = g0 ? (N + 255) / 256 : (N + 7) / 8;
   k_first_pick<<<dim3((unsigned)(groups < 512 ? groups : 512), (unsigned)B), 256, 0, s>>>(
-      cost, ldc, v, (int)N, P.m0, fx, sums, max_bits, first);
+      cost, ldc, v, (int)N, P.m0, fx0, sums, max_bits, first);
   CP_TRY_STATUS(last_launch_status());
   auto lists_fn = k_live_lists;
   if (cuda_status(cudaFuncSetAttribute(lists_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1535,10 +1599,11 @@ size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc) {
 }
 
 int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
-                    const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K, int32_t* order32, float* gains,
-                    double* objective, int* status, cudaStream_t s, const float* g0, void* ws) {
-  return launch_push(cost, ldc, slab, nbr, v, P, gain_fx(P.m0), B, N, K, order32, gains, objective,
-                     status, s, g0, ws);
+                    const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
+                    int32_t* order32, float* gains, double* objective, int* status,
+                    cudaStream_t s, const float* g0, void* ws) {
+  return launch_push(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains, objective, status, s, g0,
+                     ws);
 }
 
 }  // namespace cp

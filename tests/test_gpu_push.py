@@ -10,7 +10,7 @@ import pytest
 import torch
 
 import paper_2608_13226_gb300 as cp
-from gpu_util import batch_to_dev, scene
+from gpu_util import batch_to_dev, check_sgs_teacher_forced, scene
 
 pytestmark = pytest.mark.gpu
 
@@ -63,6 +63,23 @@ def test_push_scale_of_the_coverage_cost(m0, g):
     # relative 2^-23 a step of the sum, and N 2^-24 for the sum of v
     F = float(host(r["objective"])[0])
     assert abs((m0 - gains.sum()) - F) <= m0 * (700 * 2.0 ** -24 + 2.0 ** -20)
+
+
+@pytest.mark.parametrize("N,K,g", [(1500, 200, 0), (1500, 400, 24), (300, 300, 0)])
+@pytest.mark.parametrize("m0", [1e-3, 1e3, 1e6, 1e9, 1e12, 1e30])
+def test_push_coverage_cost_against_the_oracle(orc, m0, N, K, g):
+    """Whatever an uncovered token costs, the gains are those of the oracle's
+    greedy forced to the same picks, and each pick is its best one, within
+    the bars of the default m0; K = N runs the gains down to nothing."""
+    s = scene("long_video", 9, N=N, D=64)
+    f, pos, fr = batch_to_dev([s])
+    r = _same(f, pos, fr, K, g=g, m0=m0)
+    c = cp.coverprune_cost(f, pos, fr, cp.Params(g=g))
+    nbr = orc.knn_others(s["pos"], g - 1) if g else None
+    check_sgs_teacher_forced(orc, host(c["cost"])[0].astype(np.float64),
+                             host(c["capacity"])[0].astype(np.float64), host(r["order"])[0],
+                             host(r["gains"])[0], float(host(r["objective"])[0]),
+                             float(np.float32(m0)), g, nbr)
 
 
 @pytest.mark.parametrize("weights", [dict(lambda_f=0.0, lambda_x=0.0, lambda_tau=0.0),
