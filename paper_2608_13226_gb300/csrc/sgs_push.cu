@@ -1590,12 +1590,14 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
 
 }  // namespace
 
-// One size for every neighbourhood: a workspace of these sizes serves the
-// dense path and each local one.
+// A local selection's own lists; where the dense ones are small (64 MB) room
+// for those, so that a program may try both on one workspace.
 size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc) {
   const size_t dense = push_plan(B, N, N, ldc).total;
-  const size_t local = g < N ? push_plan(B, N, g, ldc).total : 0;
-  return local > dense ? local : dense;
+  if (g >= N) return dense;
+  const size_t local = push_plan(B, N, g, ldc).total, small = (size_t)64 << 20;
+  const size_t either = dense < small ? dense : small;
+  return local > either ? local : either;
 }
 
 int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,

@@ -105,6 +105,20 @@ def test_workspace_sizes(lib):
         ws(cp.CP_OP_SELECT, 1, 100, 64, 10, lambda_f=float("nan"))
 
 
+@pytest.mark.parametrize("B,N,D,K,g,norm_mode", [(32, 8192, 3584, 1229, 64, 0),
+                                                 (32, 8192, 3584, 1229, 64, 1),
+                                                 (1, 16384, 256, 1638, 64, 0),
+                                                 (4, 6272, 1280, 628, 24, 1)])
+def test_local_workspace_holds_no_dense_lists(lib, B, N, D, K, g, norm_mode):
+    """The dense cost (or its cosines), the inputs in Morton order and about 40
+    bytes a neighbour pair, not the 16 N bytes a token of the dense lists."""
+    n = cp.coverprune_workspace_size(cp.CP_OP_SELECT, B, N, D, K, cp.CP_BF16,
+                                     cp.Params(g=g, norm_mode=norm_mode))
+    cost = 4 * B * N * N + (2 * B * N * D if norm_mode else 0)
+    # a token's partial sums of first gains take 4 N / 64 bytes
+    assert n <= 1.02 * cost + B * N * (40 * g + N / 16 + 256) + (64 << 20)
+
+
 def _select(lib, p, B=1, N=100, D=64, K=10, dt=cp.CP_BF16, feats=FAKE, kept=FAKE, ws=FAKE,
             ws_bytes=1 << 40):
     return lib.coverprune_select(C.c_void_p(feats), dt, C.c_void_p(FAKE), C.c_void_p(FAKE), B, N,
