@@ -18,9 +18,10 @@
  * ---------------------------------------
  *  - Pointers are DEVICE pointers owned by the caller unless a comment says
  *    otherwise.  The library never allocates device memory and never frees
- *    what it is given.  Scratch memory is the caller's workspace `ws` of at
- *    least coverprune_workspace_size() bytes, 256-byte aligned; it must not
- *    be used by anything else until the stream has passed the call.
+ *    what it is given.  Scratch memory is the caller's workspace `ws`, best of
+ *    coverprune_workspace_size() bytes and of coverprune_workspace_least() at
+ *    least, 256-byte aligned; it must not be used by anything else until the
+ *    stream has passed the call.
  *  - Work is enqueued on `stream` (0 = legacy default stream) and the call
  *    returns without synchronising.  Outputs are valid once the stream has
  *    reached the call.
@@ -177,11 +178,25 @@ void cp_default_params(cp_params* p);
  * (0, 1]), clamped to [1, N].  Returns -1 if R is not in (0, 1] or N < 1. */
 int64_t coverprune_budget(double R, int64_t N);
 
-/* Bytes of workspace that entry point `op` needs for these sizes; written to
- * *bytes.  Returns CP_OK or CP_EINVAL/CP_EUNSUPPORTED for sizes the entry
- * point would reject.  Host only; touches no device. */
+/* Bytes of workspace that entry point `op` works best with for these sizes;
+ * written to *bytes.  Returns CP_OK or CP_EINVAL/CP_EUNSUPPORTED for sizes the
+ * entry point would reject.  Host only; touches no device.
+ *   A selection holds the dense cost, 4 N^2 bytes a scene.  The default dense
+ * one (sgs_mode 0, every token a neighbour) also holds lists, up to 8 N^2
+ * bytes a scene for as many scenes at a time as fit 24 GB; a larger workspace
+ * is of no use to it.  It runs in less, see coverprune_workspace_least. */
 int coverprune_workspace_size(int op, int64_t B, int64_t N, int64_t D, int64_t K,
                               int dtype, const cp_params* p, size_t* bytes);
+
+/* The least workspace that entry point `op` runs in: the same as
+ * coverprune_workspace_size except for a selection with sgs_mode 0, whose
+ * lists may be held for one scene at a time.  The results do not depend on the
+ * size.  Between the two, a batch takes as many scenes at a time as fit; 32
+ * scenes of 8192 tokens, 1229 kept: 16.6 ms in 28.1 GB, 20.2 in 22.2, 21.6 in
+ * 16.9, 29.1 in 12.6, 96 in 9.4.  Any workspace of the least size for more
+ * scenes will do. */
+int coverprune_workspace_least(int op, int64_t B, int64_t N, int64_t D, int64_t K,
+                               int dtype, const cp_params* p, size_t* bytes);
 
 /* Static string for a cp_status value ("unknown status" otherwise). */
 const char* coverprune_status_string(int status);

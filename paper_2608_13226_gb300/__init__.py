@@ -12,7 +12,7 @@ from .binding import (CP_BF16, CP_EINVAL, CP_ETIMEOUT, CP_EUNSUPPORTED, CP_EWORK
                       coverprune_cost, coverprune_gather, coverprune_knn, coverprune_knn_noalloc,
                       coverprune_lite_select,
                       coverprune_select, coverprune_version, coverprune_workspace_size,
-                      library_path, load, status_string, workspace, coverprune_profile_enable,
+                      coverprune_workspace_least, library_path, load, status_string, workspace, coverprune_profile_enable,
                       coverprune_profile_read, STAGES)
 
 __all__ = [n for n in dir() if not n.startswith("_")]

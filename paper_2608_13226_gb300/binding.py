@@ -22,6 +22,7 @@ CP_OP_COST, CP_OP_SELECT, CP_OP_LITE, CP_OP_KNN = 0, 1, 2, 3
 
 # every symbol declared in include/coverprune.h
 EXPORTS = ("cp_default_params", "coverprune_budget", "coverprune_workspace_size",
+           "coverprune_workspace_least",
            "coverprune_status_string", "coverprune_check", "coverprune_cost",
            "coverprune_select", "coverprune_lite_select", "coverprune_knn",
            "coverprune_knn_noalloc",
@@ -126,6 +127,7 @@ def _lib():
         lib.coverprune_budget.restype = I64
         lib.coverprune_workspace_size.argtypes = [I32, I64, I64, I64, I64, I32, PP,
                                                   C.POINTER(C.c_size_t)]
+        lib.coverprune_workspace_least.argtypes = lib.coverprune_workspace_size.argtypes
         lib.coverprune_status_string.argtypes = [I32]
         lib.coverprune_status_string.restype = C.c_char_p
         lib.coverprune_check.argtypes = [P, P]
@@ -210,15 +212,38 @@ def coverprune_workspace_size(op: int, B: int, N: int, D: int, K: int, dtype: in
     return int(out.value)
 
 
+def coverprune_workspace_least(op: int, B: int, N: int, D: int, K: int, dtype: int,
+                               params: Params | None = None) -> int:
+    p = (params or Params())._c()
+    out = C.c_size_t()
+    _check(_lib().coverprune_workspace_least(op, B, N, D, K, dtype, C.byref(p), C.byref(out)),
+           "coverprune_workspace_least")
+    return int(out.value)
+
+
 def workspace(op: int, B: int, N: int, D: int, K: int, dtype: int,
               params: Params | None = None, device=None) -> torch.Tensor:
     n = coverprune_workspace_size(op, B, N, D, K, dtype, params)
     return torch.empty(max(n, 256), dtype=torch.uint8, device=device or "cuda")
 
 
+def _room(op, B, N, D, K, dt, params, device):
+    """A workspace of the best size, or the largest half, quarter, ... of it
+    that the device has room for, down to the least the call runs in."""
+    n = coverprune_workspace_size(op, B, N, D, K, dt, params)
+    least = coverprune_workspace_least(op, B, N, D, K, dt, params)
+    while True:
+        try:
+            return torch.empty(max(n, 256), dtype=torch.uint8, device=device)
+        except torch.cuda.OutOfMemoryError:
+            if n <= least:
+                raise
+            n = max(least, n // 2)
+
+
 def _ws(ws, op, B, N, D, K, dt, params, device):
     if ws is None:
-        ws = workspace(op, B, N, D, K, dt, params, device)
+        ws = _room(op, B, N, D, K, dt, params, device)
     if ws.data_ptr() % 256:
         raise ValueError("workspace must be 256-byte aligned")
     return ws

@@ -195,6 +195,7 @@ struct Plan {
   size_t perm, gs, proto, score;                  // lite
   size_t total;
   int64_t ldc;
+  int64_t wave;  // default selection: scenes whose dense lists are held at once (0: the most)
 };
 
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -217,8 +218,9 @@ static bool local_tiles_path(int op, int dtype, int64_t N, const DevParams& d) {
 }
 
 static void plan_ws(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtype,
-                    const DevParams& d, Plan* pl) {
+                    const DevParams& d, Plan* pl, int64_t wave = 0) {
   memset(pl, 0, sizeof(*pl));
+  pl->wave = wave;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     size_t at = off;
@@ -245,7 +247,7 @@ static void plan_ws(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtyp
     pl->cost = take(sizeof(float) * BN * (size_t)pl->ldc);
     if (d.sgs_mode == 2) pl->lit = take(sgs_literal_ws_bytes(B, N, K));
     if (d.g < N && d.sgs_mode != 2) pl->slab = take(sizeof(float) * BN * (size_t)d.g);
-    if (d.sgs_mode == 0) pl->push = take(sgs_push_ws_bytes(B, N, d.g, pl->ldc));
+    if (d.sgs_mode == 0) pl->push = take(sgs_push_ws_bytes(B, N, d.g, wave));
     if (local_tiles_path(op, dtype, N, d)) {
       const size_t T = (size_t)local_tiles(N);
       pl->lfeats = take(2 * BN * (size_t)D);
@@ -342,8 +344,20 @@ static int check_inputs(const void* feats, const float* pos, const int32_t* fram
 
 static int check_ws(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtype,
                     const DevParams& d, void* ws, size_t ws_bytes, Plan* pl) {
+  if (!ws || !aligned(ws, 256)) return CP_EWORKSPACE;
   plan_ws(op, B, N, D, K, dtype, d, pl);
-  if (!ws || !aligned(ws, 256) || ws_bytes < pl->total) return CP_EWORKSPACE;
+  if (ws_bytes >= pl->total) return CP_OK;
+  if (op != CP_OP_SELECT || d.sgs_mode != 0) return CP_EWORKSPACE;
+  // fewer scenes' lists at once, the most that fit
+  plan_ws(op, B, N, D, K, dtype, d, pl, 1);
+  if (ws_bytes < pl->total) return CP_EWORKSPACE;
+  int64_t fits = 1, over = sgs_push_wave(B, N) + 1;
+  while (over - fits > 1) {
+    const int64_t wave = (fits + over) / 2;
+    plan_ws(op, B, N, D, K, dtype, d, pl, wave);
+    (ws_bytes >= pl->total ? fits : over) = wave;
+  }
+  plan_ws(op, B, N, D, K, dtype, d, pl, fits);
   return CP_OK;
 }
 
@@ -405,8 +419,8 @@ int coverprune_version(void) { return 100; }
 
 const char* coverprune_last_error(void) { return t_last_error; }
 
-int coverprune_workspace_size(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtype,
-                              const cp_params* p, size_t* bytes) {
+static int workspace_bytes(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtype,
+                           const cp_params* p, size_t* bytes, int64_t wave) {
   if (!bytes) return CP_EINVAL;
   CP_TRY(check_params(p));
   if (op != CP_OP_COST && op != CP_OP_SELECT && op != CP_OP_LITE && op != CP_OP_KNN)
@@ -420,9 +434,19 @@ int coverprune_workspace_size(int op, int64_t B, int64_t N, int64_t D, int64_t K
   DevParams d = dev_params(p, N);
   CP_TRY(check_limits(op, N, d));
   Plan pl;
-  plan_ws(op, B, N, D, op == CP_OP_COST ? 0 : K, dtype, d, &pl);
+  plan_ws(op, B, N, D, op == CP_OP_COST ? 0 : K, dtype, d, &pl, wave);
   *bytes = pl.total;
   return CP_OK;
+}
+
+int coverprune_workspace_size(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtype,
+                              const cp_params* p, size_t* bytes) {
+  return workspace_bytes(op, B, N, D, K, dtype, p, bytes, 0);
+}
+
+int coverprune_workspace_least(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtype,
+                               const cp_params* p, size_t* bytes) {
+  return workspace_bytes(op, B, N, D, K, dtype, p, bytes, 1);
 }
 
 int coverprune_check(const void* ws, cp_stream_t stream) {
@@ -564,7 +588,7 @@ int coverprune_select(const void* feats, int dtype, const float* pos, const int3
     else
       CP_TRY(launch_sgs(C, pl.ldc, slab, nbr, v, d, B, N, K, order32, gains, objective,
                         at<uint64_t>(ws, pl.partials), at<uint32_t>(ws, pl.counters), status, s,
-                        g0, at<void>(ws, pl.push)));
+                        g0, at<void>(ws, pl.push), pl.wave));
   }
   Stage st(CP_STAGE_OUTPUT, s);
   CP_TRY(launch_sort_kept(order32, B, K, kept, order, s));

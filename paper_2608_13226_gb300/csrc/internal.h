@@ -164,14 +164,18 @@ int fst_apply_slots(int64_t ldc);
 int launch_sgs(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
                const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                int32_t* order32, float* gains, double* objective, uint64_t* partials,
-               uint32_t* counters, int* status, cudaStream_t s, const float* g0, void* push_ws);
+               uint32_t* counters, int* status, cudaStream_t s, const float* g0, void* push_ws,
+               int64_t push_wave);
 // sgs_mode 0: exact gains kept up to date over lists of live candidates.  g0
 // (dense, may be null): the cost pass's partial sums of the first gains.
-size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc);
+// wave: scenes whose dense lists are held at once, at most sgs_push_wave; 0:
+// that many, and for a small local selection the dense lists' room as well.
+int64_t sgs_push_wave(int64_t B, int64_t N);
+size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t wave);
 int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
                     const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                     int32_t* order32, float* gains, double* objective, int* status,
-                    cudaStream_t s, const float* g0, void* ws);
+                    cudaStream_t s, const float* g0, void* ws, int64_t wave);
 // The fixed-point scale of the gains while targets cost m0 at most, and once
 // every target is covered (sgs_gain.cuh).
 int gain_fx(float m0);

@@ -239,10 +239,11 @@ static int sgs_launch_impl(const float* cost, int64_t ldc, const float* slab, co
 int launch_sgs(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
                const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                int32_t* order32, float* gains, double* objective, uint64_t* partials,
-               uint32_t* counters, int* status, cudaStream_t s, const float* g0, void* push_ws) {
+               uint32_t* counters, int* status, cudaStream_t s, const float* g0, void* push_ws,
+               int64_t push_wave) {
   if (P.sgs_mode == 0)
     return launch_sgs_push(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains, objective, status,
-                           s, g0, push_ws);
+                           s, g0, push_ws, push_wave);
   auto* part = reinterpret_cast<unsigned long long*>(partials);
   if (P.g < N)
     return sgs_launch_impl<true>(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains, objective,

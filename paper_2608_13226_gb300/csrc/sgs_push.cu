@@ -1324,12 +1324,11 @@ size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 // Scenes whose lists are held at once.  A dense scene's lists take 8 N^2
 // bytes at their largest (twice its cost), its joined lists and rows up to
 // 16 RD_ROW N more, so a large batch runs in waves: as many scenes as fit 24
-// GB less a twelfth of the whole cost, at least one (entries are then
-// numbered in 32 bits).
-int64_t push_wave(int64_t B, int64_t N, int64_t ldc) {
+// GB (entries are then numbered in 32 bits), whatever the batch, so that no
+// larger batch needs less; at least one.
+int64_t push_wave(int64_t B, int64_t N) {
   const double per = 8.0 * (double)N * (double)(N + PUSH_CMAX + 2 * row_room(N));
-  const double room = 24.0e9 - 4.0 * (double)B * (double)N * (double)ldc / 12.0;
-  const int64_t w = room > per ? (int64_t)(room / per) : 1;
+  const int64_t w = 24.0e9 > per ? (int64_t)(24.0e9 / per) : 1;
   return w < B ? w : B;
 }
 
@@ -1339,7 +1338,8 @@ struct PushPlan {
   size_t join0;  // dense: entries before the joined lists
   int64_t wave;
 };
-PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t ldc) {
+// wave > 0: that many scenes' dense lists at once.
+PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t wave) {
   PushPlan p{};
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -1358,7 +1358,7 @@ PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t ldc) {
     p.max_bits = take(sizeof(uint32_t) * (size_t)B);
     p.zero_bytes = off;
     p.sums = take(sizeof(float) * BN);
-    p.wave = push_wave(B, N, ldc);
+    p.wave = wave > 0 ? wave : push_wave(B, N);
     const size_t WN = (size_t)p.wave * (size_t)N;
     p.lens = take(sizeof(uint32_t) * WN * PUSH_CMAX);
     p.join0 = WN * (size_t)(N + PUSH_CMAX);
@@ -1463,11 +1463,11 @@ int launch_rounds(Fn fn, RoundArgs& a, int64_t scenes, const DeviceInfo& di, cud
 int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
                 const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                 int32_t* order32, float* gains, double* objective, int* status, cudaStream_t s,
-                const float* g0, void* ws) {
+                const float* g0, void* ws, int64_t wave) {
   DeviceInfo di;
   if (device_info(&di) != CP_OK) return CP_ECUDA;
   const bool local = P.g < N;
-  const PushPlan pl = push_plan(B, N, P.g, ldc);
+  const PushPlan pl = push_plan(B, N, P.g, wave);
   unsigned char* base = static_cast<unsigned char*>(ws);
   gain_t* gains64 = reinterpret_cast<gain_t*>(base + pl.gains);
   const int fx0 = gain_fx(P.m0);                    // uncovered targets cost m0,
@@ -1590,12 +1590,15 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
 
 }  // namespace
 
+int64_t sgs_push_wave(int64_t B, int64_t N) { return push_wave(B, N); }
+
 // A local selection's own lists; where the dense ones are small (64 MB) room
 // for those, so that a program may try both on one workspace.
-size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc) {
-  const size_t dense = push_plan(B, N, N, ldc).total;
+size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t wave) {
+  if (wave > 0) return push_plan(B, N, g, wave).total;
+  const size_t dense = push_plan(B, N, N, 0).total;
   if (g >= N) return dense;
-  const size_t local = push_plan(B, N, g, ldc).total, small = (size_t)64 << 20;
+  const size_t local = push_plan(B, N, g, 0).total, small = (size_t)64 << 20;
   const size_t either = dense < small ? dense : small;
   return local > either ? local : either;
 }
@@ -1603,9 +1606,9 @@ size_t sgs_push_ws_bytes(int64_t B, int64_t N, int64_t g, int64_t ldc) {
 int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
                     const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                     int32_t* order32, float* gains, double* objective, int* status,
-                    cudaStream_t s, const float* g0, void* ws) {
+                    cudaStream_t s, const float* g0, void* ws, int64_t wave) {
   return launch_push(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains, objective, status, s, g0,
-                     ws);
+                     ws, wave);
 }
 
 }  // namespace cp

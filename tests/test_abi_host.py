@@ -105,6 +105,26 @@ def test_workspace_sizes(lib):
         ws(cp.CP_OP_SELECT, 1, 100, 64, 10, lambda_f=float("nan"))
 
 
+@pytest.mark.parametrize("g", [0, 64])
+@pytest.mark.parametrize("N", [1000, 8192, 12288, 16384])
+def test_workspace_serves_every_smaller_batch(lib, N, g):
+    """A program sizes one workspace for its largest batch: a size does not
+    fall as the batch grows (the dense lists' waves among it), and the least
+    workspace of a batch is within that of any larger one."""
+    prm = cp.Params(g=g)
+    size = [cp.coverprune_workspace_size(cp.CP_OP_SELECT, B, N, 256, 100, cp.CP_BF16, prm)
+            for B in range(1, 110)]
+    least = [cp.coverprune_workspace_least(cp.CP_OP_SELECT, B, N, 256, 100, cp.CP_BF16, prm)
+             for B in range(1, 110)]
+    assert all(a <= b for a, b in zip(size, size[1:]))
+    assert all(a <= b for a, b in zip(least, least[1:]))
+    assert all(a <= b for a, b in zip(least, size))
+    # one scene's lists beside the cost, not the whole batch's
+    assert least[99] <= 1.03 * 4 * 100 * N * N + 100 * N * (256 + 40 * g + N / 16) + 13 * N * N
+    assert least[0] <= cp.coverprune_workspace_least(cp.CP_OP_SELECT, 1, N + 1 if N < 16384 else N,
+                                                     256, 100, cp.CP_BF16, prm)
+
+
 @pytest.mark.parametrize("B,N,D,K,g,norm_mode", [(32, 8192, 3584, 1229, 64, 0),
                                                  (32, 8192, 3584, 1229, 64, 1),
                                                  (1, 16384, 256, 1638, 64, 0),

@@ -97,6 +97,29 @@ def test_push_ties(weights):
         assert host(r["order"])[0].tolist() == list(range(250))
 
 
+@pytest.mark.parametrize("g", [0, 20])
+def test_push_in_the_least_workspace(g):
+    """Any workspace from the least size on gives the same results; one byte
+    less is refused."""
+    B, N, D, K = 7, 1025, 64, 120
+    scs = [scene("long_video", sd, N=N, D=D) for sd in range(B)]
+    f, pos, fr = batch_to_dev(scs)
+    prm = cp.Params(g=g)
+    ref = cp.coverprune_select(f, pos, fr, K, prm)
+    size = cp.coverprune_workspace_size(cp.CP_OP_SELECT, B, N, D, K, cp.CP_BF16, prm)
+    least = cp.coverprune_workspace_least(cp.CP_OP_SELECT, B, N, D, K, cp.CP_BF16, prm)
+    assert least < size
+    for n in (least, (least + size) // 2, size - 1):
+        ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+        a = cp.coverprune_select(f, pos, fr, K, prm, ws=ws)
+        assert cp.coverprune_check(ws) == cp.CP_OK
+        for k in ("kept", "order", "gains", "objective"):
+            assert torch.equal(a[k], ref[k]), (n, k)
+    with pytest.raises(cp.CoverPruneError) as e:
+        cp.coverprune_select(f, pos, fr, K, prm, ws=ws[:least - 1])
+    assert e.value.status == cp.CP_EWORKSPACE
+
+
 def test_push_batch_in_waves():
     """A batch whose lists exceed the bound on them runs in waves of scenes:
     every scene equals the same scene alone."""
