@@ -112,6 +112,17 @@ int device_info(DeviceInfo* out) {
   return CP_OK;
 }
 
+int allow_smem(const void* fn, size_t smem, const char* where) {
+  if (smem <= 40 * 1024) return CP_OK;  // within the default limit of 48 KB, the static part too
+  DeviceInfo di;
+  cudaFuncAttributes fa;
+  if (device_info(&di) != CP_OK) return CP_ECUDA;
+  CP_TRY_STATUS(cuda_status(cudaFuncGetAttributes(&fa, fn), where));
+  return cuda_status(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          di.max_smem_optin - (int)fa.sharedSizeBytes),
+                     where);
+}
+
 // bf16 features: tcgen05 tensor cores; fp32 features: fp32 FMA tiles (TF32
 // would round the features to 10 mantissa bits).  cos_out (may be null):
 // every cosine (bf16) or dot product (fp32) of a pair i <= j stored

@@ -88,6 +88,12 @@ struct DeviceInfo {
 };
 int device_info(DeviceInfo* out);
 
+// Lets kernel `fn` take `smem` bytes of dynamic shared memory.  The limit is
+// the kernel's, not the launch's, and is set to all that the device has beside
+// the kernel's static part, so that a call with fewer tokens on another host
+// thread does not lower it between here and the launch.
+int allow_smem(const void* fn, size_t smem, const char* where);
+
 // ---------------------------------------------------------------------------
 // Launchers (each returns a cp_status; all enqueue on `s`).
 // ---------------------------------------------------------------------------

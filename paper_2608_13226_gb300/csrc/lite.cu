@@ -149,11 +149,7 @@ int launch_morton(const float* pos, const SceneStats* stats, const DevParams& P,
                   int32_t* perm, cudaStream_t s) {
   const int Np = (int)((N + 7) & ~(int64_t)7);
   const size_t smem = 12 * (size_t)Np + sizeof(uint16_t) * MT_WARPS * MT_BINS;
-  if (smem > 40 * 1024 &&
-      cuda_status(cudaFuncSetAttribute(k_morton, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem),
-                  "launch_morton: smem attribute") != CP_OK)
-    return CP_ECUDA;
+  CP_TRY_STATUS(allow_smem((const void*)k_morton, smem, "launch_morton: smem attribute"));
   k_morton<<<(unsigned)B, 32 * MT_WARPS, smem, s>>>(pos, stats, P.voxel, (int)N, Np, perm);
   return last_launch_status();
 }
@@ -277,11 +273,7 @@ __global__ void __launch_bounds__(1024) k_groups(const float* __restrict__ v_all
 int launch_groups(const float* v, const int32_t* perm, int64_t B, int64_t N, int64_t K,
                   int32_t* gs, cudaStream_t s) {
   const size_t smem = sizeof(unsigned long long) * (size_t)N;
-  if (smem > 40 * 1024 &&
-      cuda_status(cudaFuncSetAttribute(k_groups, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem),
-                  "launch_groups: smem attribute") != CP_OK)
-    return CP_ECUDA;
+  CP_TRY_STATUS(allow_smem((const void*)k_groups, smem, "launch_groups: smem attribute"));
   k_groups<<<(unsigned)B, 1024, smem, s>>>(v, perm, (int)N, (int)K, gs);
   return last_launch_status();
 }

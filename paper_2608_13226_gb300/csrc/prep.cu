@@ -432,11 +432,7 @@ int launch_knn(const float* pos, const float4* tok, int64_t B, int64_t N, int kk
   while (list_len < kk) list_len <<= 1;
   if (list_len < 2) list_len = 2;
   const size_t smem = sizeof(unsigned long long) * list_len + sizeof(uint32_t) * (size_t)N;
-  if (smem > 48 * 1024 &&
-      cuda_status(cudaFuncSetAttribute(k_knn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem),
-                  "launch_knn: smem attribute") != CP_OK)
-    return CP_ECUDA;
+  CP_TRY_STATUS(allow_smem((const void*)k_knn, smem, "launch_knn: smem attribute"));
   dim3 grid((unsigned)N, (unsigned)B);
   k_knn<<<grid, KNN_THREADS, smem, s>>>(pos, (int)N, kk, list_len, nbr, stats);
   return last_launch_status();
@@ -1127,14 +1123,8 @@ int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr
   const int gmax = grid_cells_max(N);
   if (kk > kKnnGridMax || (kk > 0 && kk >= N)) return CP_EINVAL;  // the search needs kk others
   const size_t smem = sizeof(int) * (size_t)(gmax + 1);
-  if (smem > 40 * 1024 &&  // beside ~1 KB of static shared memory
-      (cuda_status(cudaFuncSetAttribute(k_grid_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem),
-                   "launch_knn_grid: smem attribute") != CP_OK ||
-       cuda_status(cudaFuncSetAttribute(k_diameter_grid,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                   "launch_knn_grid: smem attribute") != CP_OK))
-    return CP_ECUDA;
+  CP_TRY_STATUS(allow_smem((const void*)k_grid_build, smem, "launch_knn_grid: smem attribute"));
+  CP_TRY_STATUS(allow_smem((const void*)k_diameter_grid, smem, "launch_knn_grid: smem attribute"));
   k_grid_build<<<(unsigned)B, 1024, smem, s>>>(pos, (int)N, gmax, info, cell_start, sorted);
   CP_TRY_STATUS(last_launch_status());
   k_diameter_grid<<<dim3(DIA_PARTS, (unsigned)B), DIA_THREADS, smem, s>>>((int)N, gmax, info,

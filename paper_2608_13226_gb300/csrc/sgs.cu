@@ -195,10 +195,7 @@ static int sgs_launch_impl(const float* cost, int64_t ldc, const float* slab, co
   const int64_t ncols = LOCAL ? N : ldc;
   const size_t smem = 2 * sizeof(float) * (size_t)ncols + sizeof(uint32_t) * (size_t)((N + 31) / 32);
   auto fn = k_sgs<LOCAL>;
-  if (smem > 48 * 1024 &&
-      cuda_status(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                  "launch_sgs: smem attribute") != CP_OK)
-    return CP_ECUDA;
+  CP_TRY_STATUS(allow_smem((const void*)fn, smem, "launch_sgs: smem attribute"));
   int per_sm = 0;
   if (cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, SGS_THREADS, smem),
                   "launch_sgs: occupancy") != CP_OK)
@@ -315,11 +312,7 @@ int launch_sort_kept(const int32_t* idx32, int64_t B, int64_t K, int64_t* kept, 
   int L = 2;
   while (L < K) L <<= 1;
   const size_t smem = sizeof(int32_t) * (size_t)L;
-  if (smem > 48 * 1024 &&
-      cuda_status(cudaFuncSetAttribute(k_sort_kept, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem),
-                  "launch_sort_kept: smem attribute") != CP_OK)
-    return CP_ECUDA;
+  CP_TRY_STATUS(allow_smem((const void*)k_sort_kept, smem, "launch_sort_kept: smem attribute"));
   k_sort_kept<<<(unsigned)B, 1024, smem, s>>>(idx32, (int)K, L, kept, order64);
   return last_launch_status();
 }

@@ -781,11 +781,7 @@ int launch_sgs_literal(const float* cost, int64_t ldc, const int32_t* nbr, const
     CP_TRY_STATUS(last_launch_status());
   }
   const size_t smem = sizeof(float) * (size_t)N;
-  if (smem > 48 * 1024 &&
-      cuda_status(cudaFuncSetAttribute(k_lit_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem),
-                  "launch_sgs_literal: smem attribute") != CP_OK)
-    return CP_ECUDA;
+  CP_TRY_STATUS(allow_smem((const void*)k_lit_finish, smem, "launch_sgs_literal: smem attribute"));
   k_lit_finish<<<(unsigned)B, 1024, smem, s>>>(cost, ldc, n, k, g, kk, nbr, v, keys, P.m0,
                                                order32, gains, objective);
   return last_launch_status();

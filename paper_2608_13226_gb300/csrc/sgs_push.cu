@@ -1400,10 +1400,7 @@ int push_config(Fn fn, PushArgs& a, int C0, int64_t scenes, const DeviceInfo& di
   for (int C = C0; C >= 1; C >>= 1) {
     const size_t smem = push_shape(a, C, a.ldc);
     if (smem + 2048 > (size_t)di.max_smem_optin) continue;
-    if (cuda_status(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem),
-                    "launch_sgs_push: smem attribute") != CP_OK)
-      return CP_ECUDA;
+    CP_TRY_STATUS(allow_smem((const void*)fn, smem, "launch_sgs_push: smem attribute"));
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3((unsigned)(scenes * C));
     cfg->blockDim = dim3(PUSH_THREADS);
@@ -1453,9 +1450,7 @@ int launch_rounds(Fn fn, RoundArgs& a, int64_t scenes, const DeviceInfo& di, cud
     if (smem + 7168 <= (size_t)di.max_smem_optin) break;
     if (a.emax <= 256) return CP_EUNSUPPORTED;
   }
-  CP_TRY_STATUS(cuda_status(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem),
-                            "launch_sgs_push: rounds smem attribute"));
+  CP_TRY_STATUS(allow_smem((const void*)fn, smem, "launch_sgs_push: rounds smem attribute"));
   fn<<<(unsigned)scenes, RD_THREADS, smem, s>>>(a);
   return launch_status("launch_sgs_push: rounds");
 }
