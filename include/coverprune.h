@@ -393,7 +393,9 @@ int coverprune_profile_read(double* ms, int64_t* launches, int n);
  *                     and steps, each from one row of the cost (N floats) or
  *                     of the local slab (g floats); sgs_mode 0: terms of
  *                     gains updated after the first pick, one per live
- *                     (candidate, target) pair of a lowered target
+ *                     (candidate, target) pair of a lowered target (of a few
+ *                     tokens only, K <= 16, the gains computed after the
+ *                     first pick, each from one row)
  *   rounds            decision rounds over all scenes: sgs_mode 1 one per
  *                     step, sgs_mode 0 at most that (late rounds make many
  *                     picks)

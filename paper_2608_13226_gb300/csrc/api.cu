@@ -258,7 +258,9 @@ static void plan_ws(int op, int64_t B, int64_t N, int64_t D, int64_t K, int dtyp
     pl->cost = take(sizeof(float) * BN * (size_t)pl->ldc);
     if (d.sgs_mode == 2) pl->lit = take(sgs_literal_ws_bytes(B, N, K));
     if (d.g < N && d.sgs_mode != 2) pl->slab = take(sizeof(float) * BN * (size_t)d.g);
-    if (d.sgs_mode == 0) pl->push = take(sgs_push_ws_bytes(B, N, d.g, wave));
+    if (d.sgs_mode == 0)
+      pl->push = take(few_picks(d, N, K) ? sgs_push_first_bytes(B, N)
+                                         : sgs_push_ws_bytes(B, N, d.g, wave));
     if (local_tiles_path(op, dtype, N, d)) {
       const size_t T = (size_t)local_tiles(N);
       pl->lfeats = take(2 * BN * (size_t)D);

@@ -182,6 +182,23 @@ int launch_sgs_push(const float* cost, int64_t ldc, const float* slab, const int
                     const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                     int32_t* order32, float* gains, double* objective, int* status,
                     cudaStream_t s, const float* g0, void* ws, int64_t wave);
+// The default dense selection of so few tokens sweeps its candidates behind
+// bounds (k_sgs) instead of forming the live lists, which read the whole cost
+// and cost as much as ~20 sweeps.  Selection ms, lists / sweeps: one scene of
+// 8192 K = 1 0.86 / 0.32, 8 1.59 / 0.64, 16 1.74 / 0.96; 32 of 8192 13.5 / 5.4,
+// 12.1 / 8.5, 12.0 / 9.6; one of 1024 0.172 / 0.115, 0.208 / 0.194, 0.240 /
+// 0.285; 8 of 4096 1.29 / 0.52, 1.35 / 0.86, 1.39 / 1.06.
+inline bool few_picks(const DevParams& P, int64_t N, int64_t K) {
+  return P.sgs_mode == 0 && P.g >= N && (K <= 8 || (K <= 16 && N >= 2048));
+}
+// A dense selection's first pick, [B] keys left at *first in ws
+// (sgs_push_first_bytes bytes), the sums that bound the first gains [B][N] at
+// *bound (no g0: very large numbers) and [B][N] zeros at *zeros.
+size_t sgs_push_first_bytes(int64_t B, int64_t N);
+int launch_first_pick(const float* cost, int64_t ldc, const float* v, const DevParams& P, int64_t B,
+                      int64_t N, cudaStream_t s, const float* g0, void* ws,
+                      const unsigned long long** first, float** bound = nullptr,
+                      unsigned long long** zeros = nullptr);
 // The fixed-point scale of the gains while targets cost m0 at most, and once
 // every target is covered (sgs_gain.cuh).
 int gain_fx(float m0);

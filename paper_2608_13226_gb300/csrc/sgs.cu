@@ -1,7 +1,8 @@
 // K5: Spatial-Guided Greedy Selection (Sec. 3.5, Eqs. srpot, local_neighbor,
-// greedy_flow, sgs_select, sgs_update), every gain every step (sgs_mode 1),
-// and the choice between the selection kernels (sgs_push.cu holds the
-// default one, sgs_literal.cu the rule as printed).
+// greedy_flow, sgs_select, sgs_update), every gain every step (sgs_mode 1; the
+// default selection of a few tokens, behind bounds), and the choice between the
+// selection kernels (sgs_push.cu holds the default one, sgs_literal.cu the rule
+// as printed).
 //
 // The semi-relaxed OT of Eq. srpot, with the source support and its capacity
 // as decision variables, has a closed-form plan: every target t_j sends its
@@ -44,11 +45,20 @@ int gain_fx_covered(const DevParams& P) {
   return gain_fx(c < P.m0 ? c : P.m0);
 }
 
-template <bool LOCAL>
+// FEW (dense): the default selection of few tokens, its first pick given.  A
+// gain computed at an earlier step bounds the current one, so a candidate
+// whose bound is not above the best gain that any warp of the scene has found
+// in this step is passed over; each warp evaluates its highest bound first.
+struct FewArgs {
+  const gain_t* first;          // [B] key of the first pick
+  float* bound;                 // [B][N] at the start: sums of the first gains, inexact
+  unsigned long long* running;  // [2][B] zeros: the best key so far, by turn
+};
+template <bool LOCAL, bool FEW>
 __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
     const float* __restrict__ cost, int64_t ldc, const float* __restrict__ slab,
     const int32_t* __restrict__ nbr, const float* __restrict__ v_all, DevParams P, int N, int K,
-    int cps, int scene0, int fx, int fx1, int32_t* __restrict__ order32, float* __restrict__ gains,
+    int cps, int scene0, int fx, int fx1, FewArgs few, int32_t* __restrict__ order32, float* __restrict__ gains,
     double* __restrict__ objective, unsigned long long* partials, uint32_t* counters,
     int* status) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -76,6 +86,23 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
   }
   for (int i = threadIdx.x; i < nchosen; i += SGS_THREADS) chosen[i] = 0u;
   __syncthreads();
+  int step = 0;
+  if (FEW) {  // the first pick is known
+    const gain_t key = few.first[b];
+    const int pick = key_token(key);
+    for (int j = threadIdx.x; j < N; j += SGS_THREADS)
+      sm_m[j] = fminf(sm_m[j], __ldg(Cb + (size_t)pick * ldc + j));
+    if (threadIdx.x == 0) {
+      chosen[pick >> 5] = 1u << (pick & 31);
+      if (c == 0) {
+        order32[(size_t)b * K] = pick;
+        if (gains) gains[(size_t)b * K] = key_gain(key);
+      }
+    }
+    step = 1;
+    fx = fx1;
+    __syncthreads();
+  }
 
   const int gw = c * SGS_WARPS + w, nw = cps * SGS_WARPS;
   const size_t nscenes = gridDim.x / cps;
@@ -83,17 +110,62 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
   unsigned long long my_evals = 0ull;  // rows this warp evaluated (lane 0 counts)
   unsigned long long my_update_bytes = 0ull;  // coverage-update reads (thread 0 of block 0)
   uint32_t turn = 0;  // sweeps: one a step, one more where the scale is refitted
-  for (int step = 0; step < K && alive;) {
+  while (step < K && alive) {
     unsigned long long best = 0ull;
-    for (int t = gw; t < N; t += nw) {
-      if (chosen[t >> 5] & (1u << (t & 31))) continue;
-      const gain_t acc =
-          LOCAL ? local_row_gain(Sb + (size_t)t * P.g, NB + (size_t)t * P.kk, t, P.g, sm_m, sm_v,
-                                 fx, lane)
-                : dense_row_gain(Cb + (size_t)t * ldc, sm_m, sm_v, ncols, fx, lane);
-      ++my_evals;
-      const unsigned long long key = gain_key(gain_bits(acc, fx), t);
-      best = key > best ? key : best;
+    if (FEW) {
+      float* bound = few.bound + (size_t)b * N;
+      // this turn's slot; the other's last readers are behind the last barrier
+      unsigned long long* run = few.running + 2 * (size_t)b;
+      if (c == 0 && threadIdx.x == 0) run[(turn + 1u) & 1u] = 0ull;
+      run += turn & 1u;
+      // what the gain of candidate i of this warp is known not to exceed
+      auto above = [&](int i) -> gain_t {
+        const int t = gw + i * nw;
+        if (t >= N || (chosen[t >> 5] & (1u << (t & 31)))) return 0ull;
+        // 1 + 2^-15: the first sums are as far off (k_first_bounds)
+        const float x = __fmul_ru(__ldcg(bound + t), 1.000030517578125f);
+        return gain_key(__float_as_uint(x), t);
+      };
+      auto evaluate = [&](int t) {
+        const gain_t acc = dense_row_gain(Cb + (size_t)t * ldc, sm_m, sm_v, ncols, fx, lane);
+        ++my_evals;
+        const uint32_t bits = gain_bits(acc, fx);
+        const gain_t key = gain_key(bits, t);
+        if (lane == 0) {
+          __stcg(bound + t, __uint_as_float(bits));
+          if (key > best) atomicMax(run, key);
+        }
+        best = key > best ? key : best;
+      };
+      const int mine = gw < N ? (N - gw + nw - 1) / nw : 0;
+      gain_t top = 0ull;
+      for (int i = lane; i < mine; i += 32) top = max(top, above(i));
+      top = warp_max_key(top);
+      const int seed = top ? key_token(top) : -1;
+      if (seed >= 0) evaluate(seed);
+      for (int i0 = 0; i0 < mine; i0 += 32) {
+        const gain_t k = i0 + lane < mine ? above(i0 + lane) : 0ull;
+        uint32_t todo = 0xFFFFFFFFu;
+        while (todo) {
+          const gain_t seen = warp_max_key(lane == 0 ? *(volatile gain_t*)run : best);
+          todo &= __ballot_sync(0xFFFFFFFFu, k > seen && gw + (i0 + lane) * nw != seed);
+          if (!todo) break;
+          const int l = __ffs(todo) - 1;
+          todo &= todo - 1u;
+          evaluate(gw + (i0 + l) * nw);
+        }
+      }
+    } else {
+      for (int t = gw; t < N; t += nw) {
+        if (chosen[t >> 5] & (1u << (t & 31))) continue;
+        const gain_t acc =
+            LOCAL ? local_row_gain(Sb + (size_t)t * P.g, NB + (size_t)t * P.kk, t, P.g, sm_m, sm_v,
+                                   fx, lane)
+                  : dense_row_gain(Cb + (size_t)t * ldc, sm_m, sm_v, ncols, fx, lane);
+        ++my_evals;
+        const unsigned long long key = gain_key(gain_bits(acc, fx), t);
+        best = key > best ? key : best;
+      }
     }
     if (lane == 0) s_best[w] = best;
     __syncthreads();
@@ -143,6 +215,10 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
     }
     if (s_fx != fx) {  // every block's answer is the same
       fx = s_fx;
+      // the bounds are of sums cut at the scale before
+      if (FEW)
+        for (int t = gw + lane * nw; t < N; t += 32 * nw)
+          __stcg(few.bound + (size_t)b * N + t, 1.0e38f);
       __syncthreads();  // before it is written again
       continue;
     }
@@ -184,17 +260,17 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
   }
 }
 
-template <bool LOCAL>
+template <bool LOCAL, bool FEW>
 static int sgs_launch_impl(const float* cost, int64_t ldc, const float* slab, const int32_t* nbr,
                            const float* v, const DevParams& P, int64_t B, int64_t N, int64_t K,
                            int32_t* order32, float* gains, double* objective,
                            unsigned long long* partials, uint32_t* counters, int* status,
-                           cudaStream_t s) {
+                           cudaStream_t s, FewArgs few = FewArgs{}) {
   DeviceInfo di;
   if (device_info(&di) != CP_OK) return CP_ECUDA;
   const int64_t ncols = LOCAL ? N : ldc;
   const size_t smem = 2 * sizeof(float) * (size_t)ncols + sizeof(uint32_t) * (size_t)((N + 31) / 32);
-  auto fn = k_sgs<LOCAL>;
+  auto fn = k_sgs<LOCAL, FEW>;
   CP_TRY_STATUS(allow_smem((const void*)fn, smem, "launch_sgs: smem attribute"));
   int per_sm = 0;
   if (cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, SGS_THREADS, smem),
@@ -222,7 +298,7 @@ static int sgs_launch_impl(const float* cost, int64_t ldc, const float* slab, co
     DevParams Pc = P;
     void* args[] = {(void*)&cost, (void*)&ldc, (void*)&slab, (void*)&nbr, (void*)&v, (void*)&Pc,
                     (void*)&Ni, (void*)&Ki, (void*)&cps, (void*)&scene0, (void*)&fx, (void*)&fx1,
-                    (void*)&order32,
+                    (void*)&few, (void*)&order32,
                     (void*)&gains, (void*)&objective, (void*)&partials, (void*)&counters,
                     (void*)&status};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)fn, dim3((unsigned)(nb * cps)),
@@ -238,15 +314,22 @@ int launch_sgs(const float* cost, int64_t ldc, const float* slab, const int32_t*
                int32_t* order32, float* gains, double* objective, uint64_t* partials,
                uint32_t* counters, int* status, cudaStream_t s, const float* g0, void* push_ws,
                int64_t push_wave) {
+  auto* part = reinterpret_cast<unsigned long long*>(partials);
+  if (few_picks(P, N, K)) {
+    FewArgs few;
+    CP_TRY_STATUS(launch_first_pick(cost, ldc, v, P, B, N, s, g0, push_ws, &few.first, &few.bound,
+                                    &few.running));
+    return sgs_launch_impl<false, true>(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains,
+                                        objective, part, counters, status, s, few);
+  }
   if (P.sgs_mode == 0)
     return launch_sgs_push(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains, objective, status,
                            s, g0, push_ws, push_wave);
-  auto* part = reinterpret_cast<unsigned long long*>(partials);
   if (P.g < N)
-    return sgs_launch_impl<true>(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains, objective,
-                                 part, counters, status, s);
-  return sgs_launch_impl<false>(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains, objective,
-                                part, counters, status, s);
+    return sgs_launch_impl<true, false>(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains,
+                                        objective, part, counters, status, s);
+  return sgs_launch_impl<false, false>(cost, ldc, slab, nbr, v, P, B, N, K, order32, gains,
+                                       objective, part, counters, status, s);
 }
 
 // Upper bound of the partial slots the launcher may use: 2 * B * cps with

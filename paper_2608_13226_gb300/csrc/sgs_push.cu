@@ -1333,7 +1333,7 @@ int64_t push_wave(int64_t B, int64_t N) {
 }
 
 struct PushPlan {
-  size_t gains, first, max_bits, zero_bytes, sums, lens, span, lists, m, stop, row_len,
+  size_t gains, first, max_bits, zero_bytes, sums, first_bytes, lens, span, lists, m, stop, row_len,
       row_ent, total;
   size_t join0;  // dense: entries before the joined lists
   int64_t wave;
@@ -1358,6 +1358,7 @@ PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t wave) {
     p.max_bits = take(sizeof(uint32_t) * (size_t)B);
     p.zero_bytes = off;
     p.sums = take(sizeof(float) * BN);
+    p.first_bytes = off;
     p.wave = wave > 0 ? wave : push_wave(B, N);
     const size_t WN = (size_t)p.wave * (size_t)N;
     p.lens = take(sizeof(uint32_t) * WN * PUSH_CMAX);
@@ -1499,9 +1500,8 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
     r.list_step = (size_t)N * (size_t)P.g;
     return launch_rounds(k_sgs_rounds<true>, r, B, di, s);
   }
-  gain_t* first = reinterpret_cast<gain_t*>(base + pl.first);
-  uint32_t* max_bits = reinterpret_cast<uint32_t*>(base + pl.max_bits);
-  float* sums = g0 ? reinterpret_cast<float*>(base + pl.sums) : nullptr;
+  const gain_t* first = nullptr;
+  CP_TRY_STATUS(launch_first_pick(cost, ldc, v, P, B, N, s, g0, ws, &first));
   r.row_len = reinterpret_cast<uint32_t*>(base + pl.row_len);
   r.row_ent = reinterpret_cast<Entry*>(base + pl.row_ent);
   r.m_in = reinterpret_cast<float*>(base + pl.m);
@@ -1526,17 +1526,6 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
   a.K = (int)K;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  CP_TRY_STATUS(cuda_status(cudaMemsetAsync(base + pl.gains, 0, pl.zero_bytes, s),
-                            "launch_sgs_push: gains"));
-  if (g0) {
-    k_first_bounds<<<dim3((unsigned)((N + 255) / 256), (unsigned)B), 256, 0, s>>>(
-        g0, fst_apply_slots(ldc), (int)N, sums, max_bits);
-    CP_TRY_STATUS(last_launch_status());
-  }
-  const int64_t groups = g0 ? (N + 255) / 256 : (N + 7) / 8;
-  k_first_pick<<<dim3((unsigned)(groups < 512 ? groups : 512), (unsigned)B), 256, 0, s>>>(
-      cost, ldc, v, (int)N, P.m0, fx0, sums, max_bits, first);
-  CP_TRY_STATUS(last_launch_status());
   auto lists_fn = k_live_lists;
   if (cuda_status(cudaFuncSetAttribute(lists_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)LL_SMEM),
@@ -1585,6 +1574,34 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
 
 }  // namespace
 
+int launch_first_pick(const float* cost, int64_t ldc, const float* v, const DevParams& P, int64_t B,
+                      int64_t N, cudaStream_t s, const float* g0, void* ws, const gain_t** first_out,
+                      float** bound, gain_t** zeros) {
+  const PushPlan pl = push_plan(B, N, N, 1);
+  unsigned char* base = static_cast<unsigned char*>(ws);
+  uint32_t* max_bits = reinterpret_cast<uint32_t*>(base + pl.max_bits);
+  float* sums = g0 ? reinterpret_cast<float*>(base + pl.sums) : nullptr;
+  gain_t* first = reinterpret_cast<gain_t*>(base + pl.first);
+  *first_out = first;
+  if (bound) *bound = reinterpret_cast<float*>(base + pl.sums);
+  if (zeros) *zeros = reinterpret_cast<gain_t*>(base + pl.gains);
+  if (bound && !g0)  // 0x7E7E7E7E: 8e37
+    CP_TRY_STATUS(cuda_status(cudaMemsetAsync(*bound, 0x7E, sizeof(float) * (size_t)(B * N), s),
+                              "launch_first_pick: bounds"));
+  CP_TRY_STATUS(cuda_status(cudaMemsetAsync(base + pl.gains, 0, pl.zero_bytes, s),
+                            "launch_first_pick: gains"));
+  if (g0) {
+    k_first_bounds<<<dim3((unsigned)((N + 255) / 256), (unsigned)B), 256, 0, s>>>(
+        g0, fst_apply_slots(ldc), (int)N, sums, max_bits);
+    CP_TRY_STATUS(last_launch_status());
+  }
+  const int64_t groups = g0 ? (N + 255) / 256 : (N + 7) / 8;
+  k_first_pick<<<dim3((unsigned)(groups < 512 ? groups : 512), (unsigned)B), 256, 0, s>>>(
+      cost, ldc, v, (int)N, P.m0, gain_fx(P.m0), sums, max_bits, first);
+  return last_launch_status();
+}
+
+size_t sgs_push_first_bytes(int64_t B, int64_t N) { return push_plan(B, N, N, 1).first_bytes; }
 int64_t sgs_push_wave(int64_t B, int64_t N) { return push_wave(B, N); }
 
 // A local selection's own lists; where the dense ones are small (64 MB) room

@@ -65,6 +65,20 @@ def test_push_scale_of_the_coverage_cost(m0, g):
     assert abs((m0 - gains.sum()) - F) <= m0 * (700 * 2.0 ** -24 + 2.0 ** -20)
 
 
+@pytest.mark.parametrize("N,B", [(1, 1), (2, 2), (300, 3), (2047, 1), (2048, 2), (4099, 5),
+                                 (9000, 1)])
+@pytest.mark.parametrize("kw", [dict(), dict(m0=1e12), dict(capacity_mode=1, lambda_x=0.0)])
+def test_few_picks_equal_full_sweep(N, B, kw):
+    """Few picks sweep their candidates behind bounds; the lists take over
+    beyond 8 (16 from 2048 tokens on)."""
+    for name in ("long_video", "tiny"):  # bf16: bounds from the cost pass; fp32: none at first
+        scs = [scene(name, sd, N=N, D=64) for sd in range(min(B, 2))]
+        f, pos, fr = batch_to_dev((scs * B)[:B])
+        for K in (1, 2, 8, 9, 16, 17):
+            if K <= N:
+                _same(f, pos, fr, K, n_cap=min(8, max(1, N - 1)), **kw)
+
+
 @pytest.mark.parametrize("N,K,g", [(1500, 200, 0), (1500, 400, 24), (300, 300, 0)])
 @pytest.mark.parametrize("m0", [1e-3, 1e3, 1e6, 1e9, 1e12, 1e30])
 def test_push_coverage_cost_against_the_oracle(orc, m0, N, K, g):
