@@ -915,20 +915,20 @@ __global__ void __launch_bounds__(128) k_knn_grid_thread(int N, int kk, int gmax
 // the remaining cells that pass the test are evaluated with the same
 // arithmetic as every other kernel, so the result is exactly the largest d^2.
 //
-// A cluster of 8 blocks per scene: each finds the extremes of its eighth of
+// A cluster of up to 8 blocks per scene: each finds the extremes of its part of
 // the points (the work is nearly all there; few dozen pairs of cells pass the
-// test), then takes the pairs whose lower cell c has c mod 8 = its rank, a
-// warp per cell; pairs of large cells are left to the whole block.  16384
-// points: 167 us before (13 directions over all points in each of 4 blocks,
-// a thread per pair of cells), 24 now; 32 scenes of 8192 88 and 38.
+// test), then takes the pairs whose lower cell c is its rank modulo their
+// number, a warp per cell; pairs of large cells are left to the whole block.
+// 16384 points: 167 us before (13 directions over all points in each of 4
+// blocks, a thread per pair of cells), 24 now; 32 scenes of 8192 88 and 38.
 constexpr int DIA_THREADS = 512, DIA_PARTS = 8, DIA_DIRS = 7, DIA_BIG = 64;
 
 __device__ __forceinline__ uint32_t warp_max_u32(uint32_t v) {
   return __reduce_max_sync(0xFFFFFFFFu, v);
 }
 
-__global__ void __cluster_dims__(DIA_PARTS, 1, 1) __launch_bounds__(DIA_THREADS) k_diameter_grid(
-    int N, int gmax, const GridInfo* __restrict__ info, const int32_t* __restrict__ cell_start,
+__global__ void __launch_bounds__(DIA_THREADS) k_diameter_grid(
+    int N, int gmax, int parts, const GridInfo* __restrict__ info, const int32_t* __restrict__ cell_start,
     const float4* __restrict__ sorted, SceneStats* stats) {
   extern __shared__ int s_cand[];  // candidate cells, [gmax]
   __shared__ unsigned long long s_ext[2 * DIA_DIRS];   // this block's extremes: (key, point)
@@ -961,7 +961,7 @@ __global__ void __cluster_dims__(DIA_PARTS, 1, 1) __launch_bounds__(DIA_THREADS)
       ih[d] = il[d] = 0;
     }
 #pragma unroll 2
-    for (int i = part * DIA_THREADS + threadIdx.x; i < N; i += DIA_PARTS * DIA_THREADS) {
+    for (int i = part * DIA_THREADS + threadIdx.x; i < N; i += parts * DIA_THREADS) {
       const float4 p = P[i];
       const float v[DIA_DIRS] = {p.x, p.y, p.z, p.x + p.y + p.z, p.x + p.y - p.z,
                                  p.x - p.y + p.z, -p.x + p.y + p.z};
@@ -995,7 +995,7 @@ __global__ void __cluster_dims__(DIA_PARTS, 1, 1) __launch_bounds__(DIA_THREADS)
     for (int r = 0; r < DIA_PARTS; ++r)
       asm volatile("ld.shared::cluster.u64 %0, [%1];"
                    : "=l"(x[r])
-                   : "r"(map_rank(smem_addr(&s_ext[threadIdx.x]), (uint32_t)r))
+                   : "r"(map_rank(smem_addr(&s_ext[threadIdx.x]), (uint32_t)min(r, parts - 1)))
                    : "memory");
     unsigned long long m = x[0];
 #pragma unroll
@@ -1049,7 +1049,7 @@ __global__ void __cluster_dims__(DIA_PARTS, 1, 1) __launch_bounds__(DIA_THREADS)
   // pairs of candidate cells A <= B
   for (int r = w; r < M; r += NW) {
     const int A = s_cand[r];
-    if (A % DIA_PARTS != part) continue;
+    if (A % parts != part) continue;
     const int ax = A % d0, ay = (A / d0) % d1, az = A / (d0 * d1);
     const int a0 = cs[A], na = cs[A + 1] - a0;
     for (int t0 = 0; t0 < M; t0 += 32) {
@@ -1127,10 +1127,31 @@ int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr
   CP_TRY_STATUS(allow_smem((const void*)k_diameter_grid, smem, "launch_knn_grid: smem attribute"));
   k_grid_build<<<(unsigned)B, 1024, smem, s>>>(pos, (int)N, gmax, info, cell_start, sorted);
   CP_TRY_STATUS(last_launch_status());
-  k_diameter_grid<<<dim3(DIA_PARTS, (unsigned)B), DIA_THREADS, smem, s>>>((int)N, gmax, info,
-                                                                          cell_start, sorted,
-                                                                          stats);
-  CP_TRY_STATUS(last_launch_status());
+  DeviceInfo di;
+  if (device_info(&di) != CP_OK) return CP_ECUDA;
+  // up to two blocks an SM: further blocks only wait, and each clears and scans
+  // the cells again.  Diameters alone (no neighbours), us, 8 blocks a scene
+  // always / by this rule: 64 scenes of 256 tokens 45 / 36, 512 of 256 184 / 55,
+  // 256 of 1024 109 / 48, 64 of 8192 75 / 65; up to one an SM the last takes 68,
+  // up to four 76.
+  int parts = DIA_PARTS;
+  while (parts > 1 && B * parts > 2 * di.sm_count) parts >>= 1;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3((unsigned)parts, (unsigned)B);
+  cfg.blockDim = dim3(DIA_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)parts;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_diameter_grid, (int)N, gmax, parts, info,
+                                           cell_start, sorted, stats);
+  note_launch();
+  CP_TRY_STATUS(cuda_status(e, "launch_knn_grid: diameter"));
   if (kk <= 0) return CP_OK;
   // A thread a query needs fewer instructions where cells hold few points, but
   // only many queries hide its latency.  kk = 8, us, thread / warp (with

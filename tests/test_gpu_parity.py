@@ -86,6 +86,17 @@ def test_knn_many_small_scenes():
     assert torch.equal(nbr[:2], few)
 
 
+@pytest.mark.parametrize("B", [1, 38, 39, 76, 77, 152, 153, 700])
+def test_diameter_of_many_scenes(B):
+    """8, 4, 2 or 1 blocks a scene find the same diameters."""
+    pos = torch.rand(B, 300, 3, device="cuda") * 5
+    pos[:, 7] = pos[:, 8] + 4
+    _, dia = cp.coverprune_knn(pos, 0)
+    for b in (0, B // 2, B - 1):
+        want = np.sqrt(np.float32(_max_d2_fp32(host(pos[b]))), dtype=np.float32)
+        assert float(dia[b]) == float(want), b
+
+
 def _max_d2_fp32(X):
     """The largest squared distance over all pairs, every operation rounded
     in fp32 in the kernels' order ((dx dx + dy dy) + dz dz)."""
