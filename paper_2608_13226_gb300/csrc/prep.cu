@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(32 * KW_WARPS) k_knn_grid(
   }
 }
 
-// Few neighbours (kk <= 8) of very many small scenes: one thread per query token
+// Few neighbours (kk <= 8) of very many queries: one thread per query token
 // scans the shells of cells at Chebyshev distance r = 0, 1, 2, ... from its
 // own cell; every point outside the first r shells is more than r h away
 // along some axis, so once the kk-th best squared distance is below ((r -
@@ -1153,12 +1153,17 @@ int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr
   note_launch();
   CP_TRY_STATUS(cuda_status(e, "launch_knn_grid: diameter"));
   if (kk <= 0) return CP_OK;
-  // A thread a query needs fewer instructions where cells hold few points, but
-  // only many queries hide its latency.  kk = 8, us, thread / warp (with
-  // k_grid_build and k_diameter_grid): 128 scenes of 1024 176 / 223, 32 of 4096
-  // 227 / 219, of 8192 8 252 / 143, 16 303 / 219, 32 508 / 383, 8 of 16384
-  // 374 / 245; 32 long videos (the whole preparation) 655 / 657.
-  if (kk <= 8 && N <= 2048 && B * N >= 131072) {
+  // Few neighbours of very many queries: a thread a query needs fewer
+  // instructions than a warp, but a chain of the longer shells' cells that only
+  // many queries hide.  us, thread / warp (with k_grid_build and
+  // k_diameter_grid), 1 and 8 neighbours: 64 scenes of 1024 104 / 103 and 120 /
+  // 119, 128 124 / 160 and 160 / 195; 32 of 2048 178 / 122 and 193 / 139, 64 182
+  // / 182 and 214 / 217; 32 of 4096 226 / 186 and 265 / 217, 64 265 / 311 and 355
+  // / 380; 16 of 8192 205 / 190 and 232 / 223, 32 261 / 320 and 378 / 384, 64 592
+  // / 588 and 710 / 715, 128 624 / 1109 and 933 / 1362; 16 of 16384 299 / 344 and
+  // 462 / 410, 32 615 / 667 and 730 / 797.
+  const int64_t many = N <= 1024 ? 65536 : N <= 2048 ? 131072 : N <= 8192 ? 262144 : 524288;
+  if (kk <= 8 && B * N >= many) {
     k_knn_grid_thread<8><<<dim3((unsigned)((N + 127) / 128), (unsigned)B), 128, 0, s>>>(
         (int)N, kk, gmax, info, cell_start, sorted, nbr);
     return last_launch_status();

@@ -86,6 +86,22 @@ def test_knn_many_small_scenes():
     assert torch.equal(nbr[:2], few)
 
 
+@pytest.mark.parametrize("k", [1, 5, 8])
+@pytest.mark.parametrize("B,N", [(66, 1000), (262, 251), (130, 2049), (30, 8990), (33, 16384)])
+def test_knn_many_queries(B, N, k):
+    """So do 65,536 in scenes of up to 1024, 262,144 up to 8192 and 524,288
+    beyond: the lists of a few of the scenes alone."""
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    pos = torch.rand(B, N, 3, generator=gen, device="cuda") * 5
+    pos[:, :40] = pos[:, 40:80]
+    pos[0, 3] = 70.0
+    pos[1, 4, 1] = float("nan")
+    nbr, _ = cp.coverprune_knn(pos, k)
+    for b in (0, 1, B - 1):
+        one, _ = cp.coverprune_knn(pos[b], k)
+        assert torch.equal(nbr[b], one), b
+
+
 @pytest.mark.parametrize("B", [1, 38, 39, 76, 77, 152, 153, 700])
 def test_diameter_of_many_scenes(B):
     """8, 4, 2 or 1 blocks a scene find the same diameters."""
