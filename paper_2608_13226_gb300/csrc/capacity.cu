@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(32 * CAP_WARPS) k_capacity_r(
   if (threadIdx.x == 0) r_all[(size_t)b * N + j] = P.n_cap > 0 ? acc / (float)P.n_cap : 0.0f;
 }
 
-// The same r_j for bf16 features, a warp a token: its row against eight of its
+// The same r_j for bf16 features, a warp a token: its row against R of its
 // neighbours' at a time.  A block's 8 tokens are neighbours themselves (their
 // places follow the neighbour grid's order), so at any moment its warps read
 // the same columns of few distinct rows, most of them from L1; a block a
@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(32 * CAP_WARPS) k_capacity_r(
 // 1.31 ms, now 1.00; one scene of 16384 87 us, now 74.  Three blocks an SM:
 // at the registers the compiler takes by itself one fits, and 1.99 ms.  Every
 // dot product and sum keeps its order.
+template <int R>
 __global__ void __launch_bounds__(256, 3) k_capacity_r_near(
     const __nv_bfloat16* __restrict__ F_all, const float* __restrict__ inv_all,
     const float* __restrict__ pos_all, const int32_t* __restrict__ frame_all,
@@ -103,28 +104,28 @@ __global__ void __launch_bounds__(256, 3) k_capacity_r_near(
   const SceneNorms nm = norms[b];
   const __nv_bfloat16* fj = F + (size_t)j * D;
   float acc = 0.0f;
-  for (int q0 = 0; q0 < P.n_cap; q0 += 8) {
-    const int mine = nb[min(q0 + (lane & 7), P.n_cap - 1)];
-    const __nv_bfloat16* fk[8];
-    float dot[8];
+  for (int q0 = 0; q0 < P.n_cap; q0 += R) {
+    const int mine = nb[min(q0 + (lane & (R - 1)), P.n_cap - 1)];
+    const __nv_bfloat16* fk[R];
+    float dot[R];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < R; ++i) {
       fk[i] = F + (size_t)__shfl_sync(0xFFFFFFFFu, mine, i) * D;
       dot[i] = 0.0f;
     }
     for (int c = lane * 8; c < D; c += 256) {
       const uint4 x = __ldg(reinterpret_cast<const uint4*>(fj + c));
-      uint4 y[8];
+      uint4 y[R];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) y[i] = __ldg(reinterpret_cast<const uint4*>(fk[i] + c));
+      for (int i = 0; i < R; ++i) y[i] = __ldg(reinterpret_cast<const uint4*>(fk[i] + c));
 #pragma unroll
-      for (int i = 0; i < 8; ++i) dot[i] = dot8_bf16(x, y[i], dot[i]);
+      for (int i = 0; i < R; ++i) dot[i] = dot8_bf16(x, y[i], dot[i]);
     }
     float own = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < R; ++i) {
       const float t = warp_sum(dot[i]);
-      own = (lane & 7) == i ? t : own;
+      own = (lane & (R - 1)) == i ? t : own;
     }
     const int k = mine;
     const float cosv = clamp_cos(own * inv[j] * inv[k]);
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(256, 3) k_capacity_r_near(
     const float tt = dt > 0 ? (float)dt * nm.t_rinv : 0.0f;
     const float term = P.alpha_f * tf + P.alpha_x * tx + P.alpha_tau * tt;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < R; ++i) {
       const float t = __shfl_sync(0xFFFFFFFFu, term, i);
       if (q0 + i < P.n_cap) acc += t;
     }
@@ -237,11 +238,19 @@ int launch_capacity(const void* feats, int dtype, const float* inv, const float*
   // one block per token, a warp per neighbour (at most CAP_WARPS)
   const dim3 grid((unsigned)N, (unsigned)B);
   const int warps = P.n_cap < 1 ? 1 : (P.n_cap < CAP_WARPS ? P.n_cap : CAP_WARPS);
+  // rows at a time: the last turn multiplies its row count whatever is left.
+  // Lite of 8 scenes of 8192, D = 3584, us, 2 / 4 / 8 rows: 1 neighbour 573 / 613 /
+  // 659 (a block a token 731), 2 576 / 619 / 662 (756), 3 625 / 623 / 674, 4 633 /
+  // 628 / 681, 5 683 / 705 / 692, 6 689 / 711 / 703, 8 746 / 720 / 720, 9 798 / 799
+  // / 852, 12 863 / 818 / 874, 13 915 / 895 / 885, 16 980 / 916 / 916.
+  const auto near = P.n_cap <= 2                                     ? k_capacity_r_near<2>
+                    : P.n_cap <= 4 || (P.n_cap > 8 && P.n_cap <= 12) ? k_capacity_r_near<4>
+                                                                     : k_capacity_r_near<8>;
   if (cos)
     k_capacity_r_cos<<<dim3((unsigned)((N + 255) / 256), (unsigned)B), 256, 0, s>>>(
         cos, ldc, pos, frame, norms, nbr, P, (int)N, pos_of, r);
   else if (dtype == CP_BF16 && order)
-    k_capacity_r_near<<<dim3((unsigned)((N + 7) / 8), (unsigned)B), 256, 0, s>>>(
+    near<<<dim3((unsigned)((N + 7) / 8), (unsigned)B), 256, 0, s>>>(
         (const __nv_bfloat16*)feats, inv, pos, frame, norms, nbr, order, P, (int)N, (int)D, r);
   else if (dtype == CP_BF16)
     k_capacity_r<__nv_bfloat16><<<grid, 32 * warps, 0, s>>>(

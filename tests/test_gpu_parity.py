@@ -692,7 +692,7 @@ def _lite_check(orc, s, K, prm, dtype):
     return near
 
 
-@pytest.mark.parametrize("n_cap", [3, 8, 12])
+@pytest.mark.parametrize("n_cap", [1, 2, 3, 4, 5, 8, 9, 12, 13, 17])
 @pytest.mark.parametrize("N,D,seed", [(1001, 512, 6), (4100, 1280, 7), (777, 200, 8)])
 def test_capacity_from_features(orc, n_cap, N, D, seed):
     """The capacity computed from the bf16 features (Lite, and cost calls
