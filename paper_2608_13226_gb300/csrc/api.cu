@@ -333,8 +333,7 @@ static int run_front(const void* feats, int dtype, const float* pos, const int32
                              at<GridInfo>(ws, pl.grid_info), at<int32_t>(ws, pl.grid_start),
                              at<float4>(ws, pl.grid_pts), s));
     else
-      CP_TRY(launch_knn(pos, at<float4>(ws, pl.tok), B, N, d.kk, at<int32_t>(ws, pl.nbr), stats,
-                        s));
+      CP_TRY(launch_knn(pos, B, N, d.kk, at<int32_t>(ws, pl.nbr), stats, s));
   }
   // the Gram gives the min-max feature normaliser and the stored products;
   // with the bounded normaliser and none to store (Lite) it does not run
@@ -680,7 +679,7 @@ int coverprune_knn(const float* pos, int64_t B, int64_t N, int64_t k, int32_t* n
                            at<GridInfo>(ws, gi_off), at<int32_t>(ws, gs_off),
                            at<float4>(ws, gp_off), s));
   else
-    CP_TRY(launch_knn(pos, nullptr, B, N, (int)k, nbr, stats, s));
+    CP_TRY(launch_knn(pos, B, N, (int)k, nbr, stats, s));
   if (diameter) CP_TRY(launch_diameter(stats, B, diameter, s));
   return CP_OK;
 }

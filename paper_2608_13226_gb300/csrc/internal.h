@@ -114,7 +114,7 @@ constexpr int kKnnGridMax = 128;
 int launch_knn_grid(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr,
                     SceneStats* stats, GridInfo* info, int32_t* cell_start, float4* sorted,
                     cudaStream_t s);
-int launch_knn(const float* pos, const float4* tok, int64_t B, int64_t N, int kk, int32_t* nbr, SceneStats* stats,
+int launch_knn(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr, SceneStats* stats,
                cudaStream_t s);
 // K2 (fp32 SIMT and bf16 tensor-core variants): max and min cosine over all
 // pairs into stats.

@@ -299,23 +299,20 @@ __global__ void __launch_bounds__(256) k_knn_warp(const float* __restrict__ pos,
 }
 
 // K1 for kk <= 8, two tokens per warp, 16 per block: the block stages the
-// candidate positions in shared-memory tiles of 2048 (from the float4 token
-// table when one is given, else from the xyz array), so each position is
+// candidate positions in shared-memory tiles of 2048, so each position is
 // read from L2 once per 16 query rows; the quick test on the d^2 bits skips
 // the 64-bit key compare for almost every candidate.  Same keys, same lists
 // as k_knn_warp.
 constexpr int KNN_TILE = 2048;
 
-template <int KK, bool TOK>
-__global__ void __launch_bounds__(256) k_knn_pair(const float* __restrict__ pos,
-                                                  const float4* __restrict__ tok, int N, int kk,
+template <int KK>
+__global__ void __launch_bounds__(256) k_knn_pair(const float* __restrict__ pos, int N, int kk,
                                                   int32_t* __restrict__ nbr, SceneStats* stats) {
   __shared__ float4 s_p[KNN_TILE];
   const int j0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 2;
   const int b = blockIdx.y;
   const int lane = threadIdx.x & 31;
   const float* X = pos + (size_t)b * N * 3;
-  const float4* T = TOK ? tok + (size_t)b * N : nullptr;
   const bool active = j0 < N;
   const bool two = j0 + 1 < N;
   const int j1 = two ? j0 + 1 : j0;
@@ -332,12 +329,8 @@ __global__ void __launch_bounds__(256) k_knn_pair(const float* __restrict__ pos,
     const int n = min(KNN_TILE, N - base);
     __syncthreads();  // the previous tile is consumed
     for (int i = threadIdx.x; i < n; i += 256) {
-      if (TOK) {
-        s_p[i] = __ldg(T + base + i);
-      } else {
-        const int k = base + i;
-        s_p[i] = make_float4(__ldg(X + 3 * k), __ldg(X + 3 * k + 1), __ldg(X + 3 * k + 2), 0.f);
-      }
+      const int k = base + i;
+      s_p[i] = make_float4(__ldg(X + 3 * k), __ldg(X + 3 * k + 1), __ldg(X + 3 * k + 2), 0.f);
     }
     __syncthreads();
     if (!active) continue;
@@ -410,14 +403,11 @@ __global__ void __launch_bounds__(256) k_knn_pair(const float* __restrict__ pos,
   }
 }
 
-int launch_knn(const float* pos, const float4* tok, int64_t B, int64_t N, int kk, int32_t* nbr,
-               SceneStats* stats, cudaStream_t s) {
+int launch_knn(const float* pos, int64_t B, int64_t N, int kk, int32_t* nbr, SceneStats* stats,
+               cudaStream_t s) {
   if (kk <= 8) {
     dim3 grid((unsigned)((N + 15) / 16), (unsigned)B);
-    if (tok)
-      k_knn_pair<8, true><<<grid, 256, 0, s>>>(pos, tok, (int)N, kk, nbr, stats);
-    else
-      k_knn_pair<8, false><<<grid, 256, 0, s>>>(pos, nullptr, (int)N, kk, nbr, stats);
+    k_knn_pair<8><<<grid, 256, 0, s>>>(pos, (int)N, kk, nbr, stats);
     return last_launch_status();
   }
   if (kk <= 32) {

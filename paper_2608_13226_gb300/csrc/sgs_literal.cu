@@ -188,8 +188,7 @@ __global__ void __launch_bounds__(LC_COLS * LC_GROUPS) k_lit_cols(
 // columns are the block's own.
 //
 // The iterations run on the factors of the plan, P_ij = F_i E_ij G_j with
-// E = exp(-C / eps) formed once (correctly rounded to a few ulp: the argument
-// in two parts), F = exp(f / eps) = (1 / K) / sum_j E_ij G_j and G = exp(g /
+// E = exp(-C / eps) formed once (to a few ulp: the argument in two parts), F = exp(f / eps) = (1 / K) / sum_j E_ij G_j and G = exp(g /
 // eps) = min(1, v_j / sum_i F_i E_ij): a multiply-add a term, no exponential
 // and no logarithm.  Nothing over- or underflows while C <= 80 eps and a row's
 // sum is at least 2^-80 (F <= 2^80; a flushed product is below 2^-126, 2^-46

@@ -65,9 +65,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 // One live candidate of a target: the candidate's index in its owner block
 // and its cost bits.
 typedef uint2 Entry;
-// Chunks load whole, up to 127 entries past a list's end: entries past the
-// last list of the buffer.
-constexpr size_t LIST_PAD = 128;
 
 // ---------------------------------------------------------------------------
 // The first pick of the dense path.  The cost pass's partial sums (g0, one
@@ -1352,7 +1349,7 @@ PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t wave) {
   if (g < N) {
     p.wave = B;
     p.span = take(sizeof(uint2) * BN);
-    p.lists = take(sizeof(Entry) * (BN * (size_t)g + LIST_PAD));
+    p.lists = take(sizeof(Entry) * BN * (size_t)g);
   } else {
     p.first = take(sizeof(gain_t) * (size_t)B);
     p.max_bits = take(sizeof(uint32_t) * (size_t)B);
@@ -1363,12 +1360,12 @@ PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t wave) {
     const size_t WN = (size_t)p.wave * (size_t)N;
     p.lens = take(sizeof(uint32_t) * WN * PUSH_CMAX);
     p.join0 = WN * (size_t)(N + PUSH_CMAX);
-    p.lists = take(sizeof(Entry) * (p.join0 + WN * (size_t)row_room(N) + LIST_PAD));
+    p.lists = take(sizeof(Entry) * (p.join0 + WN * (size_t)row_room(N)));
     p.span = take(sizeof(uint2) * WN);
     p.m = take(sizeof(float) * WN);
     p.stop = take(sizeof(int) * (size_t)p.wave);
     p.row_len = take(sizeof(uint32_t) * (WN + (size_t)p.wave));  // and the joined lists' cursors
-    p.row_ent = take(sizeof(Entry) * (WN * (size_t)row_room(N) + LIST_PAD));
+    p.row_ent = take(sizeof(Entry) * WN * (size_t)row_room(N));
   }
   p.total = off;
   return p;
@@ -1563,8 +1560,8 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
         cudaMemsetAsync(r.row_len, 0, sizeof(uint32_t) * ((size_t)nb * (size_t)N + (size_t)nb), s),
         "launch_sgs_push: rows"));
     k_join_lists<<<dim3((unsigned)((N + 7) / 8), (unsigned)nb), 256, 0, s>>>(
-        a.lists, a.lens, (int)N, a.C, a.lgC, a.NC, pl.join0, (uint32_t)(N * row_room(N)), cursor, r.span,
-        r.row_len, r.row_ent);
+        a.lists, a.lens, (int)N, a.C, a.lgC, a.NC, pl.join0, (uint32_t)(N * row_room(N)), cursor,
+        r.span, r.row_len, r.row_ent);
     CP_TRY_STATUS(last_launch_status());
     r.scene0 = (int)b0;
     CP_TRY_STATUS(launch_rounds(k_sgs_rounds<false>, r, nb, di, s));
