@@ -1530,11 +1530,13 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
     return CP_ECUDA;
   for (int64_t b0 = 0; b0 < B; b0 += pl.wave) {
     const int64_t nb = B - b0 < pl.wave ? B - b0 : pl.wave;
-    // as many blocks a scene as let the wave's scenes run at once, 128
-    // candidates a block or more (selection of 1024 tokens, ms, on 4 / 8 / 16
-    // blocks: 0.314 / 0.295 / 0.294)
+    // as many blocks a scene as let the wave's scenes run at once, 64
+    // candidates a block or more (the whole selection, us, with 32 / 64 / 128 /
+    // 256 at least: one scene of 300 220 / 221 / 230 / 243, of 700 307 / 313 /
+    // 328 / 362, of 1500 481 / 481 / 497 / 554, of 3000 875 / 876 / 876 / 972; 4 of
+    // 300 251 / 249 / 255 / 264, of 1500 568 / 568 / 572 / 611)
     int C0 = PUSH_CMAX;
-    while (C0 > 1 && ((int64_t)C0 * nb > di.sm_count || N / C0 < 128)) C0 >>= 1;
+    while (C0 > 1 && ((int64_t)C0 * nb > di.sm_count || N / C0 < 64)) C0 >>= 1;
     if (C0 < 2 && N > 12288) C0 = 2;
     // lanes a list (its part in one block: N / C candidates at most): short
     // parts leave most of a warp idle, and a list is a chain of latencies;
