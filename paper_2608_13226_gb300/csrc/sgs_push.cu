@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
   const int nown = N > rank ? (N - rank + a.C - 1) >> lgC : 0;
   const float* v = a.v + (size_t)b * N;
   const float* R = a.cost + (size_t)b * N * (size_t)a.ldc;
-  unsigned long long my_ent = 0ull;  // list entries read (lane 0's count)
+  uint32_t my_ent = 0u;  // list entries read (a list's first lane counts; at most N^2 < 2^32)
 
   // state at the start: the first pick, m and the gains
   const gain_t f0 = a.first[b];
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
         }
       }
       if (gl == 0 && on) {
-        my_ent += (unsigned long long)lenc;
+        my_ent += (uint32_t)lenc;
         if (out != lenc) __stcg(a.lens + lj, (uint32_t)out);
         sm_m[jc] = mnc;
       }
@@ -616,8 +616,8 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
   unsigned long long* cstats = reinterpret_cast<unsigned long long*>(
       reinterpret_cast<unsigned char*>(a.status) + kCallStatsOffset);
   if ((lane & (LW - 1)) == 0 && my_ent) {
-    atomicAdd(&cstats[0], my_ent);
-    atomicAdd(&cstats[2], 8ull * my_ent);
+    atomicAdd(&cstats[0], (unsigned long long)my_ent);
+    atomicAdd(&cstats[2], 8ull * (unsigned long long)my_ent);
   }
   if (rank == 0 && threadIdx.x == 0) {
     atomicAdd(&cstats[1], (unsigned long long)step);
@@ -837,7 +837,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
   const int32_t* NB = LOCAL ? a.nbr + (size_t)b * N * a.kk : nullptr;
   uint2* span = a.span + (size_t)bl * N;
   Entry* lists = LOCAL ? a.lists + (size_t)bl * a.list_step : a.lists;
-  unsigned long long my_ent = 0ull, my_row = 0ull, my_rounds = 0ull;
+  uint32_t my_ent = 0u, my_row = 0u, my_rounds = 0u;  // at most N^2 < 2^32 each
 
   int step = LOCAL ? 0 : a.start[bl];
   for (int j = threadIdx.x; j < N; j += RD_THREADS)
@@ -1025,7 +1025,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
         }
       }
       if (lane == 0) {
-        my_row += (unsigned long long)(stored ? len : 0);
+        my_row += stored ? (uint32_t)len : 0u;
         if (!LOCAL && stored && n2 != len) __stcg(a.row_len + (size_t)bl * N + t, (uint32_t)n2);
         if (!fits) {
           s_mtok[i] = -1;
@@ -1216,7 +1216,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
         if (a.out_gains) a.out_gains[(size_t)b * a.K + step] = key_gain(best);
         s_pick[0] = pick;
         s_np = 1;
-        my_row += (unsigned long long)len;
+        my_row += (uint32_t)len;
       }
     }
     // ---- the lists of the lowered targets; a lone pick's row in pieces
@@ -1289,7 +1289,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
             }
           }
           if (gl == 0 && n) {
-            my_ent += (unsigned long long)n;
+            my_ent += (uint32_t)n;
             if (out != n) __stcg(&span[j].y, (uint32_t)out);
           }
         }
@@ -1306,10 +1306,10 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
   unsigned long long* cstats = reinterpret_cast<unsigned long long*>(
       reinterpret_cast<unsigned char*>(a.status) + kCallStatsOffset);
   if ((lane & 7) == 0) {
-    if (my_ent) atomicAdd(&cstats[0], my_ent);
-    atomicAdd(&cstats[2], 8ull * (my_ent + my_row));
+    if (my_ent) atomicAdd(&cstats[0], (unsigned long long)my_ent);
+    atomicAdd(&cstats[2], 8ull * ((unsigned long long)my_ent + my_row));
   }
-  if (threadIdx.x == 0) atomicAdd(&cstats[1], my_rounds);
+  if (threadIdx.x == 0) atomicAdd(&cstats[1], (unsigned long long)my_rounds);
   if (a.objective) {
     const double F = objective_sum(sm_m, v, N);
     if (threadIdx.x == 0) a.objective[b] = F;
