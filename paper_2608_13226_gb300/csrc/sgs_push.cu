@@ -727,9 +727,10 @@ __global__ void __launch_bounds__(256) k_join_lists(Entry* __restrict__ lists,
 constexpr int RD_WARPS = 32, RD_THREADS = 32 * RD_WARPS;
 constexpr int RD_EPT = 4;                        // row entries a thread holds at most
 constexpr int RD_EMAX = RD_EPT * RD_THREADS;     // ... and a round
-// Members a slice gives at most.  Selection, ms, at 2 / 4 / 8: N = 8192 3.51 /
-// 3.26 / 4.00, 4 local scenes of 6272 1.53 / 1.53 / 2.42: fewer picks a round
-// on one side, more rows to stage and rank on the other.
+// Members a slice gives at most (fewer where the rows' room is small, see
+// launch_rounds).  Selection, ms, at 2 / 4 / 8: N = 8192 3.51 / 3.26 / 4.00, 4
+// local scenes of 6272 1.53 / 1.53 / 2.42: fewer picks a round on one side, more
+// rows to stage and rank on the other.
 constexpr int RD_TOP = 4;
 constexpr int RD_MEMBERS = RD_TOP * RD_WARPS;
 constexpr uint32_t NO_ENTRY = 0xFFFFFFFFu;
@@ -757,6 +758,7 @@ struct RoundArgs {
   int N, K, g, kk;
   int S;                   // candidates a slice, ceil(N / 32) made odd
   int emax;                // row entries a round holds, at most RD_EMAX
+  int top;                 // members a slice gives at most, at most RD_TOP
   int tmask;               // size of the table of least ranks - 1
   int scene0;
   uint32_t off_lo, off_hi, off_ent, off_em, off_qm, off_qj, off_bits, off_tab;  // dynamic shared memory
@@ -872,8 +874,9 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
     // a lane whose three are used up bounds its rest by the third.  Fixed bits
     // of the scale, ranked by before, did not tell late gains apart: rounds of
     // a selection and ms, then / now, 4096 of 16384 tokens 972 / 534 and 29.3 /
-    // 15.0; 1229 of 8192 at m0 = 1000 1002 / 199 and 12.4 / 4.0; at the default
-    // m0 190 / 189 and 3.25 / 3.28 (the shift and the variable scale)
+    // 15.0 (with as many members a slice); 1229 of 8192 at m0 = 1000 1002 / 199
+    // and 12.4 / 4.0; at the default m0 190 / 189 and 3.24 / 3.27 (the shift and
+    // the variable scale)
     int cnt = 0, left = -1;
     {
       const int sh = s_sh;
@@ -889,7 +892,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
       const int third = v3;
       bool real = true;  // the head is a candidate, not a bound
 #pragma unroll 1
-      for (; cnt < RD_TOP; ++cnt) {
+      for (; cnt < a.top; ++cnt) {
         const int best = __reduce_max_sync(0xFFFFFFFFu, v1);
         const uint32_t who = __ballot_sync(0xFFFFFFFFu, v1 == best && real);
         if (best < 0 || who == 0u) break;  // warp-uniform
@@ -1448,6 +1451,12 @@ int launch_rounds(Fn fn, RoundArgs& a, int64_t scenes, const DeviceInfo& di, cud
     if (smem + 7168 <= (size_t)di.max_smem_optin) break;
     if (a.emax <= 256) return CP_EUNSUPPORTED;
   }
+  // Members whose rows do not all fit hold one another up: each that is left out
+  // bounds the picks by its gain.  Selection, ms, at 4 / 3 / 2 a slice: with 1024
+  // row entries (15000 tokens) a tenth kept 7.69 / 7.52 / 7.67, a quarter 8.71 /
+  // 8.65 / 9.14, local 4.34 / 3.62 / 3.13; with 512 (16384) 13.97 / 10.22 / 9.22,
+  // 15.30 / 11.41 / 10.79, local 7.02 / 5.80 / 4.45; 2048 fit.
+  a.top = a.emax >= 2048 ? RD_TOP : (a.emax >= 1024 && a.g >= N ? 3 : 2);
   CP_TRY_STATUS(allow_smem((const void*)fn, smem, "launch_sgs_push: rounds smem attribute"));
   fn<<<(unsigned)scenes, RD_THREADS, smem, s>>>(a);
   return launch_status("launch_sgs_push: rounds");
