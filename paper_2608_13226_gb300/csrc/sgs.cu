@@ -52,15 +52,15 @@ int gain_fx_covered(const DevParams& P) {
 struct FewArgs {
   const gain_t* first;          // [B] key of the first pick
   float* bound;                 // [B][N] at the start: sums of the first gains, inexact
-  unsigned long long* running;  // [2][B] zeros: the best key so far, by turn
+  unsigned long long* running;  // [B][2] zeros: the best key so far, by turn
 };
 template <bool LOCAL, bool FEW>
 __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
     const float* __restrict__ cost, int64_t ldc, const float* __restrict__ slab,
     const int32_t* __restrict__ nbr, const float* __restrict__ v_all, DevParams P, int N, int K,
-    int cps, int scene0, int fx, int fx1, FewArgs few, int32_t* __restrict__ order32, float* __restrict__ gains,
-    double* __restrict__ objective, unsigned long long* partials, uint32_t* counters,
-    int* status) {
+    int cps, int scene0, int fx, int fx1, FewArgs few, int32_t* __restrict__ order32,
+    float* __restrict__ gains, double* __restrict__ objective, unsigned long long* partials,
+    uint32_t* counters, int* status) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int ncols = LOCAL ? N : (int)ldc;  // dense rows are padded to ldc (C = 0, v = 0)
   float* sm_m = reinterpret_cast<float*>(smem);                  // [ncols] coverage cost m_j
@@ -298,9 +298,8 @@ static int sgs_launch_impl(const float* cost, int64_t ldc, const float* slab, co
     DevParams Pc = P;
     void* args[] = {(void*)&cost, (void*)&ldc, (void*)&slab, (void*)&nbr, (void*)&v, (void*)&Pc,
                     (void*)&Ni, (void*)&Ki, (void*)&cps, (void*)&scene0, (void*)&fx, (void*)&fx1,
-                    (void*)&few, (void*)&order32,
-                    (void*)&gains, (void*)&objective, (void*)&partials, (void*)&counters,
-                    (void*)&status};
+                    (void*)&few, (void*)&order32, (void*)&gains, (void*)&objective,
+                    (void*)&partials, (void*)&counters, (void*)&status};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)fn, dim3((unsigned)(nb * cps)),
                                                 dim3(SGS_THREADS), args, smem, s);
     note_launch();

@@ -878,8 +878,8 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
     // and 12.4 / 4.0; at the default m0 190 / 189 and 3.24 / 3.27 (the shift and
     // the variable scale)
     int cnt = 0, left = -1;
+    const int sh = s_sh;
     {
-      const int sh = s_sh;
       int v1 = -1, v2 = -1, v3 = -1;
 #pragma unroll 4
       for (int i = lane, q = 0; i < S; i += 32, ++q) {
@@ -920,11 +920,10 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
     }
     __syncthreads();  // every slice's bound is in
     // ---- S: the slices' candidates above the leading bits of all left out
-    const int sh = s_sh;
     left = __reduce_max_sync(0xFFFFFFFFu, s_left[lane]);
     if (threadIdx.x == 0) {
       s_np = 0;
-      if (left >= 0) atomicMax(&s_tau, (gain_t)(left + 1) << (32 - sh));
+      if (left >= 0) atomicMax(&s_tau, (gain_t)((uint32_t)left + 1u) << (32 - sh));
     }
     if (cnt > 0) {
       const int t = lane < cnt ? s_top[lane][w] : 0;
