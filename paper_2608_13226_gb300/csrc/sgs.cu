@@ -86,6 +86,14 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
   }
   for (int i = threadIdx.x; i < nchosen; i += SGS_THREADS) chosen[i] = 0u;
   __syncthreads();
+  // the scale after the first pick: m0's while a target is still uncovered (its
+  // cost undefined, as of a token with an infinite coordinate)
+  auto second_scale = [&]() -> int {
+    if (fx1 == fx) return fx;
+    bool open = false;
+    for (int j = threadIdx.x; j < N; j += SGS_THREADS) open |= !(sm_m[j] < P.m0);
+    return __syncthreads_or(open) ? fx : fx1;
+  };
   int step = 0;
   if (FEW) {  // the first pick is known
     const gain_t key = few.first[b];
@@ -100,8 +108,8 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
       }
     }
     step = 1;
-    fx = fx1;
     __syncthreads();
+    fx = second_scale();
   }
 
   const int gw = c * SGS_WARPS + w, nw = cps * SGS_WARPS;
@@ -242,9 +250,8 @@ __global__ void __launch_bounds__(SGS_THREADS, LOCAL ? 3 : 2) k_sgs(
         sm_m[j] = fminf(sm_m[j], srow[k]);
       }
     }
-    ++step;
-    fx = step == 1 ? fx1 : fx;
     __syncthreads();
+    if (++step == 1) fx = second_scale();
   }
 
   unsigned long long* cstats = reinterpret_cast<unsigned long long*>(

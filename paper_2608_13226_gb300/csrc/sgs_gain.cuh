@@ -12,7 +12,7 @@
 //
 // The scale follows the gains, not m0, which may be any number: it starts
 // from m0 (sum v = 1), on the dense path from the largest cost once the first
-// pick has covered every target (fx in launch_sgs), and whenever the best
+// pick has covered every target (gain_fx_covered), and whenever the best
 // gain left is below 2^-24 of it, it is fitted to that gain and the gains are
 // summed afresh before the pick (gain_floor, gain_refit; at most 8 times in a
 // selection, as it falls by 2^24 or more each time).  A term loses at most

@@ -142,6 +142,21 @@ __global__ void __launch_bounds__(256) k_first_pick(const float* __restrict__ co
   if (lane == 0 && best) atomicMax(first + b, best);
 }
 
+// The scale after the first pick where m0's and the largest cost's differ: m0's
+// while a target is still uncovered (its cost undefined, as of a token with an
+// infinite coordinate).
+__global__ void __launch_bounds__(256) k_first_scale(const float* __restrict__ cost, int64_t ldc,
+                                                     const gain_t* __restrict__ first, int N,
+                                                     float m0, int fx0, int fx,
+                                                     int* __restrict__ fxs) {
+  const int b = blockIdx.x;
+  const float* row = cost + ((size_t)b * N + key_token(first[b])) * ldc;
+  bool open = false;
+  for (int j = threadIdx.x; j < N; j += 256) open |= !(__ldg(row + j) < m0);
+  open = __syncthreads_or(open);
+  if (threadIdx.x == 0) fxs[b] = open ? fx0 : fx;
+}
+
 // ---------------------------------------------------------------------------
 // The live candidates after the first pick w0, m_j = min(m0, C(w0, j)), and
 // every candidate's gain there: one pass over the cost.  A block owns 128
@@ -162,11 +177,12 @@ constexpr int LL_PITCH = LL_COLS + 4;  // lanes of a 16-byte read (a lane a row)
 constexpr int LL_COLS_W = LL_COLS / LL_WARPS;
 constexpr size_t LL_SMEM = sizeof(float) * LL_STAGES * LL_ROWS * LL_PITCH;
 
+template <bool SCALED>  // the scene's scale is fxs[b]
 __global__ void __launch_bounds__(32 * LL_WARPS) k_live_lists(
     const float* __restrict__ cost, int64_t ldc, const float* __restrict__ v_all,
     const gain_t* __restrict__ first, int N, int C, int lgC, int NC, int scene0, float m0,
-    int fx, gain_t* __restrict__ gains, Entry* __restrict__ lists,
-    uint32_t* __restrict__ lens) {
+    int fx_all, const int* __restrict__ fxs, gain_t* __restrict__ gains,
+    Entry* __restrict__ lists, uint32_t* __restrict__ lens) {
   extern __shared__ __align__(16) float s_tile[];  // [LL_STAGES][LL_ROWS][LL_PITCH]
   __shared__ gain_t s_part[2][LL_WARPS][32];
   const int col0 = blockIdx.x * LL_COLS, rank = blockIdx.y, bl = blockIdx.z, b = scene0 + bl;
@@ -174,6 +190,7 @@ __global__ void __launch_bounds__(32 * LL_WARPS) k_live_lists(
   const float* Cb = cost + (size_t)b * N * ldc;
   const float* v = v_all + (size_t)b * N;
   gain_t* G = gains + (size_t)b * N;
+  const int fx = SCALED ? __ldg(fxs + b) : fx_all;
   const int nown = N > rank ? (N - rank + C - 1) >> lgC : 0;
   const int ntile = (nown + LL_ROWS - 1) / LL_ROWS;
   const int w0 = key_token(first[b]);
@@ -360,6 +377,7 @@ struct PushArgs {
   int* status;
   int64_t ldc;
   uint64_t timeout_ns;
+  const int* fxs;         // [B] the scenes' scales, or null: fx
   float m0;
   int fx;
   int N, K;
@@ -388,7 +406,7 @@ __device__ __forceinline__ void chunk_high(uint32_t* hi, uint32_t at, gain_t d, 
     if (dh) atomicAdd(hi + at, 0u - dh);
   }
 }
-template <int LW>
+template <int LW, bool SCALED = false>
 __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_constant__ PushArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   float* sm_m = reinterpret_cast<float*>(smem);                     // [ldc] coverage cost
@@ -404,7 +422,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 1) k_sgs_push(const __grid_const
   const int rank = (int)cluster_ctarank();
   const int bl = (int)(blockIdx.x >> a.lgC), b = a.scene0 + bl;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int N = a.N, lgC = a.lgC, fx = a.fx;
+  const int N = a.N, lgC = a.lgC, fx = SCALED ? __ldg(a.fxs + b) : a.fx;
   const int ncols = (int)a.ldc;
   const int nown = N > rank ? (N - rank + a.C - 1) >> lgC : 0;
   const float* v = a.v + (size_t)b * N;
@@ -752,6 +770,7 @@ struct RoundArgs {
   double* objective;       // [B] or null
   int* status;
   int64_t ldc;
+  const int* fxs;          // [B] the scenes' scales, or null: fx
   size_t list_step;        // local: entries between the lists of adjacent scenes
   float m0;
   int fx;
@@ -854,7 +873,7 @@ __global__ void __launch_bounds__(RD_THREADS, 1) k_sgs_rounds(const __grid_const
   for (int i = threadIdx.x; i <= a.tmask; i += RD_THREADS) tab[i] = NO_RANK;
   if (threadIdx.x == 0) {
     s_np = 0;
-    s_fx = a.fx;
+    s_fx = a.fxs ? a.fxs[b] : a.fx;
     s_sh = 0;
   }
   __syncthreads();
@@ -1332,7 +1351,7 @@ int64_t push_wave(int64_t B, int64_t N) {
 }
 
 struct PushPlan {
-  size_t gains, first, max_bits, zero_bytes, sums, first_bytes, lens, span, lists, m, stop, row_len,
+  size_t gains, first, max_bits, zero_bytes, sums, first_bytes, fxs, lens, span, lists, m, stop, row_len,
       row_ent, total;
   size_t join0;  // dense: entries before the joined lists
   int64_t wave;
@@ -1358,6 +1377,7 @@ PushPlan push_plan(int64_t B, int64_t N, int64_t g, int64_t wave) {
     p.zero_bytes = off;
     p.sums = take(sizeof(float) * BN);
     p.first_bytes = off;
+    p.fxs = take(sizeof(int) * (size_t)B);
     p.wave = wave > 0 ? wave : push_wave(B, N);
     const size_t WN = (size_t)p.wave * (size_t)N;
     p.lens = take(sizeof(uint32_t) * WN * PUSH_CMAX);
@@ -1531,7 +1551,13 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
   a.K = (int)K;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  auto lists_fn = k_live_lists;
+  if (fx != fx0) {  // m0 is well above every cost
+    int* fxs = reinterpret_cast<int*>(base + pl.fxs);
+    k_first_scale<<<(unsigned)B, 256, 0, s>>>(cost, ldc, first, (int)N, P.m0, fx0, fx, fxs);
+    CP_TRY_STATUS(last_launch_status());
+    a.fxs = r.fxs = fxs;
+  }
+  auto lists_fn = a.fxs ? k_live_lists<true> : k_live_lists<false>;
   if (cuda_status(cudaFuncSetAttribute(lists_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)LL_SMEM),
                   "launch_sgs_push: lists smem attribute") != CP_OK)
@@ -1554,13 +1580,15 @@ int launch_push(const float* cost, int64_t ldc, const float* slab, const int32_t
     // 8 of 8192 (16) 4.45 / 4.32 / 4.46, 16 (8) 7.15 / 7.05 / 7.40, 32 (4) 8.71
     // / 8.24 / 7.99; 32 of 2048 (4) 0.99 / 0.98 / 1.03.
     const int64_t part = N / C0;
-    auto push_fn = part >= 2048 ? k_sgs_push<32>
-                                : (nb == 1 && part <= 512 ? k_sgs_push<8> : k_sgs_push<16>);
+    auto push_fn = a.fxs                          ? k_sgs_push<16, true>
+                   : part >= 2048                 ? k_sgs_push<32>
+                   : (nb == 1 && part <= 512) ? k_sgs_push<8>
+                                                  : k_sgs_push<16>;
     CP_TRY_STATUS(push_config(push_fn, a, C0, nb, di, s, &cfg, attr));
     a.scene0 = (int)b0;
     lists_fn<<<dim3((unsigned)((N + LL_COLS - 1) / LL_COLS), (unsigned)a.C, (unsigned)nb),
                32 * LL_WARPS, LL_SMEM, s>>>(cost, ldc, v, first, (int)N, a.C, a.lgC, a.NC,
-                                            (int)b0, P.m0, fx, gains64, a.lists, a.lens);
+                                            (int)b0, P.m0, fx, a.fxs, gains64, a.lists, a.lens);
     CP_TRY_STATUS(launch_status("launch_sgs_push: lists"));
     const cudaError_t e = cudaLaunchKernelEx(&cfg, push_fn, a);
     note_launch();

@@ -96,6 +96,21 @@ def test_push_coverage_cost_against_the_oracle(orc, m0, N, K, g):
                              float(np.float32(m0)), g, nbr)
 
 
+@pytest.mark.parametrize("K", [6, 40])
+@pytest.mark.parametrize("m0", [5.0, 1e3, 1e12])
+def test_push_uncovered_after_the_first_pick(m0, K):
+    """A token at infinity has no cost to any other: the first pick leaves it
+    uncovered, and it is the second for its own m0 v (C(j, j) = 0)."""
+    s = scene("long_video", 2, N=400, D=64)
+    s["pos"][13, 1] = np.inf
+    f, pos, fr = batch_to_dev([s, scene("long_video", 4, N=400, D=64)])
+    r = _same(f, pos, fr, K, m0=m0)
+    v = host(cp.coverprune_cost(f, pos, fr, cost=False)["capacity"])[0, 13]
+    if m0 * v > 1.0:
+        assert host(r["order"])[0, 1] == 13
+        assert host(r["gains"])[0, 1] == np.float32(v) * np.float32(m0)
+
+
 @pytest.mark.parametrize("weights", [dict(lambda_f=0.0, lambda_x=0.0, lambda_tau=0.0),
                                      dict(lambda_x=0.0, lambda_tau=0.0), dict(lambda_f=0.0)])
 def test_push_ties(weights):
