@@ -589,8 +589,8 @@ def test_sgs_batch32_launch_shape(g):
                                              ("long_video", 1200, 64, 300, 2, 2),
                                              ("long_video", 1600, 128, 200, 0, 16)])
 def test_sgs_lazy_equals_full_sweep(name, N, D, K, g, B):
-    """Lazy evaluation only skips candidates whose earlier (upper-bound) gain
-    cannot win, so it must reproduce the full sweep bit for bit."""
+    """The default selection keeps exact gains up to date, so it must reproduce
+    the full sweep bit for bit."""
     scs = [scene(name, sd, N=N, D=D) for sd in range(min(B, 4))]
     f, pos, fr = batch_to_dev((scs * B)[:B])
     lazy = cp.coverprune_select(f, pos, fr, K, cp.Params(g=g, sgs_mode=0))

@@ -2,7 +2,7 @@
 candidates) against the full sweep, which sums every gain afresh every step:
 both add the same fixed-point terms, so picks, gains and objectives are equal
 bit for bit.  Sizes sit at the edges of the kernels' tiles (32 rows, 128
-columns, a list chunk of 32, clusters of 1 to 16 blocks), at the smallest and
+columns, 8 to 32 lanes a list, clusters of 1 to 16 blocks), at the smallest and
 the largest selections, and at coverage costs that move the fixed-point scale.
 """
 import numpy as np
@@ -52,7 +52,9 @@ def test_push_equals_full_sweep(N, K, g, B):
 @pytest.mark.parametrize("g", [0, 24])
 @pytest.mark.parametrize("m0", [1e-12, 0.05, 0.7, 40.0, 1e12])
 def test_push_scale_of_the_coverage_cost(m0, g):
-    """m0 sets the fixed-point scale (and, below the costs, what is live)."""
+    """m0 sets the first fixed-point scale (and, below the costs, what is live).
+    Both modes share the rule of the scales; the gains themselves are compared
+    with the oracle's below."""
     s = scene("short_clip", 3, N=700, D=64)
     f, pos, fr = batch_to_dev([s])
     r = _same(f, pos, fr, 150, g=g, m0=m0)
