@@ -500,7 +500,7 @@ def run_ours(args, rank, world, local_rank, raw):
     f_ms = fprof["sgs"][0] / max(fprof["sgs"][1], 1)
     f_bytes = fstats["cost_bytes_read"]
     f_gbs = f_bytes / (f_ms / 1000.0) / 1e9
-    sweep = {"bound": "hbm", "kernel": "k_sgs<0>", "achieved": round(f_gbs, 1), "peak": hbm,
+    sweep = {"bound": "hbm", "kernel": "k_sgs<0, 0>", "achieved": round(f_gbs, 1), "peak": hbm,
              "unit": "GB/s", "frac": round(f_gbs / hbm, 4),
              "frac_of_nominal": round(f_gbs / HBM_NOMINAL_GBS, 4),
              "traffic": read_traffic("k_sgs", f_bytes),

@@ -21,7 +21,8 @@ def _lib():
 
 
 @pytest.mark.parametrize("call,sizes,kw", [
-    ("select", (700, 2600, 1100, 1900), dict()),
+    ("select", (700, 2600, 1100, 1900), dict()),  # 2600: few picks
+    ("select", (2100, 2600, 3300, 4500), dict()),
     ("select", (900, 3100, 1300), dict(g=20)),
     ("select", (6500, 7900), dict(sgs_mode=1)),
     ("lite", (5200, 9000, 6100), dict(norm_mode=1)),
